@@ -50,8 +50,9 @@
  *                                  forward can complete before the backward times out
  *   STACKLSTM_STEP_KERNELS=1       one launch per time step instead of the persistent and
  *                                  cluster kernels (fp32: instead of one CTA for all steps)
- *   STACKLSTM_FWD_CLUSTER=0        no thread-block-cluster forward for one row tile
- *   STACKLSTM_BWD_CLUSTER=0        no thread-block-cluster backward for one row tile
+ *   STACKLSTM_FWD_CLUSTER=0        no thread-block-cluster forward
+ *   STACKLSTM_BWD_CLUSTER=0        no thread-block-cluster backward
+ *   STACKLSTM_ROW_CLUSTER=0        no clusters of eight rows (bf16_rows.cu): the 64-row ones
  *   STACKLSTM_BWD_SPLIT=k          the persistent backward with its 4H contraction split
  *                                  over k CTAs per 64-unit column tile (k = 4)
  *   STACKLSTM_SPLIT_CLUSTER=0      the parts of a split contraction trade their partial
@@ -191,9 +192,9 @@ sl_status stacklstm_steps_run(stacklstm_t s, int *steps);
  * and the action history of Sec. 4.1; Table 1 gives each transition's stack and buffer
  * ops); with the transitions known, their recurrences are independent of one another.
  * The result is that of calling stacklstm_forward (stacklstm_backward) on each handle,
- * each on its own stream. When every handle runs the one-row-tile cluster kernels (B <= 64)
- * with the same cluster size (the same H), their step kernels run as ONE launch of one
- * thread-block cluster per handle, on the first handle's stream; each handle's stream
+ * each on its own stream. When every handle runs cluster kernels on one 64-row tile (B <= 64)
+ * with the same cluster size (the same H), their step kernels run as ONE launch of each
+ * handle's thread-block clusters, on the first handle's stream; each handle's stream
  * joins that stream before the launch and waits for it afterwards. Otherwise each handle
  * launches its own. The work before and after the steps stays on each handle's stream.
  * Timing: the one launch counts in the first handle's forward (backward) phase.

@@ -82,6 +82,44 @@ __device__ __forceinline__ void pack_bwd_slice_elem(size_t e, const __nv_bfloat1
     out[((size_t)blk * kWChunkB + byte) / 2] = v;
 }
 
+// Weights of the row-group cluster kernels (bf16_rows.cu), whose CTA ct holds hidden units 32 ct ..
+// + 31 (eight a warp). mma.sync A fragments: value (lo, reg, lane) of a 16 x 16 tile is row
+// lane / 4 + 8 (reg & 1), column 2 (lane % 4) + lo + 8 (reg >> 1).
+// Forward, W_h: element e of [ct][warp 4][M tile 2][K step KH][lane 32][reg 4][2]; M tile i
+// holds gate 2 i (rows 0..7) and gate 2 i + 1 (rows 8..15) of the warp's units, K is the h unit.
+__device__ __forceinline__ void pack_rows_wh_elem(size_t e, const __nv_bfloat16 *__restrict__ W, int I, int H, int KH,
+                                                __nv_bfloat16 *__restrict__ out)
+{
+    const int lo = (int)(e & 1), reg = (int)(e >> 1) & 3, lane = (int)(e >> 3) & 31;
+    const uint32_t blk = (uint32_t)(e >> 8), ks = blk % KH, i = (blk / KH) & 1, warp = (blk / KH >> 1) & 3;
+    const int ct = (int)(blk / KH >> 3);
+    const int gate = 2 * (int)i + (reg & 1), unit = 32 * ct + 8 * (int)warp + (lane >> 2);
+    const int k = 16 * (int)ks + 2 * (lane & 3) + lo + 8 * (reg >> 1);
+    out[e] = unit < H && k < H ? W[(size_t)(I + k) * 4 * H + gate * H + unit] : __float2bfloat16(0.0f);
+}
+// Forward, W_x as it lies in shared memory: element e of [ct][128 rows][16 KX + 8], row
+// 32 warp + 16 i + r the row r of M tile i as above, K the x column.
+__device__ __forceinline__ void pack_rows_wx_elem(size_t e, const __nv_bfloat16 *__restrict__ W, int I, int H, int ld,
+                                                __nv_bfloat16 *__restrict__ out)
+{
+    const uint32_t row = (uint32_t)(e / ld), m = row & 127;
+    const int k = (int)(e - (size_t)row * ld), ct = (int)(row >> 7);
+    const int gate = 2 * (int)((m >> 4) & 1) + (int)((m >> 3) & 1), unit = 32 * ct + 8 * (int)(m >> 5) + (int)(m & 7);
+    out[e] = unit < H && k < I ? W[(size_t)k * 4 * H + gate * H + unit] : __float2bfloat16(0.0f);
+}
+// Backward, W_h: element e of [ct][warp 8][MT][K step 8][lane 32][reg 4][2]; M tile
+// 8 i + warp holds 16 units of dh_read, K = 4 (unit of ct) + gate over the CTA's gate columns.
+__device__ __forceinline__ void pack_rows_wb_elem(size_t e, const __nv_bfloat16 *__restrict__ W, int I, int H, int MT,
+                                                __nv_bfloat16 *__restrict__ out)
+{
+    const int lo = (int)(e & 1), reg = (int)(e >> 1) & 3, lane = (int)(e >> 3) & 31, ks = (int)(e >> 8) & 7;
+    const uint32_t blk = (uint32_t)(e >> 11), i = blk % MT, warp = blk / MT & 7;
+    const int ct = (int)(blk / MT >> 3);
+    const int row = 16 * (8 * (int)i + (int)warp) + (lane >> 2) + 8 * (reg & 1);
+    const int k = 16 * ks + 2 * (lane & 3) + lo + 8 * (reg >> 1), unit = 32 * ct + (k >> 2), gate = k & 3;
+    out[e] = row < H && unit < H ? W[(size_t)(I + row) * 4 * H + gate * H + unit] : __float2bfloat16(0.0f);
+}
+
 template <int N>
 struct TmemCols {
     static constexpr uint32_t value = N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : 256;
@@ -190,7 +228,7 @@ struct StepArgs {
     __nv_bfloat16 *hist_h;      // [T+1][B][H]
     __nv_bfloat16 *hr;          // [T+1][B][H] h operand of each step
     float *hist_c;              // [T+1][B][H]
-    __half *gates;              // [T][B][4H], or (gates_blk) [T][B][H / 16][4][16]
+    __half *gates;              // [T][B][4H], or (gates_blk) [T][B][H / 16][4][16], or (bf16_rows.cu) [T][B][H][4]
     int gates_blk;              // the blocked gate layout (the cluster forward and backward pair)
     const float *bias;          // [4H]
     const uint8_t *wpack;       // packed B-operand tiles of this kernel
@@ -276,6 +314,18 @@ cudaError_t bf16_launch_fwd_persist(stacklstm *s, const StepArgs &a, const CUten
                                     const CUtensorMap &tm_hc);
 cudaError_t bf16_launch_bwd_persist(stacklstm *s, const StepArgs &a, const CUtensorMap &tm_g, float *dx,
                                     bool *dx_done);
+
+// ---- thread-block clusters of few rows, H <= 256 (bf16_rows.cu)
+bool bf16_plan_rows(stacklstm *s, bool fwd, PersistPlan *pl);
+// elements of their packed weights (pack_rows_*_elem), and the contraction steps they are built for
+size_t bf16_rows_wh_elems(int H);
+size_t bf16_rows_wx_elems(int I, int H);
+size_t bf16_rows_wb_elems(int H);
+int bf16_rows_k(int H);
+// The steps of n handles as one launch (n > 1: grouped calls). Backward: d_top[m] is the
+// gradient of the final tops' h that is still to be added (null: none, or already seeded).
+cudaError_t bf16_launch_rows(stacklstm *const *hs, const StepArgs *as, const float *const *d_top, int n, bool fwd,
+                             cudaStream_t st);
 
 // ---- small batches on CUDA cores (bf16_small.cu)
 bool bf16_plan_small(stacklstm *s, PersistPlan *pl);

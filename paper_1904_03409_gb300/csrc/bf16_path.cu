@@ -425,14 +425,16 @@ struct SetupArgs {
     int nx;
     __nv_bfloat16 *wcl;  // cluster backward slices (n_cl; 0: not needed)
     int n_ctc;
+    __nv_bfloat16 *wrh, *wrx, *wrb;  // row-group clusters: forward W_h and W_x, backward W_h (n_rh, n_rx, n_rb)
+    int kh, ldx;
     const uint4 *h0, *c0;  // 16-byte pieces: n_h of h0, n_c of c0
     uint4 *hist_h, *hr, *hist_c;
-    size_t n_f, n_b, n_dx, n_cl, n_h, n_c;
+    size_t n_f, n_b, n_dx, n_cl, n_rh, n_rx, n_rb, n_h, n_c;
 };
 
 __global__ void setup_kernel(SetupArgs a)
 {
-    const size_t n = a.n_h + a.n_c + a.n_f + a.n_b + a.n_dx + a.n_cl;
+    const size_t n = a.n_h + a.n_c + a.n_f + a.n_b + a.n_dx + a.n_cl + a.n_rh + a.n_rx + a.n_rb;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
         size_t r = e;
         if (r < a.n_h) {
@@ -457,7 +459,19 @@ __global__ void setup_kernel(SetupArgs a)
             pack_w_rows_elem(r, a.W, a.H, 0, a.I, a.nx, a.kcb, a.wdx);
             continue;
         }
-        pack_bwd_slice_elem(r - a.n_dx, a.W, a.I, a.H, a.n_ctc, a.wcl);
+        if ((r -= a.n_dx) < a.n_cl) {
+            pack_bwd_slice_elem(r, a.W, a.I, a.H, a.n_ctc, a.wcl);
+            continue;
+        }
+        if ((r -= a.n_cl) < a.n_rh) {
+            pack_rows_wh_elem(r, a.W, a.I, a.H, a.kh, a.wrh);
+            continue;
+        }
+        if ((r -= a.n_rh) < a.n_rx) {
+            pack_rows_wx_elem(r, a.W, a.I, a.H, a.ldx, a.wrx);
+            continue;
+        }
+        pack_rows_wb_elem(r - a.n_rx, a.W, a.I, a.H, (a.kh + 7) / 8, a.wrb);
     }
 }
 
@@ -618,18 +632,19 @@ std::string bf16_describe(const stacklstm *s)
 {
     char buf[1024];
     const int rt = (int)ceil_div(s->B, kRows);
-    const PersistPlan &f = s->cc.on ? s->cc : s->fc.on ? s->fc : s->pf, &b = s->cc.on ? s->cc : s->bc.on ? s->bc : s->pb;
+    const PersistPlan &f = s->cc.on ? s->cc : s->fr.on ? s->fr : s->fc.on ? s->fc : s->pf;
+    const PersistPlan &b = s->cc.on ? s->cc : s->br.on ? s->br : s->bc.on ? s->bc : s->pb;
     snprintf(buf, sizeof buf,
              "bf16 tcgen05; row tiles %d; chunks fwd %d (x %d) bwd %d; "
              "forward %s U=%d [EP %d G %d ring %d slots %d cluster %d col tiles %d w_res %d smem %u threads %d "
-             "per SM %d]; "
+             "per SM %d rows %d]; "
              "backward %s U=%d [EP %d G %d ring %d slots %d cluster %d col tiles %d w_res %d smem %u threads %d "
-             "per SM %d "
+             "per SM %d rows %d "
              "contraction parts %d dx CTAs %d ring %d]; "
              "step rings fwd %d bwd %d; dx N=%d x%d ring %d; dW %dx%d tiles of %dx%d x%d splits ring %d",
-             rt, s->kcf, s->kcx, s->kcb, s->cc.on ? "cuda-core" : s->fc.on ? "cluster" : f.on ? "persistent" : "per-step", s->uf, f.EP, f.G, f.S, f.slot, f.cl, f.n_ct,
-             f.w_res, f.smem, f.threads, f.per_sm, s->cc.on ? "cuda-core" : s->bc.on ? "cluster" : b.on ? "persistent" : "per-step", s->bc.on ? s->bc.U : s->ub, b.EP, b.G, b.S, b.slot, b.cl, b.n_ct,
-             b.w_res, b.smem, b.threads, b.per_sm, b.KS, b.n_dx, b.dx_S, s->sf, s->sb, s->nx, s->nxt, s->sx, s->dw_mt, s->dw_nt, s->dw_mtile, s->dw_ntile, s->dw_split, s->sw);
+             rt, s->kcf, s->kcx, s->kcb, s->cc.on ? "cuda-core" : s->fr.on || s->fc.on ? "cluster" : f.on ? "persistent" : "per-step", s->fr.on ? f.U : s->uf, f.EP, f.G, f.S, f.slot, f.cl, f.n_ct,
+             f.w_res, f.smem, f.threads, f.per_sm, f.rows, s->cc.on ? "cuda-core" : s->br.on || s->bc.on ? "cluster" : b.on ? "persistent" : "per-step", s->br.on || s->bc.on ? b.U : s->ub, b.EP, b.G, b.S, b.slot, b.cl, b.n_ct,
+             b.w_res, b.smem, b.threads, b.per_sm, b.rows, b.KS, b.n_dx, b.dx_S, s->sf, s->sb, s->nx, s->nxt, s->sx, s->dw_mt, s->dw_nt, s->dw_mtile, s->dw_ntile, s->dw_split, s->sw);
     return buf;
 }
 
@@ -676,9 +691,14 @@ cudaError_t bf16_prepare(stacklstm *s)
             s->pf.on = 0;
         }
         bf16_plan_bwd_cluster(s, &s->bc);  // (the persistent plan stays as the fallback)
+        // few rows: clusters of 8 rows instead (both directions: they share a gate layout)
+        if (bf16_plan_rows(s, true, &s->fr) && bf16_plan_rows(s, false, &s->br))
+            s->fc.on = s->pf.on = s->bc.on = 0;
+        else
+            s->fr.on = s->br.on = 0;
         // small batches: both directions on CUDA cores instead
         if (bf16_plan_small(s, &s->cc)) {
-            s->pf.on = s->pb.on = s->fc.on = s->bc.on = 0;
+            s->pf.on = s->pb.on = s->fc.on = s->bc.on = s->fr.on = s->br.on = 0;
             s->uf = s->ub = s->cc.U;
         }
     }
@@ -707,6 +727,16 @@ cudaError_t bf16_prepare(stacklstm *s)
         s->allocs.push_back(p); s->w_bcl = p;
         if ((e = cudaMalloc(&p, bf16_bwd_cluster_block_bytes(T, B, H)))) return e;
         s->allocs.push_back(p); s->g_bcl = p;
+    }
+    if (s->fr.on) {
+        if ((e = cudaMalloc(&p, 2 * bf16_rows_wh_elems(H)))) return e;
+        s->allocs.push_back(p); s->w_rh = p;
+        if ((e = cudaMalloc(&p, 2 * bf16_rows_wx_elems(I, H)))) return e;
+        s->allocs.push_back(p); s->w_rx = p;
+    }
+    if (s->br.on) {
+        if ((e = cudaMalloc(&p, 2 * bf16_rows_wb_elems(H)))) return e;
+        s->allocs.push_back(p); s->w_rb = p;
     }
     if (s->cc.on) {
         if ((e = cudaMalloc(&p, bf16_small_weight_bytes(I, H, true)))) return e;
@@ -770,14 +800,17 @@ cudaError_t bf16_forward_setup_state(stacklstm *s, const __nv_bfloat16 *h0, cons
     // the CUDA-core kernels have weight layouts of their own
     if (s->cc.on && (e = bf16_pack_small(s, W))) return e;
     if (!s->cc.on) {
-        const int nctf = std::max((int)ceil_div(H, s->uf), s->pf.on ? s->pf.n_ct : 0);
-        a.wf = (__nv_bfloat16 *)s->w_fwd;
-        a.uf = s->uf;
-        a.kcx = s->kcx;
-        a.kcf = s->kcf;
-        a.n_f = (size_t)nctf * s->kcf * 4 * s->uf * kChunk;
+        // (the row-group clusters have weight layouts of their own)
+        if (!s->fr.on) {
+            const int nctf = std::max((int)ceil_div(H, s->uf), s->pf.on ? s->pf.n_ct : 0);
+            a.wf = (__nv_bfloat16 *)s->w_fwd;
+            a.uf = s->uf;
+            a.kcx = s->kcx;
+            a.kcf = s->kcf;
+            a.n_f = (size_t)nctf * s->kcf * 4 * s->uf * kChunk;
+        }
         // the persistent and per-step backward's weight tiles (the cluster backward has its own)
-        if (!s->bc.on) {
+        if (!s->bc.on && !s->br.on) {
             const int nctb = std::max((int)ceil_div(H, s->ub), s->pb.on ? s->pb.n_ct : 0);
             a.wb = (__nv_bfloat16 *)s->w_bwd;
             a.ub = s->ub;
@@ -793,6 +826,18 @@ cudaError_t bf16_forward_setup_state(stacklstm *s, const __nv_bfloat16 *h0, cons
         a.n_ctc = s->bc.n_ct;
         a.n_cl = (size_t)s->bc.n_ct * s->bc.n_ct * 16 * 64;
     }
+    a.kh = bf16_rows_k(H);
+    if (s->fr.on) {
+        a.wrh = (__nv_bfloat16 *)s->w_rh;
+        a.n_rh = bf16_rows_wh_elems(H);
+        a.wrx = (__nv_bfloat16 *)s->w_rx;
+        a.ldx = (int)ceil_div(I, 16) * 16 + 8;
+        a.n_rx = bf16_rows_wx_elems(I, H);
+    }
+    if (s->br.on) {
+        a.wrb = (__nv_bfloat16 *)s->w_rb;
+        a.n_rb = bf16_rows_wb_elems(H);
+    }
     a.h0 = (const uint4 *)h0;
     a.c0 = (const uint4 *)c0;
     a.hist_h = (uint4 *)s->hist_h;
@@ -801,7 +846,7 @@ cudaError_t bf16_forward_setup_state(stacklstm *s, const __nv_bfloat16 *h0, cons
     a.n_h = (size_t)B * H / 8;  // H % 8 == 0: whole 16-byte pieces
     a.n_c = (size_t)B * H / 4;
     // a few blocks per SM: the prepass, launched just before on the caller's stream, keeps its SMs
-    const size_t n = a.n_h + a.n_c + a.n_f + a.n_b + a.n_dx + a.n_cl;
+    const size_t n = a.n_h + a.n_c + a.n_f + a.n_b + a.n_dx + a.n_cl + a.n_rh + a.n_rx + a.n_rb;
     setup_kernel<<<(unsigned)std::max<size_t>(1, std::min<size_t>(ceil_div(n, 256), (size_t)s->num_sms * 4)), 256, 0,
                    s->stream>>>(a);
     s->launches += 1;
@@ -829,6 +874,10 @@ cudaError_t bf16_forward_steps(stacklstm *s, const float *bias)
     const int nctf = std::max((int)ceil_div(H, s->uf), s->pf.on ? s->pf.n_ct : 0);
     cudaError_t e;
     if (s->cc.on) return bf16_launch_fwd_small(s, step_args(s, bias, s->w_ccf, s->kcx, s->kcf, 0));
+    if (s->fr.on) {
+        const StepArgs a = step_args(s, bias, nullptr, s->kcx, s->kcf, 0);
+        return bf16_launch_rows(&s, &a, nullptr, 1, true, s->stream);
+    }
     if (s->fc.on)
         return bf16_launch_fwd_cluster(s, step_args(s, bias, s->w_fwd, s->kcx, s->kcf, 0), map(s, kMapX64));
     if (s->pf.on)
@@ -856,6 +905,9 @@ cudaError_t bf16_forward_steps(stacklstm *s, const float *bias)
 // Pointwise backward of the last step, before the reverse loop.
 cudaError_t bf16_backward_setup(stacklstm *s, const float *d_top_h)
 {
+    // the row-group clusters run every step themselves, and add the final tops' gradient
+    s->d_top_seed = s->br.on ? d_top_h : nullptr;
+    if (s->br.on) return cudaSuccess;
     StepArgs a = bwd_args(s, s->w_bwd, s->kcb, s->sb);
     a.gates_blk = s->fc.on && s->bc.on;  // the layout the cluster forward wrote for the cluster backward
     // the final top's history row of each instance (virtual, in push-only mode)
@@ -873,6 +925,10 @@ cudaError_t bf16_backward_steps(stacklstm *s, float *dx, bool *dx_done)
     cudaError_t e;
     const StepArgs a = bwd_args(s, s->w_bwd, s->kcb, s->sb);
     if (s->cc.on) return bf16_launch_bwd_small(s, bwd_args(s, s->w_ccb, s->kcb, 0));
+    if (s->br.on) {
+        const StepArgs ar = bwd_args(s, nullptr, s->kcb, 0);
+        return bf16_launch_rows(&s, &ar, &s->d_top_seed, 1, false, s->stream);
+    }
     if (s->bc.on) return bf16_launch_bwd_cluster(s, bwd_args(s, s->w_bcl, s->kcb, 0));
     // one row tile of at most 64 instances: 64-row boxes (the rest of each stage is never
     // loaded and only feeds accumulator rows that are not stored)
@@ -894,12 +950,19 @@ cudaError_t bf16_backward_steps(stacklstm *s, float *dx, bool *dx_done)
     return cudaGetLastError();
 }
 
+// the one-launch plan of a handle's steps: row-group clusters, or one 64-row cluster
+static const PersistPlan &group_plan(const stacklstm *s, bool fwd)
+{
+    return fwd ? (s->fr.on ? s->fr : s->fc) : (s->br.on ? s->br : s->bc);
+}
+
 bool bf16_can_group(stacklstm *const *hs, int n, bool fwd)
 {
+    const PersistPlan &p0 = group_plan(hs[0], fwd);
     for (int m = 0; m < n; ++m) {
         const stacklstm *s = hs[m];
-        const PersistPlan &pl = fwd ? s->fc : s->bc;
-        if (s->dt != SL_BF16 || s->cc.on || !pl.on || pl.slot != 1 || pl.n_ct != (fwd ? hs[0]->fc : hs[0]->bc).n_ct ||
+        const PersistPlan &pl = group_plan(s, fwd);
+        if (s->dt != SL_BF16 || s->cc.on || !pl.on || pl.slot != 1 || pl.n_ct != p0.n_ct || pl.rows != p0.rows ||
             s->device != hs[0]->device)
             return false;
     }
@@ -910,6 +973,10 @@ cudaError_t bf16_forward_steps_group(stacklstm *const *hs, int n, const float *c
 {
     StepArgs as[kMaxGroup];
     const CUtensorMap *tms[kMaxGroup];
+    if (hs[0]->fr.on) {
+        for (int m = 0; m < n; ++m) as[m] = step_args(hs[m], bias[m], nullptr, hs[m]->kcx, hs[m]->kcf, 0);
+        return bf16_launch_rows(hs, as, nullptr, n, true, st);
+    }
     for (int m = 0; m < n; ++m) {
         as[m] = step_args(hs[m], bias[m], hs[m]->w_fwd, hs[m]->kcx, hs[m]->kcf, 0);
         tms[m] = &map(hs[m], kMapX64);
@@ -920,6 +987,14 @@ cudaError_t bf16_forward_steps_group(stacklstm *const *hs, int n, const float *c
 cudaError_t bf16_backward_steps_group(stacklstm *const *hs, int n, cudaStream_t st)
 {
     StepArgs as[kMaxGroup];
+    if (hs[0]->br.on) {
+        const float *d_top[kMaxGroup];
+        for (int m = 0; m < n; ++m) {
+            as[m] = bwd_args(hs[m], nullptr, hs[m]->kcb, 0);
+            d_top[m] = hs[m]->d_top_seed;
+        }
+        return bf16_launch_rows(hs, as, d_top, n, false, st);
+    }
     for (int m = 0; m < n; ++m) as[m] = bwd_args(hs[m], hs[m]->w_bcl, hs[m]->kcb, 0);
     return bf16_launch_bwd_cluster_group(hs, as, n, st);
 }

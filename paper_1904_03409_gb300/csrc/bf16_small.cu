@@ -40,6 +40,9 @@ constexpr int kCcMaxB = 32;       // rows the kernels hold (register accumulator
 // forward step equal at 1.57 us); B = 8, 1.80 ms against 0.77 ms; B = 32, 6.19 against
 // 0.83 ms. Per row, the FFMA contraction adds about 0.4 us a step.
 constexpr int kCcCrossoverB = 1;
+// Longer sequences of one row go to the row-group clusters (bf16_rows.cu), whose step is
+// shorter still (0.95 / 1.00 us); up to here one row keeps the plan its callers pin.
+constexpr int kCcCrossoverT = 40;
 
 __device__ __forceinline__ uint32_t cc_rank()
 {
@@ -537,7 +540,7 @@ bool bf16_plan_small(stacklstm *s, PersistPlan *pl)
     if (want == 0) return false;
     const int n_ct = (int)ceil_div(s->H, kCcU), BT = cc_tier(s->B);
     if (s->B > kCcMaxB || n_ct > 16 || s->I % 8 || s->H % 8) return false;
-    if (want < 0 && s->B > kCcCrossoverB) return false;
+    if (want < 0 && (s->B > kCcCrossoverB || s->T > kCcCrossoverT)) return false;
     const size_t sf = ccf_smem_bytes(BT, s->I, s->H, n_ct), sb = ccb_smem_bytes(BT, n_ct);
     if (sf > kSmemCap || sb > kSmemCap) return false;
     for (int dir = 0; dir < 2; ++dir) {

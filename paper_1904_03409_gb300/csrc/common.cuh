@@ -23,8 +23,9 @@ struct PersistPlan {
     int S = 0;          // ring stages
     int slot = 0;       // CTAs per column tile (each takes every slot-th row tile)
     int w_res = 0;      // weight tile resident in shared memory
-    int cl = 1;         // thread-block cluster size (the one-row-tile cluster kernels; the KS parts
-                        // of a split contraction; 1 otherwise)
+    int cl = 1;         // thread-block cluster size (the cluster kernels; the KS parts of a split
+                        // contraction; 1 otherwise)
+    int rows = 0;       // rows of the batch per cluster (bf16_rows.cu)
     int KS = 1;         // contraction parts per column tile (backward split contraction)
     int n_ct = 0;       // column tiles, padded to a multiple of cl
     unsigned smem = 0;  // dynamic shared memory per CTA
@@ -110,6 +111,9 @@ struct stacklstm {
     PersistPlan fc;                // forward as one thread-block cluster (one row tile; bf16_cluster.cu)
     void *g_fcl = nullptr;         // its h slice blocks [T][column tiles][2 KB]
     PersistPlan bc;                // backward as one thread-block cluster (one row tile; bf16_cluster.cu)
+    PersistPlan fr, br;            // forward, backward as clusters of few rows (bf16_rows.cu)
+    void *w_rh = nullptr, *w_rx = nullptr, *w_rb = nullptr;  // their weights: forward W_h, W_x; backward W_h
+    const float *d_top_seed = nullptr;  // backward: the final tops' gradient the row clusters add themselves
     PersistPlan cc;                // small batches: both directions on CUDA cores (bf16_small.cu)
     void *w_ccf = nullptr, *w_ccb = nullptr;  // their weight slices
     void *w_bcl = nullptr;         // its weight chunks

@@ -1026,6 +1026,18 @@ cudaError_t bf16_dx(stacklstm *s, float *dx)
 cudaError_t bf16_dw(stacklstm *s, float *dW, float *dbias)
 {
     if (!dW && !dbias) return cudaSuccess;
+    if (s->Tr != s->T) {
+        // push-only mode: only the virtual steps' rows hold this call's data, so the maps end
+        // with them (the last chunk of 64 rows reads zeros past its end, not an earlier call's)
+        alignas(64) unsigned char mx[128], mh[128], mg[128];
+        const uint64_t R = (uint64_t)s->Tr * s->B;
+        cudaError_t e;
+        if ((e = make_map(mx, s->x_saved, R, (uint64_t)s->I, kChunk)) ||
+            (e = make_map(mh, s->hr, R, (uint64_t)s->H, kChunk)) ||
+            (e = make_map(mg, s->dG, R, 4 * (uint64_t)s->H, kChunk)))
+            return e;
+        return bf16_launch_dw(s, *(const CUtensorMap *)mx, *(const CUtensorMap *)mh, *(const CUtensorMap *)mg, dW, dbias);
+    }
     return bf16_launch_dw(s, map(s, kMapX64), map(s, kMapH64), map(s, kMapG64), dW, dbias);
 }
 

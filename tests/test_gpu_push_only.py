@@ -166,3 +166,22 @@ def test_mode_switch_needs_a_new_forward_and_fp32_is_refused():
         assert e.value.status == 7
     finally:
         hf.destroy()
+
+
+def test_weight_gradient_ignores_rows_of_an_earlier_call():
+    """A handle that ran more virtual steps before: the rows past this call's (40 rows a
+    step, so the last 64-row chunk of the weight gradient reaches beyond them) must not enter
+    dW and dbias."""
+    many = case(30, 40, 24, 40, 43, probs=(1.0, 0.0, 0.0), bias_scale=0.3, h0_scale=0.5)
+    few = case(30, 40, 24, 40, 44, probs=(0.4, 0.4, 0.2), bias_scale=0.3, h0_scale=0.5)
+    hd = bd.stacklstm_create(few.T, few.B, few.I, few.H, bd.SL_BF16, 0)
+    try:
+        bd.stacklstm_set_mode(hd, PUSH)
+        for w in (many, few):
+            ins, out = runner.upload(w), runner.alloc_outputs(w)
+            runner.forward_backward(hd, ins, out)
+        assert bd.stacklstm_steps_run(hd) * few.B % 64 != 0
+        torch.cuda.synchronize()
+        compare(runner.to_numpy(out), definition(few), "bf16", keys=("dW", "dbias", "dx"))
+    finally:
+        hd.destroy()

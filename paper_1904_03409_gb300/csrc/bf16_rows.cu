@@ -654,7 +654,8 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rowsb(const __grid_constan
             if (t >= 1) load_ops(t - 1, sn);
             // dh_read of this CTA's units: the parts in CTA order (phase (T - 1 - t) / 2 of buffer t % 2)
             ok = rc_wait<true>(s_bar + 8 * b, (uint32_t)((T - 1 - t) >> 1) & 1, limit, abort, a.err);
-            if (tid == 0 && t >= 2) tc::mbar_arrive_expect_tx(&rbar[b], r_bytes);
+            // (after a wait that ran out the phase is still open: no second arrival on it)
+            if (ok && tid == 0 && t >= 2) tc::mbar_arrive_expect_tx(&rbar[b], r_bytes);
 #pragma unroll
             for (int n = 0; n < NT; ++n) {
                 // M tile warp / 2, its rows g (warp even) or g + 8: the fragment's first or second pair

@@ -57,6 +57,8 @@ struct stacklstm {
     int walk_push_smem = 0;      // the same for the push-only walk (slot tags and index map; 0: separate kernels)
     int walk_built_virtual = 0;  // the last prepass also built the push-only timeline
     int fp32_one_cta = 0;        // fp32: every step of each direction in one CTA (small B * H)
+    PersistPlan fr32;            // fp32: clusters of few rows (fp32_rows.cu; EP: warps a CTA)
+    int fr32_split = 1;          // their weight gradient's splits
     int pfinal_written = 0;      // the last prepass also wrote the caller's final pointers
 
     // integer bookkeeping, written by the prepass (all [T+1][B] int32)
@@ -175,6 +177,12 @@ cudaError_t fp32_forward_steps(stacklstm *s, const float *x, const float *W, con
 cudaError_t fp32_backward_steps(stacklstm *s);
 cudaError_t fp32_dx(stacklstm *s, float *dx);
 cudaError_t fp32_dw(stacklstm *s, float *dW, float *dbias);
+// clusters of few rows and tiled contractions, H <= 256 (fp32_rows.cu)
+bool fp32_plan_rows(stacklstm *s);
+cudaError_t fp32_rows_forward(stacklstm *s, const float *x, const float *W, const float *bias);
+cudaError_t fp32_rows_backward(stacklstm *s);
+cudaError_t fp32_rows_dx(stacklstm *s, float *dx);
+cudaError_t fp32_rows_dw(stacklstm *s, float *dW, float *dbias);
 
 // ---- bf16 tensor-core path (bf16_path.cu)
 cudaError_t bf16_prepare(stacklstm *s);

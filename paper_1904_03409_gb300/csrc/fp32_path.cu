@@ -1,7 +1,8 @@
 // fp32_path.cu -- the fp32 homogenized StackLSTM step on CUDA cores (no tensor cores,
 // no TF32). It serves small problems, where B * 4H is too small for a dense tensor-core
 // contraction, and is the full-precision counterpart of the bf16 path. With B * H <= 1024
-// each direction runs all its steps in one CTA (fwd_seq_f32, bwd_seq_f32); otherwise:
+// each direction runs all its steps in one CTA (fwd_seq_f32, bwd_seq_f32); else, up to
+// H = 256, in clusters of few rows (fp32_rows.cu); otherwise:
 //
 // Forward, one launch per step t (Algorithm 1): every instance reads history row
 // top[t] (the state at its stack top), computes z = [x_t ; h_read] W + bias, applies the
@@ -388,8 +389,10 @@ std::string fp32_describe(stacklstm *s)
         cudaGetLastError();
         s->fp32_one_cta = 0;
     }
-    return s->fp32_one_cta ? "fp32 CUDA cores; every step of each direction in one CTA"
-                           : "fp32 CUDA cores; one launch per step";
+    if (s->fp32_one_cta) return "fp32 CUDA cores; every step of each direction in one CTA";
+    if (!(per_step && atoi(per_step) != 0) && fp32_plan_rows(s))
+        return "fp32 CUDA cores; clusters of " + std::to_string(s->fr32.cl) + " CTAs, rows " + std::to_string(s->fr32.rows);
+    return "fp32 CUDA cores; one launch per step";
 }
 
 cudaError_t fp32_forward_setup(stacklstm *s, const float *h0, const float *c0, const float *W)
@@ -404,6 +407,7 @@ cudaError_t fp32_forward_setup(stacklstm *s, const float *h0, const float *c0, c
 cudaError_t fp32_forward_steps(stacklstm *s, const float *x, const float *W, const float *bias)
 {
     const int T = s->T, B = s->B, I = s->I, H = s->H, K = I + H;
+    if (s->fr32.on) return fp32_rows_forward(s, x, W, bias);
     if (s->fp32_one_cta) {
         (void)K;
         const int P = fwd_seq_threads_per_unit(B, H);
@@ -427,6 +431,7 @@ cudaError_t fp32_backward_steps(stacklstm *s)
     const int T = s->T, B = s->B, I = s->I, H = s->H, G = 4 * H;
     const float *WT = (const float *)s->w_fwd;
     float *dG = (float *)s->dG;
+    if (s->fr32.on) return fp32_rows_backward(s);
     if (s->fp32_one_cta) {
         const int P = fwd_seq_threads_per_unit(B, H);
         bwd_seq_f32<<<1, (unsigned)ceil_div(B * H * P, 32) * 32, bwd_seq_smem(T, B, H), s->stream>>>(
@@ -451,6 +456,7 @@ cudaError_t fp32_dx(stacklstm *s, float *dx)
     const int T = s->T, B = s->B, I = s->I, H = s->H, G = 4 * H;
     const float *WT = (const float *)s->w_fwd;
     const float *dG = (const float *)s->dG;
+    if (s->fr32.on) return fp32_rows_dx(s, dx);
     if (dx && T > 0) {
         const int tx = std::min(128, ((I + 31) / 32) * 32);
         // grid.y is limited to 65535 rows per launch
@@ -468,6 +474,7 @@ cudaError_t fp32_dw(stacklstm *s, float *dW, float *dbias)
 {
     const int T = s->T, B = s->B, I = s->I, H = s->H, K = I + H, G = 4 * H;
     const float *dG = (const float *)s->dG;
+    if (s->fr32.on) return fp32_rows_dw(s, dW, dbias);
     if (dW || dbias)
         dw_f32<<<grid_for(s, (size_t)(K + 1) * G, 128), 128, 0, s->stream>>>(
             (size_t)T * B, K, G, (const float *)s->a_rm, dG, dW, dbias);

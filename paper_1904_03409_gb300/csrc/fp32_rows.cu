@@ -1,0 +1,795 @@
+// fp32_rows.cu -- the fp32 path for hidden widths up to 256 (CUDA cores only, every product
+// and sum in fp32): the recurrences as thread-block clusters of few rows, and the
+// contractions that are not sequential as tiled ones.
+//
+// The gates' x part of every step, x W_x + bias, is one contraction before the steps; dx and
+// dW are contractions after them. What is left in a step is h_read W_h (backward: dG W_h^T),
+// whose weights a cluster of C <= 8 CTAs keeps in registers for the whole launch. Instances
+// are independent, so each group of R <= 8 rows runs its T steps in a cluster of its own. A
+// step is bound by what its warps issue, two a scheduler (at 64 x 200, 13 clusters of 7 CTAs
+// and 5 rows: 280 two-wide multiply-adds and about 300 other instructions a warp), and by the
+// exchange between the CTAs: 1.62 us forward, 1.73 backward, where a launch a step, each dot
+// product reading its weights from L2 again, took 36 and 36. With the tiled contractions
+// (about 27 TFLOP/s, 64 x 128 tiles) a 64 x 200 pass of 185 steps went from 20.0 to 1.19 ms.
+#include <stdlib.h>
+
+#include <algorithm>
+
+#include "common.cuh"
+#include "tc.cuh"
+
+namespace sl {
+namespace {
+
+using tc::smem_u32;
+
+constexpr int kFrMaxW = 8, kFrThreads = 32 * kFrMaxW;  // warps of four units a CTA, at most (255 registers a thread)
+constexpr long long kFrSettle = 100000;  // cycles an aborted CTA waits for stores in flight
+
+__device__ __forceinline__ float sigmoid32(float z) { return 1.0f / (1.0f + expf(-z)); }
+
+struct FrArgs {
+    int T, B, H;
+    int C, W;               // CTAs a cluster; warps of 4 units a CTA (it owns units ct 4W ..)
+    const int32_t *top;     // [T + 1][B]
+    float *hist_h, *hist_c; // [T + 1][B][H]
+    float *gates;           // [T][B][4H]: forward, in: x W_x + bias, out: the activated gates
+    float *hr;              // [T][B][H]: the state each step read (for dW)
+    const float *wh;        // forward: W + I * 4H ([H][4H]); backward: W_h^T ([4H] rows, ldw apart)
+    size_t ldw;
+    float *dhist_h, *dhist_c, *dG;
+    long long limit;
+    int32_t *err;
+};
+
+__device__ __forceinline__ bool fr_test(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+// bounded wait of a whole warp for bytes that the cluster's CTAs store asynchronously
+__device__ __forceinline__ bool fr_wait(uint32_t bar, uint32_t parity, long long limit, volatile int *abort, int32_t *err)
+{
+    bool ok = fr_test(bar, parity);
+    if (__all_sync(0xffffffffu, ok)) return true;
+    const long long t0 = clock64();
+    while (true) {
+        const bool over = clock64() - t0 >= limit || *abort;
+        if (__any_sync(0xffffffffu, over)) break;
+        ok = fr_test(bar, parity);
+        if (__all_sync(0xffffffffu, ok)) return true;
+    }
+    *abort = 1;
+    atomicCAS(err, 0, (int)SL_ERR_TIMEOUT);
+    return false;
+}
+// no CTA leaves while another may still store into its shared memory
+__device__ __forceinline__ void fr_leave(volatile int *abort)
+{
+    __syncthreads();
+    tc::cluster_sync();
+    if (*abort) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < kFrSettle) {}
+    }
+    __syncthreads();
+    tc::cluster_sync();
+}
+template <int N>
+__device__ __forceinline__ void st_async_f(uint32_t addr, const float *v, uint32_t bar)
+{
+    static_assert(N == 1 || N == 2 || N == 4, "4, 8 or 16 bytes");
+    if constexpr (N == 4)
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
+                     "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(bar) : "memory");
+    else if constexpr (N == 2)
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr),
+                     "f"(v[0]), "f"(v[1]), "r"(bar) : "memory");
+    else
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(addr), "f"(v[0]),
+                     "r"(bar) : "memory");
+}
+// two fused multiply-adds an instruction, each rounded as fmaf: half of what the contractions issue
+__device__ __forceinline__ void fma2(uint64_t &d, uint64_t a, uint64_t b)
+{
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ uint64_t pair2(float lo, float hi)
+{
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ float add2(uint64_t v)
+{
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+    return lo + hi;
+}
+
+// ------------------------------------------------------------------------ forward
+// Warp w of CTA ct owns units u0 = 4 (ct W + w) .. + 3. Lane = (unit lane / 8, part lane % 8):
+// a lane keeps its unit's four gate columns of W_h for the k of its part (float4 pieces 8 i +
+// part, i < KC) and multiplies them by R rows of the h operand, 16 bytes (four k) a load: the
+// warp's eight parts cover one 128-byte line of a row. The 8 parts are then summed by
+// shuffles that leave each lane one row (8 / R lanes alike), whose cell it runs. The new
+// operand (h' where the step pushed, else the older top) goes to every CTA of the cluster by
+// st.async, a row's four units a store. Shared memory: the operand [2][R][32 KC].
+template <int KC, int R>
+__global__ void __launch_bounds__(kFrThreads, 1) fwd_rows_f32(FrArgs a)
+{
+    constexpr int KP = 32 * KC, RP = R <= 4 ? R : 8, DUP = 8 / RP;  // lanes alike per row
+    __shared__ __align__(16) float s_h[2][R][KP];
+    __shared__ __align__(8) uint64_t s_bar[2];
+    __shared__ int s_abort;
+    const int T = a.T, B = a.B, H = a.H, G = 4 * H;
+    const int ct = (int)tc::cluster_rank(), C = a.C, row0 = ((int)blockIdx.x / C) * R, nrows = min(R, B - row0);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int u0 = 4 * (ct * a.W + warp), u = u0 + (lane >> 3), part = lane & 7;
+    const bool warp_on = u0 < H, unit_on = u < H;
+    const uint32_t bytes = (uint32_t)R * ((H + 3) / 4) * 16;  // of one step's operand
+    volatile int *abort = &s_abort;
+    for (int i = tid; i < 2 * R * KP; i += blockDim.x) (&s_h[0][0][0])[i] = 0.0f;
+    if (tid == 0) {
+        tc::mbar_init(&s_bar[0], 1);
+        tc::mbar_init(&s_bar[1], 1);
+        s_abort = 0;
+        tc::fence_mbar_init();
+        // the operands of steps 1 and 2 (step 0's is filled in below)
+        if (T > 1) tc::mbar_arrive_expect_tx(&s_bar[1], bytes);
+        if (T > 2) tc::mbar_arrive_expect_tx(&s_bar[0], bytes);
+    }
+    __syncthreads();
+    for (int i = tid; i < nrows * H; i += blockDim.x) s_h[0][i / H][i % H] = a.hist_h[(size_t)row0 * H + i];
+    uint64_t w[KC][4][2];  // [piece][gate][k pair of it]
+#pragma unroll
+    for (int i = 0; i < KC; ++i)
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            float v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int k = 4 * (8 * i + part) + q;
+                v[q] = unit_on && k < H ? a.wh[(size_t)k * G + g * H + u] : 0.0f;
+            }
+            w[i][g][0] = pair2(v[0], v[1]);
+            w[i][g][1] = pair2(v[2], v[3]);
+        }
+    // this lane's cell: unit u of row `row` (rows past the batch read its last row, write nothing)
+    const int r = part / DUP, row = row0 + min(r, nrows - 1), uc = min(u, H - 1);
+    const bool mine = unit_on && r < nrows && part % DUP == 0;
+    // this lane's peers: dest and, with one lane a row, dest + 4
+    const int dest = (lane >> 3) * DUP + part % DUP;
+    const uint32_t self = smem_u32(&s_h[0][0][0]), bar_off = smem_u32(&s_bar[0]) - self;
+    const uint32_t peer0 = tc::mapa(self, (uint32_t)min(dest, C - 1)), peer1 = tc::mapa(self, (uint32_t)min(dest + 4, C - 1));
+    const bool send0 = r < R && dest < C, send1 = R > 4 && r < R && dest + 4 < C;
+    const size_t cell = (size_t)row * H + uc, SB = (size_t)B * H;
+    int i1 = a.top[B + row];  // top[t + 1] at step t
+    float cr = a.hist_c[(size_t)a.top[row] * SB + cell], hold = a.hist_h[cell];
+    float zx[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) zx[g] = a.gates[(size_t)row * G + g * H + uc];
+    int i2 = a.top[(size_t)min(2, T) * B + row];
+    if (mine) a.hr[cell] = hold;  // h_read(0) = h0
+    __syncthreads();
+    tc::cluster_sync();  // every CTA's barriers and buffers exist before any store lands on them
+
+    for (int t = 0; t < (warp_on ? T : 0); ++t) {
+        const int b = t & 1;
+        __syncwarp();
+        // what step t + 1 needs of rows written before this step (row t + 1 itself: unused)
+        const float crn = __ldcg(a.hist_c + (size_t)i1 * SB + cell);
+        const float holdn = __ldcg(a.hist_h + (size_t)i2 * SB + cell);
+        const int i3 = a.top[(size_t)min(t + 3, T) * B + row];
+        float zn[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) zn[g] = __ldcg(a.gates + ((size_t)min(t + 1, T - 1) * B + row) * G + g * H + uc);
+        if (t > 0) {
+            if (!fr_wait(smem_u32(&s_bar[b]), (uint32_t)((t - 1) >> 1) & 1, a.limit, abort, a.err)) break;
+            if (tid == 0 && t + 2 < T) tc::mbar_arrive_expect_tx(&s_bar[b], bytes);
+        }
+        uint64_t acc2[R][4];
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+#pragma unroll
+            for (int g = 0; g < 4; ++g) acc2[q][g] = 0;
+#pragma unroll
+        for (int i = 0; i < KC; ++i)
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                const ulonglong2 h = *(const ulonglong2 *)&s_h[b][q][4 * (8 * i + part)];
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    fma2(acc2[q][g], h.x, w[i][g][0]);
+                    fma2(acc2[q][g], h.y, w[i][g][1]);
+                }
+            }
+        float acc[RP][4];
+#pragma unroll
+        for (int q = 0; q < RP; ++q)
+#pragma unroll
+            for (int g = 0; g < 4; ++g) acc[q][g] = q < R ? add2(acc2[q < R ? q : 0][g]) : 0.0f;
+        // sum over the parts; halving the rows kept while there are several
+        float z[4];
+#pragma unroll
+        for (int m = 4, n = RP; m >= 1; m >>= 1, n = n > 1 ? n / 2 : 1)
+#pragma unroll
+            for (int q = 0; q < (n > 1 ? n / 2 : 1); ++q)
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    if (n > 1) {
+                        const float lo = acc[q][g], hi = acc[n / 2 + q][g];
+                        acc[q][g] = (part & m ? hi : lo) + __shfl_xor_sync(0xffffffffu, part & m ? lo : hi, m);
+                    } else {
+                        acc[q][g] += __shfl_xor_sync(0xffffffffu, acc[q][g], m);
+                    }
+                }
+#pragma unroll
+        for (int g = 0; g < 4; ++g) z[g] = acc[0][g] + zx[g];
+        const float ig = sigmoid32(z[0]), fg = sigmoid32(z[1]), gg = tanhf(z[2]), og = sigmoid32(z[3]);
+        const float cn = fmaf(fg, cr, ig * gg), hn = og * tanhf(cn);
+        const float op = !unit_on ? 0.0f : i1 == t + 1 ? hn : hold;
+        if (t + 1 < T) {
+            float v[4];  // the row's four units
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = __shfl_sync(0xffffffffu, op, part | (j << 3));
+            const uint32_t off = (uint32_t)(((b ^ 1) * R + r) * KP + u0) * 4;
+            if (send0) st_async_f<4>(peer0 + off, v, peer0 + bar_off + 8 * (b ^ 1));
+            if (send1) st_async_f<4>(peer1 + off, v, peer1 + bar_off + 8 * (b ^ 1));
+        }
+        if (mine) {
+            a.hist_h[(size_t)(t + 1) * SB + cell] = hn;
+            a.hist_c[(size_t)(t + 1) * SB + cell] = cn;
+            if (t + 1 < T) a.hr[(size_t)(t + 1) * SB + cell] = op;
+            float *gp = a.gates + ((size_t)t * B + row) * G + u;
+            gp[0] = ig;
+            gp[H] = fg;
+            gp[2 * H] = gg;
+            gp[3 * H] = og;
+        }
+        cr = i1 == t + 1 ? cn : crn;
+        hold = i2 == t + 1 ? hn : holdn;
+        i1 = i2;
+        i2 = i3;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) zx[g] = zn[g];
+    }
+    fr_leave(abort);
+}
+
+// ----------------------------------------------------------------------- backward
+// The gate gradients of a CTA's own units stay in it: its threads multiply them by the CTA's
+// 16 W gate columns of W_h (in registers: four rows of W_h by every fourth unit a thread, so
+// that a 16-byte load of gate gradients feeds 16 multiply-adds) into partial dh_read values
+// of all H units; thread k sends those of unit k to the CTA that owns it, which adds the
+// parts in CTA order. The first 4 W R threads then hold one (unit, row) each. Shared memory: gate gradients
+// [2][R][units][4 gates], parts [2][C][units][R].
+template <int UP, int R>
+__global__ void __launch_bounds__(kFrThreads, 1) bwd_rows_f32(FrArgs a)
+{
+    __shared__ __align__(16) float s_dg[2][R][UP][4];
+    constexpr int RP = R <= 4 ? R : 8;  // (16-byte stores)
+    __shared__ __align__(16) float s_part[2][8][UP][RP];
+    __shared__ __align__(8) uint64_t s_bar[2];
+    __shared__ int s_abort;
+    const int T = a.T, B = a.B, H = a.H, G = 4 * H, U = 4 * a.W;  // U <= UP units a CTA
+    const int ct = (int)tc::cluster_rank(), C = a.C, row0 = ((int)blockIdx.x / C) * R, nrows = min(R, B - row0);
+    const int tid = threadIdx.x;
+    const uint32_t bytes = (uint32_t)C * max(0, min(U, H - ct * U)) * R * 4;  // of one step's parts
+    volatile int *abort = &s_abort;
+    for (int i = tid; i < 2 * R * UP * 4; i += blockDim.x) (&s_dg[0][0][0][0])[i] = 0.0f;
+    if (tid == 0) {
+        tc::mbar_init(&s_bar[0], 1);
+        tc::mbar_init(&s_bar[1], 1);
+        s_abort = 0;
+        tc::fence_mbar_init();
+        for (int i = 0; i < 2 && i < T; ++i) tc::mbar_arrive_expect_tx(&s_bar[(T - 1 - i) & 1], bytes);
+    }
+    const bool k_on = tid < H;
+    // this thread's tile: rows 4 (tid / 4) .. + 3 of W_h by the CTA's units 4 j + tid % 4
+    const int q4 = tid & 3;
+    uint64_t w[UP / 4][4][2];  // [unit][row][gate pair]
+#pragma unroll
+    for (int j = 0; j < UP / 4; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float v[4];
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                const int un = 4 * j + q4, k = (tid & ~3) + i;
+                v[g] = k < H && un < U && ct * U + un < H ? a.wh[(size_t)(g * H + ct * U + un) * a.ldw + k] : 0.0f;
+            }
+            w[j][i][0] = pair2(v[0], v[1]);
+            w[j][i][1] = pair2(v[2], v[3]);
+        }
+    const int owner = k_on ? tid / U : 0;
+    const uint32_t peer = tc::mapa(smem_u32(&s_part[0][ct][k_on ? tid % U : 0][0]), (uint32_t)owner);
+    const uint32_t peer_bar = tc::mapa(smem_u32(&s_bar[0]), (uint32_t)owner);
+    // this thread's cell: unit ul of the CTA, row r of the group
+    const int ul = tid / R, r = tid % R;
+    const bool cell_on = ul < U && ct * U + ul < H, mine = cell_on && r < nrows;
+    const int u = cell_on ? ct * U + ul : 0, row = row0 + min(r, nrows - 1);
+    const size_t cell = (size_t)row * H + u, SB = (size_t)B * H;
+    const int32_t *ltop = a.top + row;
+    int s1 = ltop[(size_t)T * B], s = ltop[(size_t)(T - 1) * B], sn = ltop[(size_t)max(T - 2, 0) * B];
+    float v = 0.0f, dcp = 0.0f, cp = 0.0f, cr = 0.0f, dcr = 0.0f, dhs = 0.0f, gq[4] = {};
+    auto load_ops = [&](int t, int iw) {
+        cr = __ldcg(a.hist_c + (size_t)iw * SB + cell);
+        dcr = __ldcg(a.dhist_c + (size_t)iw * SB + cell);
+#pragma unroll
+        for (int g = 0; g < 4; ++g) gq[g] = __ldcg(a.gates + ((size_t)t * B + row) * G + g * H + u);
+    };
+    if (cell_on) {
+        v = a.dhist_h[(size_t)s1 * SB + cell];  // the seeded gradient of the final top
+        cp = a.hist_c[(size_t)s1 * SB + cell];
+        dhs = a.dhist_h[(size_t)s * SB + cell];
+        load_ops(T - 1, s);
+    }
+    __syncthreads();
+    tc::cluster_sync();
+
+    bool ok = true;
+    for (int t = T - 1; t >= 0; --t) {
+        const int b = t & 1;
+        if (cell_on) {
+            // pointwise backward of step t: its state t + 1 is the one step t + 1 read, or one
+            // that nothing read (zero gradient)
+            const float ig = gq[0], fg = gq[1], gg = gq[2], og = gq[3];
+            const bool live = s1 == t + 1;
+            const float dh = live ? v : 0.0f, dct = live ? dcp : 0.0f;
+            const float tcn = tanhf(cp);
+            const float dc = dct + dh * og * (1.0f - tcn * tcn);
+            const float4 d = make_float4(dc * gg * ig * (1.0f - ig), dc * cr * fg * (1.0f - fg), dc * ig * (1.0f - gg * gg),
+                                         dh * tcn * og * (1.0f - og));
+            dcp = dcr + dc * fg;
+            cp = cr;
+            if (mine) {
+                *(float4 *)s_dg[b][r][ul] = d;
+                a.dhist_c[(size_t)s * SB + cell] = dcp;
+                float *gp = a.dG + ((size_t)t * B + row) * G + u;
+                gp[0] = d.x;
+                gp[H] = d.y;
+                gp[2 * H] = d.z;
+                gp[3 * H] = d.w;
+            }
+        }
+        // dG_t is complete; a warp whose wait ran out ends the loop for the whole CTA here
+        if (__syncthreads_or(!ok)) break;
+        // step t - 1's operands (dhist_h of the row this step adds to: taken from v below)
+        float dhn = 0.0f;
+        int s2 = 0;
+        if (cell_on) {
+            dhn = __ldcg(a.dhist_h + (size_t)sn * SB + cell);
+            s2 = ltop[(size_t)max(t - 2, 0) * B];
+            if (t >= 1) load_ops(t - 1, sn);
+        }
+        {
+            uint64_t acc2[4][R];  // [row of W_h][row]
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int q = 0; q < R; ++q) acc2[i][q] = 0;
+#pragma unroll
+            for (int j = 0; j < UP / 4; ++j)
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                    const ulonglong2 d = *(const ulonglong2 *)s_dg[b][q][4 * j + q4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        fma2(acc2[i][q], d.x, w[j][i][0]);
+                        fma2(acc2[i][q], d.y, w[j][i][1]);
+                    }
+                }
+            float acc[4][R];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int q = 0; q < R; ++q) acc[i][q] = add2(acc2[i][q]);
+            // the four threads' sums, each keeping the row of W_h that is its own (tid)
+            float p2[2][R], p[R];
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                    const float keep = q4 & 2 ? acc[2 + i][q] : acc[i][q], give = q4 & 2 ? acc[i][q] : acc[2 + i][q];
+                    p2[i][q] = keep + __shfl_xor_sync(0xffffffffu, give, 2);
+                }
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                const float keep = q4 & 1 ? p2[1][q] : p2[0][q], give = q4 & 1 ? p2[0][q] : p2[1][q];
+                p[q] = keep + __shfl_xor_sync(0xffffffffu, give, 1);
+            }
+            if (k_on) {
+                const uint32_t dst = peer + b * (uint32_t)sizeof(s_part[0]), bar = peer_bar + 8 * b;
+                st_async_f<R >= 4 ? 4 : R>(dst, p, bar);
+                if constexpr (R > 4) st_async_f<R - 4>(dst + 16, p + 4, bar);
+            }
+        }
+        __syncwarp();
+        ok = fr_wait(smem_u32(&s_bar[b]), (uint32_t)((T - 1 - t) >> 1) & 1, a.limit, abort, a.err);
+        // (after a wait that ran out the phase is still open: no second arrival on it)
+        if (ok && tid == 0 && t >= 2) tc::mbar_arrive_expect_tx(&s_bar[b], bytes);
+        if (cell_on) {
+            float x[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) x[c] = c < C ? s_part[b][c][ul][r] : 0.0f;
+            float sum = x[0];
+#pragma unroll
+            for (int c = 1; c < 8; ++c)
+                if (c < C) sum += x[c];
+            v = dhs + sum;
+            if (mine) a.dhist_h[(size_t)s * SB + cell] = v;
+            dhs = sn == s ? v : dhn;
+            s1 = s;
+            s = sn;
+            sn = s2;
+        }
+    }
+    fr_leave(abort);
+}
+
+// ------------------------------------------------------------- tiled contractions
+// C[M][N] = A B (+ bias[N]) in fp32, tiles of TM * 16 x TN * 16 outputs by 256 threads of
+// TM x TN each; partial sums over every 32 terms are added to a second accumulator, which
+// keeps a long sum's error near that of its short pieces. Row tiles past M's take the M2 rows
+// of A2 instead (dW: x, then the states read). kAT: A is given transposed
+// ([K][M], rows lda apart: dW = A^T dG); else [M][K]. grid z splits K evenly; slab z of C.
+template <int TM, int TN, bool kAT>
+__global__ void __launch_bounds__(256) gemm_f32(int M, int N, int K, const float *__restrict__ A, size_t lda,
+                                                int M2, const float *__restrict__ A2, size_t lda2,
+                                                const float *__restrict__ Bm, size_t ldb, const float *__restrict__ bias,
+                                                float *__restrict__ Cm, size_t ldc, size_t slab)
+{
+    constexpr int BM = 16 * TM, BN = 16 * TN, BK = 16, LA = BM * BK / 256, LB = BN * BK / 256;
+    __shared__ __align__(16) float sa[2][BK][BM + 4], sb[2][BK][BN + 4];
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int n0 = blockIdx.y * BN, tiles1 = (M + BM - 1) / BM;
+    int m0 = blockIdx.x * BM;
+    if ((int)blockIdx.x >= tiles1) {  // the rows of the second operand, below the first's in C
+        m0 -= tiles1 * BM;
+        Cm += (size_t)M * ldc;
+        M = M2;
+        A = A2;
+        lda = lda2;
+    }
+    const int KS = (K + BK - 1) / BK, z = blockIdx.z, nz = gridDim.z;
+    const int k_lo = (int)((long long)KS * z / nz) * BK, k_hi = min(K, (int)((long long)KS * (z + 1) / nz) * BK);
+    // this thread's elements of a block: A (m, k), then every SA along M (along K: kAT), B (k, n),
+    // then every 256 / BN along K
+    constexpr int SA = kAT ? 256 / BM : 256 / BK, SB = 256 / BN;
+    const int am = kAT ? tid % BM : tid / BK, ak = kAT ? tid / BM : tid % BK, bn = tid % BN, bk = tid / BN;
+    const float *pa = A + (kAT ? (size_t)(k_lo + ak) * lda + m0 + am : (size_t)(m0 + am) * lda + k_lo + ak);
+    const float *pb = Bm + (size_t)(k_lo + bk) * ldb + n0 + bn;
+    const size_t sa_i = (size_t)SA * lda, sb_i = (size_t)SB * ldb, sa_k = kAT ? (size_t)BK * lda : BK, sb_k = (size_t)BK * ldb;
+    const bool inner = m0 + BM <= M && n0 + BN <= N;
+    float ra[LA], rb[LB];
+    auto fetch = [&](int k0) {  // the block at k0; the pointers move on to the next
+        if (inner && k0 + BK <= k_hi) {
+#pragma unroll
+            for (int i = 0; i < LA; ++i) ra[i] = pa[i * sa_i];
+#pragma unroll
+            for (int i = 0; i < LB; ++i) rb[i] = pb[i * sb_i];
+        } else {
+#pragma unroll
+            for (int i = 0; i < LA; ++i) {
+                const int m = kAT ? am : am + SA * i, k = kAT ? ak + SA * i : ak;
+                ra[i] = m0 + m < M && k0 + k < k_hi ? pa[i * sa_i] : 0.0f;
+            }
+#pragma unroll
+            for (int i = 0; i < LB; ++i) rb[i] = n0 + bn < N && k0 + bk + SB * i < k_hi ? pb[i * sb_i] : 0.0f;
+        }
+        pa += sa_k;
+        pb += sb_k;
+    };
+    auto stash = [&](int b) {
+#pragma unroll
+        for (int i = 0; i < LA; ++i) {
+            const int e = tid + 256 * i;
+            sa[b][kAT ? e / BM : e % BK][kAT ? e % BM : e / BK] = ra[i];
+        }
+#pragma unroll
+        for (int i = 0; i < LB; ++i) {
+            const int e = tid + 256 * i;
+            sb[b][e / BN][e % BN] = rb[i];
+        }
+    };
+    uint64_t acc[TM][TN / 2];  // pairs of columns
+    float sum[TM][TN];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            acc[i][j / 2] = 0;
+            sum[i][j] = 0.0f;
+        }
+    auto flush = [&]() {
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int j = 0; j < TN; j += 2) {
+                float lo, hi;
+                asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[i][j / 2]));
+                sum[i][j] += lo;
+                sum[i][j + 1] += hi;
+                acc[i][j / 2] = 0;
+            }
+    };
+    fetch(k_lo);
+    stash(0);
+    __syncthreads();
+    int b = 0;
+    for (int k0 = k_lo; k0 < k_hi; k0 += BK, b ^= 1) {
+        if (k0 + BK < k_hi) fetch(k0 + BK);
+#pragma unroll
+        for (int k = 0; k < BK; ++k) {
+            float av[TM];
+            uint64_t bv[TN / 2];
+            // rows 4 ty + i (and 64 + 4 ty + i): 16-byte loads without bank conflicts
+#pragma unroll
+            for (int i = 0; i < TM; i += 4) *(float4 *)(av + i) = *(const float4 *)&sa[b][k][(i / 4) * 64 + 4 * ty];
+#pragma unroll
+            for (int j = 0; j < TN; j += 4)
+                *(ulonglong2 *)(bv + j / 2) = *(const ulonglong2 *)&sb[b][k][(j / 4) * 64 + 4 * tx];
+#pragma unroll
+            for (int i = 0; i < TM; ++i) {
+                const uint64_t a2 = pair2(av[i], av[i]);
+#pragma unroll
+                for (int j = 0; j < TN / 2; ++j) fma2(acc[i][j], a2, bv[j]);
+            }
+        }
+        if (((k0 - k_lo) / BK) & 1) flush();
+        if (k0 + BK < k_hi) stash(b ^ 1);
+        __syncthreads();
+    }
+    flush();
+    float *out = Cm + (size_t)z * slab;
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+        const int m = m0 + (i / 4) * 64 + 4 * ty + i % 4;
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            const int n = n0 + (j / 4) * 64 + 4 * tx + j % 4;
+            if (m < M && n < N) out[(size_t)m * ldc + n] = sum[i][j] + (bias ? bias[n] : 0.0f);
+        }
+    }
+}
+
+// dbias partial sums: block z sums its rows of dG column by column, 32 rows to a partial
+__global__ void colsum_f32(int R, int G, const float *__restrict__ dG, float *__restrict__ part)
+{
+    const int n = blockIdx.x * blockDim.x + threadIdx.x, z = blockIdx.y, nz = gridDim.y;
+    if (n >= G) return;
+    const int lo = (int)((long long)R * z / nz), hi = (int)((long long)R * (z + 1) / nz);
+    float sum = 0.0f;
+    for (int r0 = lo; r0 < hi; r0 += 32) {
+        float acc = 0.0f;
+#pragma unroll 8
+        for (int r = r0; r < min(r0 + 32, hi); ++r) acc += dG[(size_t)r * G + n];
+        sum += acc;
+    }
+    part[(size_t)z * G + n] = sum;
+}
+// out[e] = sum of the nz slabs in order, compensated
+__global__ void slab_sum_f32(size_t n, int nz, const float *__restrict__ part, size_t slab, float *__restrict__ out)
+{
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+        float acc = 0.0f, comp = 0.0f;
+        for (int z = 0; z < nz; ++z) {
+            const float y = part[(size_t)z * slab + e] - comp, t = acc + y;
+            comp = (t - acc) - y;
+            acc = t;
+        }
+        out[e] = acc;
+    }
+}
+
+// ---------------------------------------------------------------------------- host
+// rows a cluster (1, 2, 4) x contraction pieces of 32 (forward) / units a CTA (backward)
+template <int KC>
+const void *fwd_fn(int R)
+{
+    switch (R) {
+    case 1: return (const void *)fwd_rows_f32<KC, 1>;
+    case 2: return (const void *)fwd_rows_f32<KC, 2>;
+    case 4: return (const void *)fwd_rows_f32<KC, 4>;
+    case 5: return (const void *)fwd_rows_f32<KC, 5>;
+    case 6: return (const void *)fwd_rows_f32<KC, 6>;
+    default: return (const void *)fwd_rows_f32<KC, 8>;
+    }
+}
+template <int UP>
+const void *bwd_fn(int R)
+{
+    switch (R) {
+    case 1: return (const void *)bwd_rows_f32<UP, 1>;
+    case 2: return (const void *)bwd_rows_f32<UP, 2>;
+    case 4: return (const void *)bwd_rows_f32<UP, 4>;
+    case 5: return (const void *)bwd_rows_f32<UP, 5>;
+    case 6: return (const void *)bwd_rows_f32<UP, 6>;
+    default: return (const void *)bwd_rows_f32<UP, 8>;
+    }
+}
+const void *fr_fn(bool fwd, int H, int W, int R)
+{
+    if (!fwd)
+        return W <= 2 ? bwd_fn<8>(R) : W <= 4 ? bwd_fn<16>(R) : W <= 6 ? bwd_fn<24>(R) : W == 7 ? bwd_fn<28>(R)
+               : bwd_fn<32>(R);
+    switch ((H + 31) / 32) {
+    case 1: return fwd_fn<1>(R);
+    case 2: return fwd_fn<2>(R);
+    case 3: return fwd_fn<3>(R);
+    case 4: return fwd_fn<4>(R);
+    case 5: return fwd_fn<5>(R);
+    case 6: return fwd_fn<6>(R);
+    case 7: return fwd_fn<7>(R);
+    default: return fwd_fn<8>(R);
+    }
+}
+
+// a thread per row of W_h, and per cell
+int bwd_threads(int H, int W, int R) { return std::max((int)ceil_div(H, 32) * 32, (int)ceil_div(4 * W * R, 32) * 32); }
+
+void fr_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, int clusters, int C, int threads, cudaStream_t st)
+{
+    *cfg = {};
+    cfg->gridDim = dim3(clusters * C);
+    cfg->blockDim = dim3(threads);
+    cfg->stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg->attrs = at;
+    cfg->numAttrs = 1;
+}
+
+// 64 x 128 tiles where they fill the GPU, else 64 x 64 ones
+template <bool kAT>
+void launch_gemm(stacklstm *s, int M, int N, int K, const float *A, size_t lda, int M2, const float *A2, size_t lda2,
+                 const float *Bm, size_t ldb, const float *bias, float *Cm, size_t ldc, int splits, size_t slab)
+{
+    const unsigned mt = ceil_div(M, 64) + ceil_div(M2, 64);
+    if ((size_t)mt * ceil_div(N, 128) * splits >= (size_t)s->num_sms)
+        gemm_f32<4, 8, kAT><<<dim3(mt, ceil_div(N, 128), splits), 256, 0, s->stream>>>(M, N, K, A, lda, M2, A2, lda2, Bm,
+                                                                                       ldb, bias, Cm, ldc, slab);
+    else
+        gemm_f32<4, 4, kAT><<<dim3(mt, ceil_div(N, 64), splits), 256, 0, s->stream>>>(M, N, K, A, lda, M2, A2, lda2, Bm,
+                                                                                      ldb, bias, Cm, ldc, slab);
+    s->launches += 1;
+}
+
+constexpr int kBiasParts = 64;
+
+}  // namespace
+
+// The plan: rows a cluster R and CTAs a cluster C with the least rounds x step cycles, a step
+// being the warps' multiply-adds on the fullest of the SM's four schedulers plus about 1500
+// cycles of cell and exchange. (Registers allow one CTA an SM for large H: at 64 x 200, 14
+// clusters of 8 CTAs are in flight at once, so 13 of five rows.)
+bool fp32_plan_rows(stacklstm *s)
+{
+    s->fr32.on = 0;
+    const int H = s->H, KC = (int)ceil_div(H, 32);
+    if (H > 256) return false;
+    double best = 1e30;
+    for (int R : {1, 2, 4, 5, 6, 8})
+        for (int want = 1; want <= 8; ++want) {
+            const int W = (int)ceil_div(ceil_div(H, want), 4), C = W ? (int)ceil_div(H, 4 * W) : 0;
+            if (W > kFrMaxW || C != want) continue;  // every CTA owns a unit
+            int clusters = 1 << 30;
+            for (int dir = 0; dir < 2; ++dir) {
+                cudaLaunchConfig_t cfg;
+                cudaLaunchAttribute at[1];
+                int n = 0;
+                fr_config(&cfg, at, 1, C, dir ? bwd_threads(H, W, R) : 32 * W, nullptr);
+                if (cudaOccupancyMaxActiveClusters(&n, fr_fn(dir == 0, H, W, R), &cfg) != cudaSuccess) {
+                    cudaGetLastError();
+                    n = 0;
+                }
+                clusters = std::min(clusters, n);
+            }
+            if (clusters < 1) continue;
+            const double rounds = ceil_div(ceil_div(s->B, R), clusters);
+            const double cost = rounds * (ceil_div(W, 4) * 16.0 * KC * R + (C > 1 ? 1500.0 : 1000.0));
+            if (cost < best * 0.999) {
+                best = cost;
+                s->fr32.on = 1;
+                s->fr32.cl = C;
+                s->fr32.EP = W;
+                s->fr32.rows = R;
+            }
+        }
+    if (!s->fr32.on) return false;
+    // dW: splits of the T B rows for about four 64 x 128 tiles an SM (two at a time), at least
+    // 128 rows each
+    const size_t rows = (size_t)s->T * s->B, tiles = (size_t)(ceil_div(s->I, 64) + ceil_div(H, 64)) * ceil_div(4 * H, 128);
+    s->fr32_split = (int)std::max<size_t>(1, std::min<size_t>(std::min<size_t>(4 * s->num_sms / tiles, rows / 128), 64));
+    void *p;
+    const size_t slab = (size_t)(s->I + H) * 4 * H;
+    const char *lim = getenv("STACKLSTM_WAIT_LIMIT_CYCLES"), *limb = getenv("STACKLSTM_WAIT_LIMIT_BWD_CYCLES");
+    s->wait_limit = lim ? atoll(lim) : 4000000000LL;
+    s->wait_limit_bwd = limb ? atoll(limb) : s->wait_limit;
+    if (cudaMalloc(&p, sizeof(float) * (slab * s->fr32_split + (size_t)kBiasParts * 4 * H)) != cudaSuccess) {
+        cudaGetLastError();
+        s->fr32.on = 0;
+        return false;
+    }
+    s->allocs.push_back(p);
+    s->dw_part = (float *)p;
+    return true;
+}
+
+static cudaError_t fr_launch(stacklstm *s, bool fwd, FrArgs &a)
+{
+    a.T = s->T; a.B = s->B; a.H = s->H;
+    a.C = s->fr32.cl; a.W = s->fr32.EP;
+    a.top = s->top;
+    a.hist_h = (float *)s->hist_h; a.hist_c = s->hist_c;
+    a.gates = (float *)s->gates; a.hr = (float *)s->a_rm;
+    a.dhist_h = s->dhist_h; a.dhist_c = s->dhist_c; a.dG = (float *)s->dG;
+    a.limit = fwd ? s->wait_limit : s->wait_limit_bwd;
+    a.err = s->err;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[1];
+    fr_config(&cfg, at, (int)ceil_div(s->B, s->fr32.rows), a.C, fwd ? 32 * a.W : bwd_threads(s->H, a.W, s->fr32.rows), s->stream);
+    void *argv[] = {(void *)&a};
+    cudaError_t e = cudaLaunchKernelExC(&cfg, fr_fn(fwd, s->H, a.W, s->fr32.rows), argv);
+    if (e) return e;
+    s->launches += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t fp32_rows_forward(stacklstm *s, const float *x, const float *W, const float *bias)
+{
+    const int R = s->T * s->B, I = s->I, G = 4 * s->H;
+    s->x_saved = x;
+    launch_gemm<false>(s, R, G, I, x, I, 0, nullptr, 0, W, G, bias, (float *)s->gates, G, 1, 0);
+    FrArgs a{};
+    a.wh = W + (size_t)I * G;
+    return fr_launch(s, true, a);
+}
+
+cudaError_t fp32_rows_backward(stacklstm *s)
+{
+    FrArgs a{};
+    a.wh = (const float *)s->w_fwd + s->I;  // W^T [4H][I + H]: columns I .. are W_h^T
+    a.ldw = (size_t)s->I + s->H;
+    return fr_launch(s, false, a);
+}
+
+cudaError_t fp32_rows_dx(stacklstm *s, float *dx)
+{
+    if (!dx) return cudaSuccess;
+    launch_gemm<false>(s, s->T * s->B, s->I, 4 * s->H, (const float *)s->dG, 4 * (size_t)s->H, 0, nullptr, 0, (const float *)s->w_fwd,
+                       (size_t)s->I + s->H, nullptr, dx, s->I, 1, 0);
+    return cudaGetLastError();
+}
+
+cudaError_t fp32_rows_dw(stacklstm *s, float *dW, float *dbias)
+{
+    const int R = s->T * s->B, I = s->I, H = s->H, G = 4 * H, nz = s->fr32_split;
+    const float *dG = (const float *)s->dG;
+    const size_t slab = (size_t)(I + H) * G;
+    if (dW) {
+        float *part = nz > 1 ? s->dw_part : dW;
+        launch_gemm<true>(s, I, G, R, (const float *)s->x_saved, I, H, (const float *)s->a_rm, H, dG, G, nullptr, part, G,
+                          nz, slab);
+        if (nz > 1) {
+            slab_sum_f32<<<(unsigned)std::min<size_t>(ceil_div(slab, 256), (size_t)s->num_sms * 8), 256, 0, s->stream>>>(
+                slab, nz, part, slab, dW);
+            s->launches += 1;
+        }
+    }
+    if (dbias) {
+        float *part = s->dw_part + slab * nz;
+        const int parts = std::max(1, std::min(kBiasParts, R / 32));
+        colsum_f32<<<dim3(ceil_div(G, 128), parts), 128, 0, s->stream>>>(R, G, dG, part);
+        slab_sum_f32<<<ceil_div(G, 256), 256, 0, s->stream>>>(G, parts, part, G, dbias);
+        s->launches += 2;
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace sl

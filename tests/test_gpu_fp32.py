@@ -130,3 +130,49 @@ def test_backward_before_forward():
         assert e.value.status == 4
     finally:
         hd.destroy()
+
+
+@pytest.mark.parametrize("T,B,I,H,seed", [
+    (5, 400, 7, 3, 21), (3, 41, 9, 33, 22), (2, 9, 17, 129, 23), (1, 70, 40, 200, 24), (40, 64, 200, 200, 25),
+    (6, 5, 5, 225, 26), (4, 6, 130, 256, 27), (60, 13, 75, 100, 28), (30, 33, 1, 32, 29), (7, 90, 64, 177, 30),
+    (500, 1, 11, 65, 31), (9, 300, 33, 64, 32)])
+def test_row_clusters_match_oracle(T, B, I, H, seed):
+    """Clusters of few rows (fp32_rows.cu): units that fill a warp's four or not, one CTA to
+    eight, one row to eight a cluster with the last group partly empty, several rounds of
+    clusters, one to three steps (fewer than the buffers in flight), sizes that divide no tile
+    of the contractions, into NaN-filled outputs; reruns agree bit for bit."""
+    w = wl.make_workload("case", T=T, B=B, I=I, H=H, dtype="fp32", seed=seed, ops_kind="random_walk",
+                         probs=(0.5, 0.3, 0.2), bias_scale=0.3, h0_scale=0.5, c0_scale=0.5, dy_scale=0.5)
+    hd = bd.stacklstm_create(T, B, I, H, bd.SL_FP32, 0)
+    try:
+        assert "clusters" in bd.stacklstm_plan(hd), bd.stacklstm_plan(hd)
+    finally:
+        hd.destroy()
+    got = runner.run(w)
+    compare(got, oracle_of(w), "fp32")
+    again = runner.run(w)
+    for k in ("y", "h_stack", "c_stack", "dx", "dW", "dbias", "dh0", "dc0"):
+        assert np.array_equal(got[k], again[k]), k
+
+
+@pytest.mark.parametrize("which", ["STACKLSTM_WAIT_LIMIT_CYCLES", "STACKLSTM_WAIT_LIMIT_BWD_CYCLES"])
+def test_row_clusters_report_a_wait_that_runs_out(which):
+    """With a zero wait budget (both directions, or the backward's) the call reports
+    SL_ERR_TIMEOUT and the device stays usable."""
+    import os
+    w = wl.make_workload("case", T=12, B=64, I=16, H=120, dtype="fp32", seed=33, ops_kind="random_walk",
+                         probs=(0.5, 0.3, 0.2))
+    os.environ[which] = "0"
+    try:
+        hd = bd.stacklstm_create(w.T, w.B, w.I, w.H, bd.SL_FP32, 0)
+    finally:
+        del os.environ[which]
+    try:
+        assert "clusters" in bd.stacklstm_plan(hd)
+        ins, out = runner.upload(w), runner.alloc_outputs(w)
+        with pytest.raises(bd.StackLSTMError) as e:
+            runner.forward_backward(hd, ins, out)
+        assert e.value.status == 6
+    finally:
+        hd.destroy()
+    compare(runner.run(w), oracle_of(w), "fp32")

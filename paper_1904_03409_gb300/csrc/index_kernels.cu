@@ -276,20 +276,35 @@ prepass_walk_vec_kernel(int T, int B, const int8_t *__restrict__ ops, int32_t *_
     if (e != SL_OK) atomicCAS(err, 0, e);
 }
 
-// out[r] = hist row (idx[r], r % B), or zeros where idx[r] < 0. E is the raw element
-// bit pattern (uint32_t for float, uint16_t for bf16): a pure copy.
+// out[r] = hist row (idx[r], r % B), or zeros where idx[r] < 0; rows of `pieces` values of the
+// raw type E (16 bytes where the row length and the addresses allow, else 4 or 2). A warp takes
+// four rows at a time, so that its index loads and its row loads are in flight together: bound by
+// the bytes moved (195 x 1024 rows of 400 bytes, 160 MB: 23 us, 115 as one thread per 2-byte
+// value with a 64-bit division each; 256 x 256 rows of 2 KB: 32 us, 197).
 template <typename E>
-__global__ void gather_rows_kernel(const int32_t *__restrict__ idx, int B, size_t rows, int row_elems,
-                                   const E *__restrict__ hist, E *__restrict__ out)
+__global__ void __launch_bounds__(256) gather_rows_kernel(const int32_t *__restrict__ idx, int B, int rows, int pieces,
+                                                          const E *__restrict__ hist, E *__restrict__ out)
 {
-    const size_t total = rows * (size_t)row_elems;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
-         e += (size_t)gridDim.x * blockDim.x) {
-        const size_t r = e / row_elems;
-        const int k = (int)(e - r * row_elems);
-        const int src = idx[r];
-        const int b = (int)(r % B);
-        out[e] = src >= 0 ? hist[((size_t)src * B + b) * row_elems + k] : (E)0;
+    constexpr int N = 4;
+    const int lane = threadIdx.x & 31, warps = gridDim.x * (blockDim.x >> 5);
+    for (int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); (long long)g * N < rows; g += warps) {
+        const int r0 = g * N, r = min(r0 + (lane & (N - 1)), rows - 1);
+        const int s = idx[r];
+        const long long src = s >= 0 ? (long long)s * B + r % B : -1;
+        const E *from[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const long long q = __shfl_sync(0xffffffffu, src, i);
+            from[i] = q >= 0 ? hist + (size_t)q * pieces : nullptr;
+        }
+        for (int k = lane; k < pieces; k += 32) {
+            E v[N];
+#pragma unroll
+            for (int i = 0; i < N; ++i) v[i] = from[i] ? from[i][k] : E{};
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+                if (r0 + i < rows) out[(size_t)(r0 + i) * pieces + k] = v[i];
+        }
     }
 }
 
@@ -316,25 +331,85 @@ __global__ void seed_grads_kernel(int T, int B, int H, const int32_t *__restrict
     }
 }
 
-// The same seeding with per-step gradients dy, for one instance and 32 units per block:
-// the T + 1 rows' sums of those units accumulate in shared memory in the same order as
-// above (final top, then t = T-1..0), then every row is written once. The gradient
-// history is zero before the seeding, so writing the sums equals adding them.
+// The same seeding with per-step gradients dy, for one instance and 32 N units per block
+// (one warp, N units a lane): the sums of the T + 1 rows accumulate on chip in the same order
+// as above (final top, then t = T-1..0), the row that is on top in registers and the others in
+// shared memory, then every row is written once. The gradient history is zero before the
+// seeding, so writing the sums equals adding them. A warp's chain is one change of row a step
+// (a store and a load of shared memory); the loads run 24 to 32 steps ahead of it, by
+// asynchronous copies into a ring of which each lane reads back only its own (eight steps ahead
+// in registers left it waiting for memory: 64 x 200, 185 steps, 23 -> 18 us; 256 x 1024, 256 steps,
+// 281 -> 185 us). What is left is one warp's own instructions, about 190 cycles a step.
+constexpr int kSeedRing = 32, kSeedGroup = 8;  // steps in flight, steps a copy group
+template <int N>
 __global__ void __launch_bounds__(32) seed_grads_dy_kernel(int T, int B, int H, const int32_t *__restrict__ top,
                                                             const float *__restrict__ d_top_h,
                                                             const float *__restrict__ dy, float *__restrict__ dhist_h)
 {
-    extern __shared__ float acc[];  // [T + 1][32]
-    const int b = blockIdx.x, lane = threadIdx.x, j = blockIdx.y * 32 + lane;
-    for (int s = 0; s <= T; ++s) acc[s * 32 + lane] = 0.0f;
+    struct alignas(4 * N) Vec {
+        float f[N];
+    };
+    extern __shared__ __align__(16) uint8_t seed_smem[];
+    const int lane = threadIdx.x;
+    Vec *ring = (Vec *)seed_smem + lane;   // step i: ring[32 (i mod kSeedRing)]
+    Vec *slot = ring + 32 * kSeedRing;     // row s: slot[32 s]
+    const int b = blockIdx.x, j = (blockIdx.y * 32 + lane) * N;
+    const bool on = j < H;  // (H % N == 0: whole pieces)
+    const size_t step = (size_t)B * H, e = (size_t)b * H + (on ? j : 0);
+    auto fetch = [&](int i0) {  // steps T - 1 - i0 ..: one copy group
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(ring + 32 * (i0 % kSeedRing));
+#pragma unroll
+        for (int i = 0; i < kSeedGroup; ++i)
+            if (i0 + i < T)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst + i * 128 * N),
+                             "l"(dy + (size_t)(T - 1 - i0 - i) * step + e), "n"(4 * N)
+                             : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // lane l keeps the top after step T - 1 - (i0 + l), i0 a multiple of 32
+    auto tops = [&](int i0) { return top[(size_t)max(T - i0 - lane, 1) * B + b]; };
+    for (int i = 0; i < kSeedRing - kSeedGroup; i += kSeedGroup) fetch(i);
+    int s_cur = tops(0), s_nxt = T > 32 ? tops(32) : 0;
+    for (int i = lane; i < (T + 1) * 8 * N; i += 32) ((uint4 *)(slot - lane))[i] = make_uint4(0, 0, 0, 0);
     __syncwarp();
-    if (j < H) {
-        const size_t n = (size_t)B * H, e = (size_t)b * H + j;
-        if (d_top_h) acc[top[(size_t)T * B + b] * 32 + lane] += d_top_h[e];
-#pragma unroll 8
-        for (int t = T - 1; t >= 0; --t) acc[top[(size_t)(t + 1) * B + b] * 32 + lane] += dy[(size_t)t * n + e];
-        for (int s = 0; s <= T; ++s) dhist_h[((size_t)s * B + b) * H + j] = acc[s * 32 + lane];
+    int cur = top[(size_t)T * B + b];
+    Vec acc{};
+    if (d_top_h) {
+        const Vec d = *(const Vec *)(d_top_h + e);
+#pragma unroll
+        for (int i = 0; i < N; ++i) acc.f[i] += d.f[i];
     }
+    for (int i0 = 0; i0 < T; i0 += kSeedGroup) {
+        fetch(i0 + kSeedRing - kSeedGroup);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kSeedRing / kSeedGroup - 1) : "memory");
+        // the group's gradients and rows first: only the change of row stays on the chain
+        int s[kSeedGroup];
+        Vec g[kSeedGroup];
+#pragma unroll
+        for (int i = 0; i < kSeedGroup; ++i) {
+            s[i] = __shfl_sync(0xffffffffu, s_cur, (i0 + i) & 31);
+            g[i] = ring[32 * ((i0 + i) % kSeedRing)];
+        }
+#pragma unroll
+        for (int i = 0; i < kSeedGroup; ++i) {
+            if (i0 + i >= T) break;
+            if (s[i] != cur) {
+                slot[32 * cur] = acc;
+                acc = slot[32 * s[i]];
+                cur = s[i];
+            }
+#pragma unroll
+            for (int k = 0; k < N; ++k) acc.f[k] += g[i].f[k];
+        }
+        if ((i0 + kSeedGroup) % 32 == 0) {
+            s_cur = s_nxt;
+            if (i0 + kSeedGroup + 32 < T) s_nxt = tops(i0 + kSeedGroup + 32);
+        }
+    }
+    slot[32 * cur] = acc;
+    if (on)
+#pragma unroll 8
+        for (int r = 0; r <= T; ++r) *(Vec *)(dhist_h + (size_t)r * step + e) = slot[32 * r];
 }
 
 // Push-only mode: the virtual timeline of each instance. By Observation 2 of Sec. 3 only
@@ -542,15 +617,30 @@ cudaError_t launch_prepass(stacklstm *s, const int8_t *ops, int32_t *p_final)
 cudaError_t launch_gather_rows(stacklstm *s, const int32_t *idx, int rows, size_t elem_bytes,
                                const void *hist, void *out, int row_elems)
 {
-    const size_t total = (size_t)rows * row_elems;
-    const unsigned grid = (unsigned)std::min<size_t>(ceil_div(total, 256), (size_t)s->num_sms * 16);
-    if (total == 0) return cudaSuccess;
-    if (elem_bytes == 4)
-        gather_rows_kernel<uint32_t><<<grid, 256, 0, s->stream>>>(
-            idx, s->B, rows, row_elems, (const uint32_t *)hist, (uint32_t *)out);
+    if (rows == 0 || row_elems == 0) return cudaSuccess;
+    const unsigned grid = (unsigned)std::min<size_t>(ceil_div(rows, 32), (size_t)s->num_sms * 16);
+    // (hist is workspace and out 16-byte aligned: a row whose length is a multiple of 16 bytes is too)
+    const size_t row_bytes = (size_t)row_elems * elem_bytes;
+    if (row_bytes % 16 == 0)
+        gather_rows_kernel<uint4><<<grid, 256, 0, s->stream>>>(idx, s->B, rows, (int)(row_bytes / 16), (const uint4 *)hist,
+                                                               (uint4 *)out);
+    else if (elem_bytes == 4)
+        gather_rows_kernel<uint32_t><<<grid, 256, 0, s->stream>>>(idx, s->B, rows, row_elems, (const uint32_t *)hist,
+                                                                  (uint32_t *)out);
     else
-        gather_rows_kernel<uint16_t><<<grid, 256, 0, s->stream>>>(
-            idx, s->B, rows, row_elems, (const uint16_t *)hist, (uint16_t *)out);
+        gather_rows_kernel<uint16_t><<<grid, 256, 0, s->stream>>>(idx, s->B, rows, row_elems, (const uint16_t *)hist,
+                                                                  (uint16_t *)out);
+    s->launches += 1;
+    return cudaGetLastError();
+}
+
+template <int N>
+static cudaError_t seed_dy(stacklstm *s, size_t bytes, const int32_t *top, const float *d_top_h, const float *dy)
+{
+    const cudaError_t e = smem_at_least((const void *)seed_grads_dy_kernel<N>, bytes);
+    if (e) return e;
+    seed_grads_dy_kernel<N><<<dim3(s->B, ceil_div(s->H, 32 * N)), 32, bytes, s->stream>>>(s->T, s->B, s->H, top, d_top_h,
+                                                                                          dy, s->dhist_h);
     s->launches += 1;
     return cudaGetLastError();
 }
@@ -559,14 +649,12 @@ cudaError_t launch_seed_grads(stacklstm *s, const float *d_top_h, const float *d
 {
     if (!d_top_h && !dy) return cudaSuccess;
     const int32_t *top = s->push_only ? s->vy : s->top;
-    const size_t acc_bytes = (size_t)(s->T + 1) * 32 * sizeof(float);
+    // units a lane: as many as keep several warps' rows on an SM (and divide H)
+    const size_t acc_bytes = (size_t)(s->T + 1 + kSeedRing) * 32 * sizeof(float);
     if (dy && acc_bytes <= 200 * 1024) {
-        cudaError_t e = acc_bytes > 48 * 1024 ? smem_at_least((const void *)seed_grads_dy_kernel, acc_bytes) : cudaSuccess;
-        if (e) return e;
-        seed_grads_dy_kernel<<<dim3(s->B, ceil_div(s->H, 32)), 32, acc_bytes, s->stream>>>(s->T, s->B, s->H, top,
-                                                                                           d_top_h, dy, s->dhist_h);
-        s->launches += 1;
-        return cudaGetLastError();
+        if (s->H % 4 == 0 && 4 * acc_bytes <= 56 * 1024) return seed_dy<4>(s, 4 * acc_bytes, top, d_top_h, dy);
+        if (s->H % 2 == 0 && 2 * acc_bytes <= 72 * 1024) return seed_dy<2>(s, 2 * acc_bytes, top, d_top_h, dy);
+        return seed_dy<1>(s, acc_bytes, top, d_top_h, dy);
     }
     const size_t n = (size_t)s->B * s->H;
     const unsigned grid = (unsigned)std::min<size_t>(ceil_div(n, 256), (size_t)s->num_sms * 16);

@@ -52,7 +52,7 @@
  *                                  cluster kernels (fp32: instead of one CTA for all steps)
  *   STACKLSTM_FWD_CLUSTER=0        no thread-block-cluster forward
  *   STACKLSTM_BWD_CLUSTER=0        no thread-block-cluster backward
- *   STACKLSTM_ROW_CLUSTER=0        no clusters of eight rows (bf16_rows.cu): the 64-row ones
+ *   STACKLSTM_ROW_CLUSTER=0        no clusters of 8 or 16 rows (bf16_rows.cu)
  *   STACKLSTM_BWD_SPLIT=k          the persistent backward with its 4H contraction split
  *                                  over k CTAs per 64-unit column tile (k = 4)
  *   STACKLSTM_SPLIT_CLUSTER=0      the parts of a split contraction trade their partial

@@ -315,8 +315,9 @@ cudaError_t bf16_launch_fwd_persist(stacklstm *s, const StepArgs &a, const CUten
 cudaError_t bf16_launch_bwd_persist(stacklstm *s, const StepArgs &a, const CUtensorMap &tm_g, float *dx,
                                     bool *dx_done);
 
-// ---- thread-block clusters of few rows, H <= 256 (bf16_rows.cu)
-bool bf16_plan_rows(stacklstm *s, bool fwd, PersistPlan *pl);
+// ---- thread-block clusters of 8 or 16 rows, H <= 256 (bf16_rows.cu)
+// both directions (they share a gate layout) with n_tiles 8-row tiles a cluster: s->fr, s->br
+bool bf16_plan_rows(stacklstm *s, int n_tiles);
 // elements of their packed weights (pack_rows_*_elem), and the contraction steps they are built for
 size_t bf16_rows_wh_elems(int H);
 size_t bf16_rows_wx_elems(int I, int H);

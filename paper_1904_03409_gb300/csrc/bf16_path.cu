@@ -691,11 +691,10 @@ cudaError_t bf16_prepare(stacklstm *s)
             s->pf.on = 0;
         }
         bf16_plan_bwd_cluster(s, &s->bc);  // (the persistent plan stays as the fallback)
-        // few rows: clusters of 8 rows instead (both directions: they share a gate layout)
-        if (bf16_plan_rows(s, true, &s->fr) && bf16_plan_rows(s, false, &s->br))
+        // clusters of 8 rows instead where they all fit at once, or of 16 where the 64-row
+        // clusters do not (bf16_rows.cu has the figures)
+        if (bf16_plan_rows(s, 1) || (!(s->fc.on && s->bc.on) && bf16_plan_rows(s, 2)))
             s->fc.on = s->pf.on = s->bc.on = 0;
-        else
-            s->fr.on = s->br.on = 0;
         // small batches: both directions on CUDA cores instead
         if (bf16_plan_small(s, &s->cc)) {
             s->pf.on = s->pb.on = s->fc.on = s->bc.on = s->fr.on = s->br.on = 0;

@@ -1,8 +1,8 @@
 // bf16_rows.cu -- the recurrences of Algorithm 1 (forward) and of its reverse-time backward
-// (Sec. 5) for hidden widths up to 256 as thread-block clusters of eight rows.
+// (Sec. 5) for hidden widths up to 256 as thread-block clusters of 8 or 16 rows.
 //
-// Instances are independent, so a batch is cut into groups of 8 rows and each group runs
-// all T steps in one cluster of its own; a CTA holds 32 hidden units, so a cluster has
+// Instances are independent, so a batch is cut into groups of 8 (or, NT = 2, 16) rows and each
+// group runs all T steps in one cluster of its own; a CTA holds 32 hidden units, so a cluster has
 // ceil(H / 32) <= 8 CTAs. A step is a chain of one contraction, the cell and an exchange
 // between the cluster's CTAs, and with so few rows latency bounds it, not arithmetic or
 // bandwidth: the gate contraction is 128 gate columns x 8 rows x (I + H) a CTA. It therefore
@@ -11,8 +11,8 @@
 // cell's registers as soon as the last MMA is done. The 64-row tcgen05 clusters
 // (bf16_cluster.cu) spend 1.54 us a step forward and 2.07 us backward on commits, barriers,
 // tensor-memory loads and on bringing 64 rows to every CTA (I = H = 200, B = 64); here it is
-// 1.00 and 1.06 us (clock stamps: about 400 cycles of MMAs, 16 cycles each, 300 of cell,
-// 700 until every CTA's piece has landed). A 64 x 200 pass: 0.777 -> 0.576 ms.
+// 0.96 and 1.03 us (clock stamps: about 400 cycles of ldmatrix and MMAs, 300 of cell,
+// 700 until every CTA's piece has landed). A 64 x 200 pass: 0.777 -> 0.53 ms.
 //
 // Forward. Warp w of CTA ct owns units 32 ct + 8 w .. + 7: M tile 0 is their gates i and f,
 // M tile 1 gates g and o, so lane (g, t) = (lane / 4, lane % 4) holds all four gates of unit
@@ -43,7 +43,6 @@ namespace {
 
 using tc::smem_u32;
 
-constexpr int NT = 1, NR = 8 * NT;  // 8-row N tiles (rows) of a cluster; two a cluster spilled and took twice as long
 constexpr int kRcThreads = 256;  // warps 0..3: the step; 4..7: forward the x part, backward half the MMAs and dG
 constexpr int kRcX = 4;          // x_t buffers (steps in flight)
 constexpr int kRcDgLd = 136;     // row of the backward's own gate gradients: 128 + 8 (odd 16-byte pieces)
@@ -179,20 +178,22 @@ __device__ __forceinline__ const RcArgs &rc_member(const RcGroup &G, int cid, in
 }
 
 // ------------------------------------------------------------------------ forward
-// Shared memory: [W_x 128 rows][x buffers kRcX x 8 rows][h operand 2 x 8 rows]
-// [x part 4 warps x 2 x 2 fragments][barriers]; rows of 16 KX + 8 (16 KH + 8) values, an
+// Shared memory: [W_x 128 rows][x buffers kRcX x 8 NT rows][h operand 2 x 8 NT rows]
+// [x part 4 warps x 2 x 2 NT fragments][barriers]; rows of 16 KX + 8 (16 KH + 8) values, an
 // odd number of 16-byte pieces (conflict-free ldmatrix).
-__host__ __device__ constexpr uint32_t rc_fwd_smem(int KX, int KH)
+__host__ __device__ constexpr uint32_t rc_fwd_smem(int KX, int KH, int NT)
 {
     return (128u + kRcX * 8u * NT) * (KX * 16 + 8) * 2 + 2u * 8 * NT * (KH * 16 + 8) * 2 + 4u * 2 * 2 * NT * 512 + 256;
 }
 
 // registers a thread after the split of the block's 256 x 128 between its two warpgroups
-constexpr int kRcRegsStep = 200, kRcRegsX = 56;
+constexpr int kRcRegsStep = 200, kRcRegsX = 56;    // forward
+constexpr int kRcRegsBwd = 160, kRcRegsBwd2 = 96;  // backward, two N tiles
 
-template <int KH>
+template <int KH, int NT>
 __global__ void __launch_bounds__(kRcThreads, 2) step_rows(const __grid_constant__ RcGroup G)
 {
+    constexpr int NR = 8 * NT;
     constexpr uint32_t SH = (KH * 16 + 8) * 2, hb_bytes = NR * SH;  // an h operand row, a buffer
     constexpr uint32_t xf_bytes = 2 * NT * 512;                     // x part of a warp and step
     extern __shared__ __align__(128) uint8_t smem[];
@@ -245,7 +246,7 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rows(const __grid_constant
     if (warp >= 4) {
         // ---------------------------------------------- the x part: bias + x_t W_x, steps ahead
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRcRegsX));
-        // 16 threads a row; row r's pieces tl, tl + 16, ...
+        // 16 / NT threads a row; row r's pieces tl, tl + 16 / NT, ...
         const int xr = (tid & 127) / (16 / NT), tl = (tid & 127) % (16 / NT);
         const __nv_bfloat16 *xp = p.x + ((size_t)row0 + xr) * I;
         auto load_x = [&](int t) {
@@ -378,7 +379,8 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rows(const __grid_constant
                 if (!rc_wait<true>(bar(b), (uint32_t)((t - 1) >> 1) & 1, limit, abort, a.err)) break;
                 if (tid == 0 && t + 2 < T) tc::mbar_arrive_expect_tx(&bars[b], h_bytes);
             }
-            // two accumulators a tile halve the chain of dependent MMAs
+            // with one N tile, two accumulators an M tile halve the chain of dependent MMAs
+            constexpr bool kTwo = NT == 1;
             float acc2[2][NT][4];
 #pragma unroll
             for (int i = 0; i < 2; ++i)
@@ -399,7 +401,7 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rows(const __grid_constant
                     for (int i = 0; i < 2; ++i) mma16816(acc[i][n], wh[i][k], bb[0], bb[1]);
                     if (k + 1 < KH) {
 #pragma unroll
-                        for (int i = 0; i < 2; ++i) mma16816(acc2[i][n], wh[i][k + 1], bb[2], bb[3]);
+                        for (int i = 0; i < 2; ++i) mma16816(kTwo ? acc2[i][n] : acc[i][n], wh[i][k + 1], bb[2], bb[3]);
                     }
                 }
             // the cell; the operand goes out first
@@ -411,8 +413,8 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rows(const __grid_constant
                 float hn[2];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    const float ig = sigm(acc[0][n][e] + acc2[0][n][e]), fg = sigm(acc[0][n][2 + e] + acc2[0][n][2 + e]);
-                    const float gg = tanh_hw(acc[1][n][e] + acc2[1][n][e]), og = sigm(acc[1][n][2 + e] + acc2[1][n][2 + e]);
+                    auto z = [&](int i, int q) { return kTwo ? acc[i][n][q] + acc2[i][n][q] : acc[i][n][q]; };
+                    const float ig = sigm(z(0, e)), fg = sigm(z(0, 2 + e)), gg = tanh_hw(z(1, e)), og = sigm(z(1, 2 + e));
                     cn[n][e] = fmaf(fg, cr[n][e], ig * gg);
                     hn[e] = og * tanh_hw(cn[n][e]);
                     gt[n][e][0] = pack2_f16(ig, fg);
@@ -457,17 +459,17 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rows(const __grid_constant
 }
 
 // ----------------------------------------------------------------------- backward
-// Shared memory: [partial sums 2 x C parts x 2 M tiles x 32 lanes x 16 bytes]
-// [own gate gradients 2 x 8 rows][barriers]
-__host__ __device__ constexpr uint32_t rc_bwd_smem(int C)
+// Shared memory: [partial sums 2 x C parts x 2 M tiles x NT x 32 lanes x 16 bytes]
+// [own gate gradients 2 x 8 NT rows][barriers]
+__host__ __device__ constexpr uint32_t rc_bwd_smem(int C, int NT)
 {
     return 2u * C * 2 * NT * 512 + 2u * 8 * NT * kRcDgLd * 2 + 64;
 }
 
-template <int KT>
+template <int KT, int NT>
 __global__ void __launch_bounds__(kRcThreads, 2) step_rowsb(const __grid_constant__ RcGroup G)
 {
-    constexpr int MT = (KT + 7) / 8;  // M tiles a warp: 16-unit tiles warp, warp + 8
+    constexpr int NR = 8 * NT, MT = (KT + 7) / 8;  // M tiles a warp: 16-unit tiles warp, warp + 8
     constexpr uint32_t slot = NT * 512, dgb = NR * kRcDgLd * 2;
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ int s_abort;
@@ -495,10 +497,12 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rowsb(const __grid_constan
     }
     // this CTA's gate columns of W_h for the warp's M tiles, for the whole launch
     uint4 wt[MT][8];
+    auto load_weights = [&]() {
 #pragma unroll
-    for (int i = 0; i < MT; ++i)
+        for (int i = 0; i < MT; ++i)
 #pragma unroll
-        for (int k = 0; k < 8; ++k) wt[i][k] = __ldcg(p.wfrag + ((((size_t)ct * 8 + warp) * MT + i) * 8 + k) * 32 + lane);
+            for (int k = 0; k < 8; ++k) wt[i][k] = __ldcg(p.wfrag + ((((size_t)ct * 8 + warp) * MT + i) * 8 + k) * 32 + lane);
+    };
     // M tile j = 8 i + warp: units 16 j .. + 15, which CTA j / 2 owns
     uint32_t peer[MT];
 #pragma unroll
@@ -542,7 +546,9 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rowsb(const __grid_constan
     if (warp >= 4) {
         // ---------- half of the M tiles, and dG in the [T B][4H] layout (for dx and dW): thread
         // (row, 8 units, gate), the eight units' values gathered from the operand rows
+        if constexpr (NT > 1) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRcRegsBwd2));
         const int j = tid & 127;
+        load_weights();
         for (int t = T - 1; t >= 0; --t) {
             const int b = t & 1;
             if (__syncthreads_or(0)) break;
@@ -561,6 +567,8 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rowsb(const __grid_constan
             }
         }
     } else {
+        if constexpr (NT > 1) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRcRegsBwd));
+        load_weights();
         const int u0 = (int)ct * 32 + warp * 8, u = u0 + g;
         const bool warp_on = u0 < H;
         const int uc = warp_on ? u : 0;  // (lanes past H compute on unit 0's data and write nothing)
@@ -689,13 +697,19 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rowsb(const __grid_constan
 // contraction steps of 16 the kernels are built for: the least that covers H
 int rc_k(int H) { return H <= 64 ? 4 : H <= 128 ? 8 : H <= 208 ? 13 : 16; }
 
-const void *rc_fn(bool fwd, int H)
+template <int K>
+const void *rc_fn_k(bool fwd, int NT)
+{
+    if (fwd) return NT == 1 ? (const void *)step_rows<K, 1> : (const void *)step_rows<K, 2>;
+    return NT == 1 ? (const void *)step_rowsb<K, 1> : (const void *)step_rowsb<K, 2>;
+}
+const void *rc_fn(bool fwd, int H, int NT)
 {
     switch (rc_k(H)) {
-    case 4: return fwd ? (const void *)step_rows<4> : (const void *)step_rowsb<4>;
-    case 8: return fwd ? (const void *)step_rows<8> : (const void *)step_rowsb<8>;
-    case 13: return fwd ? (const void *)step_rows<13> : (const void *)step_rowsb<13>;
-    default: return fwd ? (const void *)step_rows<16> : (const void *)step_rowsb<16>;
+    case 4: return rc_fn_k<4>(fwd, NT);
+    case 8: return rc_fn_k<8>(fwd, NT);
+    case 13: return rc_fn_k<13>(fwd, NT);
+    default: return rc_fn_k<16>(fwd, NT);
     }
 }
 
@@ -714,11 +728,13 @@ void rc_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, int clusters, i
     cfg->numAttrs = 1;
 }
 
-// One direction: every cluster co-resident (two CTAs an SM), or the plan is off. At 64 x 200
-// that is 36 clusters (288 rows): 1.00 / 1.06 us a step up to 14 clusters (one CTA an SM), 1.50 /
-// 1.54 beyond, against 1.54..1.6 / 2.1..2.4 of the 64-row clusters, which take over past it
-// (a second round of clusters would double the time).
-bool rc_plan(stacklstm *s, bool fwd, PersistPlan *pl)
+// One direction with NT 8-row N tiles a cluster: every cluster co-resident (two CTAs an SM),
+// or the plan is off: a second round of clusters would double the time. At H = 200 that is 36
+// clusters: NT = 1, 288 rows, 0.96 / 1.03 us a step up to 14 clusters (one CTA an SM) and 1.50 /
+// 1.50 beyond, against 1.6 / 2.3 of the 64-row clusters; NT = 2, 576 rows at 2.66 / 2.51, against
+// 4.02 / 6.05 of the persistent kernels (the 64-row clusters reach 448 rows; at 1024, two rounds
+// of NT = 2 take 5.15 / 4.97, the persistent kernels 4.55 / 6.14).
+bool rc_plan(stacklstm *s, bool fwd, int NT, PersistPlan *pl)
 {
     pl->on = 0;
     // test hooks (include/stacklstm.h)
@@ -728,9 +744,10 @@ bool rc_plan(stacklstm *s, bool fwd, PersistPlan *pl)
     if (rows && atoi(rows) == 0) return false;
     const int C = (int)ceil_div(s->H, 32), KX = (int)ceil_div(s->I, 16);
     if (C > 8) return false;
-    const uint32_t smem = fwd ? rc_fwd_smem(KX, rc_k(s->H)) : rc_bwd_smem(C);
+    const int NR = 8 * NT;
+    const uint32_t smem = fwd ? rc_fwd_smem(KX, rc_k(s->H), NT) : rc_bwd_smem(C, NT);
     if (smem > kSmemCap) return false;
-    const void *fn = rc_fn(fwd, s->H);
+    const void *fn = rc_fn(fwd, s->H, NT);
     cudaFuncAttributes fa;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
@@ -738,7 +755,7 @@ bool rc_plan(stacklstm *s, bool fwd, PersistPlan *pl)
     int clusters = 0;
     // (the forward's split of the registers draws on what the block is launched with)
     if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess ||
-        (fwd && fa.numRegs * kRcThreads < (kRcRegsStep + kRcRegsX) * (kRcThreads / 2)) ||
+        ((fwd || NT > 1) && fa.numRegs * kRcThreads < (kRcRegsStep + kRcRegsX) * (kRcThreads / 2)) ||
         smem_at_least(fn, smem) != cudaSuccess || cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return false;
@@ -785,7 +802,7 @@ cudaError_t rc_launch(stacklstm *const *hs, const StepArgs *as, const float *con
         G.first[m + 1] = G.first[m] + (int)ceil_div(hs[m]->B, pl.rows);
         smem = std::max(smem, (uint32_t)pl.smem);
     }
-    const void *fn = rc_fn(fwd, hs[0]->H);
+    const void *fn = rc_fn(fwd, hs[0]->H, p0.rows / 8);
     cudaError_t e = smem_at_least(fn, smem);
     if (e) return e;
     cudaLaunchConfig_t cfg;
@@ -799,7 +816,12 @@ cudaError_t rc_launch(stacklstm *const *hs, const StepArgs *as, const float *con
 
 }  // namespace
 
-bool bf16_plan_rows(stacklstm *s, bool fwd, PersistPlan *pl) { return rc_plan(s, fwd, pl); }
+bool bf16_plan_rows(stacklstm *s, int n_tiles)
+{
+    if (rc_plan(s, true, n_tiles, &s->fr) && rc_plan(s, false, n_tiles, &s->br)) return true;
+    s->fr.on = s->br.on = 0;
+    return false;
+}
 
 size_t bf16_rows_wh_elems(int H) { return ceil_div(H, 32) * (size_t)4 * 2 * rc_k(H) * 256; }
 size_t bf16_rows_wx_elems(int I, int H) { return ceil_div(H, 32) * (size_t)128 * (ceil_div(I, 16) * 16 + 8); }

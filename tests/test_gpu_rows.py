@@ -1,9 +1,10 @@
-"""GPU parity of the clusters of eight rows (bf16_rows.cu) against the fp64 oracle.
+"""GPU parity of the clusters of 8 and 16 rows (bf16_rows.cu) against the fp64 oracle.
 
 The shapes sit at the edges of their tiles: hidden widths that fill a warp's 8 units, a
 CTA's 32 or an M tile's 16 exactly or partly, each contraction depth they are built for,
 batches that leave rows of a group empty, one to three steps (fewer than the buffers in
-flight), inputs wider than W_x's tiles, enough groups for two CTAs an SM. Outputs are
+flight), inputs wider than W_x's tiles, enough groups for two CTAs an SM, and more rows than
+8-row groups fit. Outputs are
 NaN-filled first; the 64-row clusters they replace run beside them.
 """
 import os
@@ -30,11 +31,12 @@ def plan_of(w):
 @pytest.mark.parametrize("T,B,I,H,seed", [
     (1, 2, 8, 8, 71), (2, 9, 8, 32, 72), (3, 8, 24, 64, 73), (5, 17, 208, 72, 74), (6, 5, 40, 128, 75),
     (50, 1, 40, 200, 76), (7, 12, 16, 208, 77), (4, 3, 72, 216, 78), (9, 10, 256, 256, 79), (6, 20, 520, 104, 80),
-    (4, 250, 16, 200, 81)])
+    (4, 250, 16, 200, 81), (4, 500, 16, 200, 83), (3, 573, 200, 176, 84), (2, 561, 24, 136, 85)])
 def test_row_clusters_match_oracle(T, B, I, H, seed):
     w = wl.make_workload("case", T=T, B=B, I=I, H=H, dtype="bf16", seed=seed, ops_kind="random_walk",
                          probs=(0.5, 0.3, 0.2), bias_scale=0.3, h0_scale=0.5, c0_scale=0.5, dy_scale=0.5)
-    assert plan_of(w).count("rows 8") == 2, plan_of(w)
+    rows = "rows 16" if B > 288 else "rows 8"
+    assert plan_of(w).count(rows) == 2, plan_of(w)
     args = (w.x, w.ops, w.h0, w.c0, w.W, w.bias)
     ref = oracle.run(*args, d_top_h=w.d_top_h, dy=w.dy)
     got = runner.run(w)
@@ -46,7 +48,7 @@ def test_row_clusters_match_oracle(T, B, I, H, seed):
             oracle.run(*args, d_top_h=w.d_top_h, dy=w.dy, mode="definition"), "bf16")
     os.environ["STACKLSTM_ROW_CLUSTER"] = "0"
     try:
-        assert "rows 8" not in plan_of(w)
+        assert rows not in plan_of(w)
         compare(runner.run(w), ref, "bf16")
     finally:
         del os.environ["STACKLSTM_ROW_CLUSTER"]

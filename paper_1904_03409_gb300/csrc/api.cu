@@ -153,6 +153,8 @@ sl_status fwd_begin(stacklstm *s, const sl_forward_args &a)
         if (p && !aligned16(p)) return fail(s, SL_ERR_ARG, "tensor pointers must be 16-byte aligned");
     cudaError_t e;
     s->fwd_done = 0;
+    // the row clusters hold each step's output already: it is the next step's h operand
+    s->y_direct = (s->fr.on || s->fr32.on) && !s->push_only ? a.y : nullptr;
     // the initial state and the weight packing do not depend on the index prepass, so they
     // run on the side stream at the same time (launched after the prepass, whose few blocks
     // then reach the SMs first); the caller's stream waits for them before the forward steps
@@ -243,7 +245,7 @@ sl_status fwd_end(stacklstm *s, const sl_forward_args &a)
         // history index of the top after each step and of each slot's last write (in
         // push-only mode: virtual indices, and each slot's last push, as in Sec. 2)
         const int32_t *ytop = s->push_only ? s->vy : s->top, *slots = s->push_only ? s->vslot : s->slot_last;
-        if (a.y && (e = sl::launch_gather_rows(s, ytop + B, T * B, es, s->hist_h, a.y, H)))
+        if (a.y && !s->y_direct && (e = sl::launch_gather_rows(s, ytop + B, T * B, es, s->hist_h, a.y, H)))
             return cuda_fail(s, e, "y");
         if (a.h_stack && (e = sl::launch_gather_rows(s, slots, (T + 1) * B, es, s->hist_h, a.h_stack, H)))
             return cuda_fail(s, e, "h_stack");

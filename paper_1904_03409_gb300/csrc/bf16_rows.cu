@@ -53,6 +53,7 @@ struct RcArgs {
     const uint4 *wfrag;        // W_h fragments (pack_rows_wh_elem / pack_rows_wb_elem)
     const uint8_t *wx;         // forward: W_x rows as they lie in shared memory (pack_rows_wx_elem)
     const __nv_bfloat16 *x;    // forward: [T][B][I]
+    __nv_bfloat16 *y;          // forward: [T][B][H] step outputs, or null
     const float *d_top;        // backward: the final top's gradient, still to be added (or null)
     const int32_t *ftop;       // backward: the final top's history row of each instance
     int KX;                    // forward: x contraction steps of 16
@@ -340,6 +341,12 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rows(const __grid_constant
         const uint32_t peer0 = tc::mapa(s_wx, t4 < C ? t4 : 0), peer1 = tc::mapa(s_wx, t4 + 4 < C ? t4 + 4 : 0);
         const bool send0 = t4 < C, send1 = t4 + 4 < C;
         const uint32_t h_off = s_h - s_wx, bar_off = s_bar - s_wx;
+        // where this lane's piece of a row goes: history row t + 1, the h operand row t + 1 (for
+        // the weight gradient), y_t (a step's output is its top's h, the operand of the next step)
+        __nv_bfloat16 *const st_base = t4 == 0 ? at_row(a.hist_h, 1, sh) : t4 == 1 ? at_row(a.hr, 1, sh) : p.y;
+        bool st_on[NT];
+#pragma unroll
+        for (int n = 0; n < NT; ++n) st_on[n] = okg[n] && t4 < (p.y ? 3 : 2);
         const uint32_t ha0 = s_h + (lane & 7) * SH + (lane >> 3) * 16;
         const uint32_t ha2 = s_h + (lane & 7) * SH + ((lane >> 3) & 1) * 16;  // an odd last K step
         for (int t = 0; t < (warp_on ? T : 0); ++t) {
@@ -433,11 +440,10 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rows(const __grid_constant
             // while the operands travel, and not against this warp's MMAs
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&bars[11 + 2 * w4 + b]);
-            // history row t + 1, the h operand row t + 1 (for the weight gradient), the gates
+            // the row pieces, c, the gates
 #pragma unroll
             for (int n = 0; n < NT; ++n) {
-                if (okg[n] && t4 < 2)
-                    *(uint4 *)(at_row(t4 == 0 ? a.hist_h : a.hr, t + 1, sh) + (size_t)rg[n] * H + u0) = t4 == 0 ? hrow[n] : op[n];
+                if (st_on[n]) *(uint4 *)(at_row(st_base, t, sh) + (size_t)rg[n] * H + u0) = t4 == 0 ? hrow[n] : op[n];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                     if (okc[n][e]) {
@@ -781,6 +787,7 @@ RcArgs rc_args(stacklstm *s, const StepArgs &a, bool fwd, const float *d_top)
     p.wfrag = (const uint4 *)(fwd ? s->w_rh : s->w_rb);
     p.wx = (const uint8_t *)s->w_rx;
     p.x = (const __nv_bfloat16 *)s->x_saved;
+    p.y = (__nv_bfloat16 *)s->y_direct;
     p.d_top = d_top;
     p.ftop = (s->push_only ? s->vy : s->top) + (size_t)s->T * s->B;
     p.KX = (int)ceil_div(s->I, 16);

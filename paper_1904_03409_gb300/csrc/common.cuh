@@ -115,6 +115,7 @@ struct stacklstm {
     PersistPlan bc;                // backward as one thread-block cluster (one row tile; bf16_cluster.cu)
     PersistPlan fr, br;            // forward, backward as clusters of few rows (bf16_rows.cu)
     void *w_rh = nullptr, *w_rx = nullptr, *w_rb = nullptr;  // their weights: forward W_h, W_x; backward W_h
+    void *y_direct = nullptr;  // y, when this forward's step kernel writes it (row clusters, homogenized mode)
     const float *d_top_seed = nullptr;  // backward: the final tops' gradient the row clusters add themselves
     PersistPlan cc;                // small batches: both directions on CUDA cores (bf16_small.cu)
     void *w_ccf = nullptr, *w_ccb = nullptr;  // their weight slices

@@ -35,6 +35,7 @@ struct FrArgs {
     float *hist_h, *hist_c; // [T + 1][B][H]
     float *gates;           // [T][B][4H]: forward, in: x W_x + bias, out: the activated gates
     float *hr;              // [T][B][H]: the state each step read (for dW)
+    float *y;               // [T][B][H] step outputs, or null
     const float *wh;        // forward: W + I * 4H ([H][4H]); backward: W_h^T ([4H] rows, ldw apart)
     size_t ldw;
     float *dhist_h, *dhist_c, *dG;
@@ -243,6 +244,7 @@ __global__ void __launch_bounds__(kFrThreads, 1) fwd_rows_f32(FrArgs a)
             a.hist_h[(size_t)(t + 1) * SB + cell] = hn;
             a.hist_c[(size_t)(t + 1) * SB + cell] = cn;
             if (t + 1 < T) a.hr[(size_t)(t + 1) * SB + cell] = op;
+            if (a.y) a.y[(size_t)t * SB + cell] = op;
             float *gp = a.gates + ((size_t)t * B + row) * G + u;
             gp[0] = ig;
             gp[H] = fg;
@@ -727,7 +729,7 @@ static cudaError_t fr_launch(stacklstm *s, bool fwd, FrArgs &a)
     a.C = s->fr32.cl; a.W = s->fr32.EP;
     a.top = s->top;
     a.hist_h = (float *)s->hist_h; a.hist_c = s->hist_c;
-    a.gates = (float *)s->gates; a.hr = (float *)s->a_rm;
+    a.gates = (float *)s->gates; a.hr = (float *)s->a_rm; a.y = (float *)s->y_direct;
     a.dhist_h = s->dhist_h; a.dhist_c = s->dhist_c; a.dG = (float *)s->dG;
     a.limit = fwd ? s->wait_limit : s->wait_limit_bwd;
     a.err = s->err;

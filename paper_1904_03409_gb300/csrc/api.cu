@@ -421,7 +421,7 @@ sl_status stacklstm_create(stacklstm_t *out, int T, int B, int I, int H, sl_dtyp
               alloc(s, &s->gates, dtype == SL_BF16 ? TB * 4 * (((size_t)H + 15) / 16 * 16) * 2 : TB * G * 4) && alloc(s, &s->a_rm, dtype == SL_FP32 ? TB * K * es : 16) &&
               alloc(s, &s->dhist_h, T1B * H * 4) && alloc(s, &s->dhist_c, T1B * H * 4) &&
               alloc(s, &s->dG, TB * G * es);
-    if (ok && dtype == SL_FP32) ok = alloc(s, &s->w_fwd, K * G * 4);
+    if (ok && dtype == SL_FP32) ok = alloc(s, &s->w_fwd, (K + 3) / 4 * 4 * G * 4);
     if (ok && dtype == SL_BF16) ok = sl::bf16_prepare(s) == cudaSuccess;
     if (ok) ok = sl::configure_prepass(s) == cudaSuccess;
     if (ok && !s->prepass_smem) ok = alloc(s, &s->slot_scratch, T1B * 4);

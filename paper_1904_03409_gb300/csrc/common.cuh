@@ -96,7 +96,7 @@ struct stacklstm {
     void *dG = nullptr;        // [T][B][4H] gate pre-activation gradients (fp32 / bf16)
 
     // packed weights (taken at forward)
-    void *w_fwd = nullptr;  // fp32: W^T [4H][I+H] float; bf16: forward operand tiles
+    void *w_fwd = nullptr;  // fp32: W^T [4H] rows of I+H floats; bf16: forward operand tiles
     void *w_bwd = nullptr;  // bf16: backward operand tiles
     void *w_dx = nullptr;   // bf16: input-gradient operand tiles
     float *dw_part = nullptr;  // split-K partials of the weight-gradient contraction
@@ -179,6 +179,8 @@ cudaError_t fp32_backward_steps(stacklstm *s);
 cudaError_t fp32_dx(stacklstm *s, float *dx);
 cudaError_t fp32_dw(stacklstm *s, float *dW, float *dbias);
 // clusters of few rows and tiled contractions, H <= 256 (fp32_rows.cu)
+// floats between the rows of W^T for the row clusters: a multiple of 16 bytes
+inline size_t ldw_f32(const stacklstm *s) { return ((size_t)s->I + s->H + 3) / 4 * 4; }
 bool fp32_plan_rows(stacklstm *s);
 cudaError_t fp32_rows_forward(stacklstm *s, const float *x, const float *W, const float *bias);
 cudaError_t fp32_rows_backward(stacklstm *s);

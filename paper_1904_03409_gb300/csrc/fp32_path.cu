@@ -67,11 +67,12 @@ __global__ void fwd_step_f32(int t, int B, int I, int H, const float *__restrict
 }
 
 // The forward setup in one launch: history row 0 = (h0, c0), the initial state (stack
-// slot 0), and W^T (out[c][r] = in[r][c], R x C) for the backward contractions, so that the
+// slot 0), and W^T (out[c][r] = in[r][c], R x C, out's rows ldo
+// apart) for the backward contractions, so that the
 // backward needs nothing the caller owns.
 __global__ void setup_f32(int n0, const float *__restrict__ h0, const float *__restrict__ c0,
                           float *__restrict__ hist_h, float *__restrict__ hist_c, int R, int C,
-                          const float *__restrict__ in, float *__restrict__ out)
+                          const float *__restrict__ in, float *__restrict__ out, size_t ldo)
 {
     const size_t n = (size_t)R * C, stride = (size_t)gridDim.x * blockDim.x;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n + n0; e += stride) {
@@ -80,7 +81,7 @@ __global__ void setup_f32(int n0, const float *__restrict__ h0, const float *__r
             hist_c[e] = c0[e];
         } else {
             const size_t f = e - n0, r = f / C, c = f - r * C;
-            out[c * R + r] = in[f];
+            out[c * ldo + r] = in[f];
         }
     }
 }
@@ -399,7 +400,7 @@ cudaError_t fp32_forward_setup(stacklstm *s, const float *h0, const float *c0, c
 {
     const int B = s->B, I = s->I, H = s->H, K = I + H, G = 4 * H;
     setup_f32<<<grid_for(s, (size_t)K * G + (size_t)B * H, 256), 256, 0, s->stream>>>(
-        B * H, h0, c0, (float *)s->hist_h, s->hist_c, K, G, W, (float *)s->w_fwd);
+        B * H, h0, c0, (float *)s->hist_h, s->hist_c, K, G, W, (float *)s->w_fwd, s->fr32.on ? ldw_f32(s) : K);
     s->launches += 1;
     return cudaGetLastError();
 }

@@ -9,8 +9,8 @@
 // step is bound by what its warps issue, two a scheduler (at 64 x 200, 13 clusters of 7 CTAs
 // and 5 rows: 280 two-wide multiply-adds and about 300 other instructions a warp), and by the
 // exchange between the CTAs: 1.62 us forward, 1.73 backward, where a launch a step, each dot
-// product reading its weights from L2 again, took 36 and 36. With the tiled contractions
-// (about 27 TFLOP/s, 64 x 128 tiles) a 64 x 200 pass of 185 steps went from 20.0 to 1.19 ms.
+// product reading its weights from L2 again, took 36 and 36. A 64 x 200 pass of 185 steps went
+// from 20.0 ms to 1.05.
 #include <stdlib.h>
 
 #include <algorithm>
@@ -433,76 +433,89 @@ __global__ void __launch_bounds__(kFrThreads, 1) bwd_rows_f32(FrArgs a)
 }
 
 // ------------------------------------------------------------- tiled contractions
-// C[M][N] = A B (+ bias[N]) in fp32, tiles of TM * 16 x TN * 16 outputs by 256 threads of
-// TM x TN each; partial sums over every 32 terms are added to a second accumulator, which
-// keeps a long sum's error near that of its short pieces. Row tiles past M's take the M2 rows
-// of A2 instead (dW: x, then the states read). kAT: A is given transposed
-// ([K][M], rows lda apart: dW = A^T dG); else [M][K]. grid z splits K evenly; slab z of C.
-template <int TM, int TN, bool kAT>
-__global__ void __launch_bounds__(256) gemm_f32(int M, int N, int K, const float *__restrict__ A, size_t lda,
-                                                int M2, const float *__restrict__ A2, size_t lda2,
-                                                const float *__restrict__ Bm, size_t ldb, const float *__restrict__ bias,
-                                                float *__restrict__ Cm, size_t ldc, size_t slab)
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float *src, uint32_t src_bytes)
 {
-    constexpr int BM = 16 * TM, BN = 16 * TN, BK = 16, LA = BM * BK / 256, LB = BN * BK / 256;
-    __shared__ __align__(16) float sa[2][BK][BM + 4], sb[2][BK][BN + 4];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int n0 = blockIdx.y * BN, tiles1 = (M + BM - 1) / BM;
-    int m0 = blockIdx.x * BM;
-    if ((int)blockIdx.x >= tiles1) {  // the rows of the second operand, below the first's in C
-        m0 -= tiles1 * BM;
-        Cm += (size_t)M * ldc;
-        M = M2;
-        A = A2;
-        lda = lda2;
-    }
-    const int KS = (K + BK - 1) / BK, z = blockIdx.z, nz = gridDim.z;
-    const int k_lo = (int)((long long)KS * z / nz) * BK, k_hi = min(K, (int)((long long)KS * (z + 1) / nz) * BK);
-    // this thread's elements of a block: A (m, k), then every SA along M (along K: kAT), B (k, n),
-    // then every 256 / BN along K
-    constexpr int SA = kAT ? 256 / BM : 256 / BK, SB = 256 / BN;
-    const int am = kAT ? tid % BM : tid / BK, ak = kAT ? tid / BM : tid % BK, bn = tid % BN, bk = tid / BN;
-    const float *pa = A + (kAT ? (size_t)(k_lo + ak) * lda + m0 + am : (size_t)(m0 + am) * lda + k_lo + ak);
-    const float *pb = Bm + (size_t)(k_lo + bk) * ldb + n0 + bn;
-    const size_t sa_i = (size_t)SA * lda, sb_i = (size_t)SB * ldb, sa_k = kAT ? (size_t)BK * lda : BK, sb_k = (size_t)BK * ldb;
-    const bool inner = m0 + BM <= M && n0 + BN <= N;
-    float ra[LA], rb[LB];
-    auto fetch = [&](int k0) {  // the block at k0; the pointers move on to the next
-        if (inner && k0 + BK <= k_hi) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
+
+struct GemmF32 {
+    int M, N, K;
+    const float *A;      // [M][K] rows lda apart; kAT: its transpose, [K][M1] rows lda apart,
+    const float *A2;     // and [K][M2 - M1] rows lda2 apart, the rows of A from M1; ones from M2
+    int M1, M2;
+    size_t lda, lda2;
+    const float *B;      // [K][N] rows ldb apart, a multiple of 4, of at least N rounded up to 4
+    size_t ldb;
+    const float *bias;   // [N] or null
+    float *C;            // [M][N] rows ldc apart; slab z of it
+    size_t ldc, slab;
+};
+
+__device__ const float kOnes[4] = {1.0f, 1.0f, 1.0f, 1.0f};
+
+// C = A B (+ bias) in fp32: WM x WN warps of 4 TM x 64 outputs, TM x 8 of them a thread. Blocks
+// of 16 terms arrive in a ring of asynchronous copies (of EA = 4 elements where A's rows are
+// aligned to that, else of one). Partial sums over every 32 terms are added to a second
+// accumulator, which keeps a long sum's error near that of its short pieces. grid z splits K
+// evenly. Bound by the multiply-add units, which are busy 64% of the time (8 x 8 outputs a
+// thread, two warps a scheduler; the pairs' duplicated operand costs a move each): 11840 x 800
+// outputs of 200 terms 90 us, 42 TFLOP/s, where 256 threads of 4 x 8 outputs with loads through
+// registers reached 27; one-wide multiply-adds lose a fifth.
+template <int WM, int WN, int TM, bool kAT, int EA>
+__global__ void __launch_bounds__(32 * WM * WN, 8 / (WM * WN)) gemm_f32(const __grid_constant__ GemmF32 g)
+{
+    constexpr int NT = 32 * WM * WN, BM = WM * 4 * TM, BN = WN * 64, BK = 16, NS = TM == 8 ? 3 : 6;
+    constexpr int LDA = kAT ? BM : BK + 4;                 // padded rows: four rows' 16 bytes in distinct banks
+    constexpr int SA = kAT ? BK * BM : BM * LDA, SB = BK * BN;
+    constexpr int NA = BM * BK / EA / NT, NB = BN * BK / 4 / NT;  // copies a thread and block
+    static_assert(NA * EA * NT == BM * BK && NB * 4 * NT == BN * BK && TM % 4 == 0, "whole copies");
+    __shared__ __align__(16) float sa[NS][SA], sb[NS][SB];
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, tx = lane % 8, ty = lane / 8;
+    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN, wm = warp / WN * 4 * TM, wn = warp % WN * 64;
+    const int KS = (g.K + BK - 1) / BK, z = blockIdx.z, nz = gridDim.z;
+    const int k_lo = (int)((long long)KS * z / nz) * BK, k_hi = min(g.K, (int)((long long)KS * (z + 1) / nz) * BK);
+
+    // rows and columns past the ends read the last ones' place instead and are not stored; terms
+    // past k_hi are zeros
+    auto load = [&](int k0, int st) {
+        const bool whole = k0 + BK <= k_hi;
 #pragma unroll
-            for (int i = 0; i < LA; ++i) ra[i] = pa[i * sa_i];
-#pragma unroll
-            for (int i = 0; i < LB; ++i) rb[i] = pb[i * sb_i];
-        } else {
-#pragma unroll
-            for (int i = 0; i < LA; ++i) {
-                const int m = kAT ? am : am + SA * i, k = kAT ? ak + SA * i : ak;
-                ra[i] = m0 + m < M && k0 + k < k_hi ? pa[i * sa_i] : 0.0f;
+        for (int i = 0; i < NA; ++i) {
+            const int c = tid + NT * i;
+            const float *src;
+            uint32_t dst, bytes = 4 * EA;
+            if constexpr (kAT) {
+                const int k = c / (BM / EA), m = c % (BM / EA) * EA, mm = m0 + m < g.M ? m0 + m : 0;
+                const int kk = whole || k0 + k < k_hi ? k0 + k : k_lo;
+                src = mm < g.M1 ? g.A + kk * g.lda + mm : mm < g.M2 ? g.A2 + kk * g.lda2 + (mm - g.M1) : kOnes;
+                dst = smem_u32(&sa[st][k * LDA + m]);
+                if (!whole && k0 + k >= k_hi) bytes = 0;
+            } else {
+                const int m = c / (BK / EA), k = c % (BK / EA) * EA;
+                src = g.A + (size_t)min(m0 + m, g.M - 1) * g.lda + k_lo;
+                if (whole || k0 + k < k_hi) src += k0 + k - k_lo;
+                dst = smem_u32(&sa[st][m * LDA + k]);
+                if (!whole) bytes = 4 * max(0, min(EA, k_hi - k0 - k));
             }
-#pragma unroll
-            for (int i = 0; i < LB; ++i) rb[i] = n0 + bn < N && k0 + bk + SB * i < k_hi ? pb[i * sb_i] : 0.0f;
-        }
-        pa += sa_k;
-        pb += sb_k;
-    };
-    auto stash = [&](int b) {
-#pragma unroll
-        for (int i = 0; i < LA; ++i) {
-            const int e = tid + 256 * i;
-            sa[b][kAT ? e / BM : e % BK][kAT ? e % BM : e / BK] = ra[i];
+            if constexpr (EA == 4) tc::cp_async16(dst, src, bytes);
+            else cp_async4(dst, src, bytes);
         }
 #pragma unroll
-        for (int i = 0; i < LB; ++i) {
-            const int e = tid + 256 * i;
-            sb[b][e / BN][e % BN] = rb[i];
+        for (int i = 0; i < NB; ++i) {
+            const int c = tid + NT * i, k = c / (BN / 4), n = c % (BN / 4) * 4;
+            const bool in = whole || k0 + k < k_hi;
+            const float *src = g.B + (in ? k0 + k : k_lo) * g.ldb + (n0 + n < g.N ? n0 + n : n0);
+            const uint32_t dst = smem_u32(&sb[st][k * BN + n]);
+            tc::cp_async16(dst, src, in ? 16 : 0);
         }
     };
-    uint64_t acc[TM][TN / 2];  // pairs of columns
-    float sum[TM][TN];
+
+    uint64_t acc[TM][4];  // pairs of columns
+    float sum[TM][8];
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) {
+        for (int j = 0; j < 8; ++j) {
             acc[i][j / 2] = 0;
             sum[i][j] = 0.0f;
         }
@@ -510,80 +523,100 @@ __global__ void __launch_bounds__(256) gemm_f32(int M, int N, int K, const float
 #pragma unroll
         for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int j = 0; j < TN; j += 2) {
+            for (int j = 0; j < 4; ++j) {
                 float lo, hi;
-                asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[i][j / 2]));
-                sum[i][j] += lo;
-                sum[i][j + 1] += hi;
-                acc[i][j / 2] = 0;
+                asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[i][j]));
+                sum[i][2 * j] += lo;
+                sum[i][2 * j + 1] += hi;
+                acc[i][j] = 0;
             }
     };
-    fetch(k_lo);
-    stash(0);
-    __syncthreads();
-    int b = 0;
-    for (int k0 = k_lo; k0 < k_hi; k0 += BK, b ^= 1) {
-        if (k0 + BK < k_hi) fetch(k0 + BK);
 #pragma unroll
-        for (int k = 0; k < BK; ++k) {
-            float av[TM];
-            uint64_t bv[TN / 2];
-            // rows 4 ty + i (and 64 + 4 ty + i): 16-byte loads without bank conflicts
+    for (int i = 0; i < NS - 1; ++i) {
+        if (k_lo + i * BK < k_hi) load(k_lo + i * BK, i);
+        tc::cp_async_commit();
+    }
+    int st = 0, in = NS - 1;
+    bool odd = false;
+    for (int k0 = k_lo; k0 < k_hi; k0 += BK) {
+        tc::cp_async_wait<NS - 2>();
+        __syncthreads();
+        if (k0 + (NS - 1) * BK < k_hi) load(k0 + (NS - 1) * BK, in);
+        tc::cp_async_commit();
+        const float *pa = kAT ? &sa[st][wm + 4 * ty] : &sa[st][(wm + ty) * LDA], *pb = &sb[st][wn + 4 * tx];
 #pragma unroll
-            for (int i = 0; i < TM; i += 4) *(float4 *)(av + i) = *(const float4 *)&sa[b][k][(i / 4) * 64 + 4 * ty];
+        for (int k = 0; k < BK; k += 4) {
+            float av[TM][4];  // kAT: [4 i + m % 4] at term q; else row ty + 4 i
+            if constexpr (!kAT) {
 #pragma unroll
-            for (int j = 0; j < TN; j += 4)
-                *(ulonglong2 *)(bv + j / 2) = *(const ulonglong2 *)&sb[b][k][(j / 4) * 64 + 4 * tx];
+                for (int i = 0; i < TM; ++i) *(float4 *)av[i] = *(const float4 *)(pa + 4 * i * LDA + k);
+            }
 #pragma unroll
-            for (int i = 0; i < TM; ++i) {
-                const uint64_t a2 = pair2(av[i], av[i]);
+            for (int q = 0; q < 4; ++q) {
+                uint64_t bv[4];
+                if constexpr (kAT) {
 #pragma unroll
-                for (int j = 0; j < TN / 2; ++j) fma2(acc[i][j], a2, bv[j]);
+                    for (int i = 0; i < TM; i += 4) {
+                        const float4 v = *(const float4 *)(pa + (k + q) * LDA + 4 * i);
+                        av[i][q] = v.x;
+                        av[i + 1][q] = v.y;
+                        av[i + 2][q] = v.z;
+                        av[i + 3][q] = v.w;
+                    }
+                }
+                *(ulonglong2 *)bv = *(const ulonglong2 *)(pb + (k + q) * BN);
+                *(ulonglong2 *)(bv + 2) = *(const ulonglong2 *)(pb + (k + q) * BN + 32);
+#pragma unroll
+                for (int i = 0; i < TM; ++i) {
+                    const uint64_t a2 = pair2(av[i][q], av[i][q]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) fma2(acc[i][j], a2, bv[j]);
+                }
             }
         }
-        if (((k0 - k_lo) / BK) & 1) flush();
-        if (k0 + BK < k_hi) stash(b ^ 1);
-        __syncthreads();
+        if (odd) flush();
+        odd = !odd;
+        st = st == NS - 1 ? 0 : st + 1;
+        in = in == NS - 1 ? 0 : in + 1;
     }
+    tc::cp_async_wait<0>();
     flush();
-    float *out = Cm + (size_t)z * slab;
+    float *out = g.C + (size_t)z * g.slab;
 #pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        const int m = m0 + (i / 4) * 64 + 4 * ty + i % 4;
+    for (int j = 0; j < 8; j += 4) {
+        const int n = n0 + wn + 4 * tx + 8 * j;
+        float bi[4] = {};
+        if (g.bias)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) {
-            const int n = n0 + (j / 4) * 64 + 4 * tx + j % 4;
-            if (m < M && n < N) out[(size_t)m * ldc + n] = sum[i][j] + (bias ? bias[n] : 0.0f);
+            for (int q = 0; q < 4; ++q)
+                if (n + q < g.N) bi[q] = g.bias[n + q];
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+            const int m = m0 + wm + (kAT ? 4 * ty + 16 * (i / 4) + i % 4 : ty + 4 * i);
+            if (m >= g.M) continue;
+            float *o = out + (size_t)m * g.ldc + n;
+            if (n < g.N && (g.ldc % 4 | g.N % 4) == 0)
+                *(float4 *)o = make_float4(sum[i][j] + bi[0], sum[i][j + 1] + bi[1], sum[i][j + 2] + bi[2], sum[i][j + 3] + bi[3]);
+            else
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (n + q < g.N) o[q] = sum[i][j + q] + bi[q];
         }
     }
 }
 
-// dbias partial sums: block z sums its rows of dG column by column, 32 rows to a partial
-__global__ void colsum_f32(int R, int G, const float *__restrict__ dG, float *__restrict__ part)
+// sums of the nz slabs in order, compensated: the first n elements to out, the rest to out2
+__global__ void slab_sum_f32(size_t n, size_t n2, int nz, const float *__restrict__ part, size_t slab,
+                             float *__restrict__ out, float *__restrict__ out2)
 {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x, z = blockIdx.y, nz = gridDim.y;
-    if (n >= G) return;
-    const int lo = (int)((long long)R * z / nz), hi = (int)((long long)R * (z + 1) / nz);
-    float sum = 0.0f;
-    for (int r0 = lo; r0 < hi; r0 += 32) {
-        float acc = 0.0f;
-#pragma unroll 8
-        for (int r = r0; r < min(r0 + 32, hi); ++r) acc += dG[(size_t)r * G + n];
-        sum += acc;
-    }
-    part[(size_t)z * G + n] = sum;
-}
-// out[e] = sum of the nz slabs in order, compensated
-__global__ void slab_sum_f32(size_t n, int nz, const float *__restrict__ part, size_t slab, float *__restrict__ out)
-{
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n + n2; e += (size_t)gridDim.x * blockDim.x) {
         float acc = 0.0f, comp = 0.0f;
         for (int z = 0; z < nz; ++z) {
             const float y = part[(size_t)z * slab + e] - comp, t = acc + y;
             comp = (t - acc) - y;
             acc = t;
         }
-        out[e] = acc;
+        *(e < n ? out + e : out2 + (e - n)) = acc;
     }
 }
 
@@ -647,22 +680,27 @@ void fr_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, int clusters, i
     cfg->numAttrs = 1;
 }
 
-// 64 x 128 tiles where they fill the GPU, else 64 x 64 ones
-template <bool kAT>
-void launch_gemm(stacklstm *s, int M, int N, int K, const float *A, size_t lda, int M2, const float *A2, size_t lda2,
-                 const float *Bm, size_t ldb, const float *bias, float *Cm, size_t ldc, int splits, size_t slab)
+// 64 x 64 tiles where they give each SM a few, else 32 x 64 ones (they are a chain of copies and
+// multiply-adds along K that more of them hide: 976 x 75 outputs of 400 terms 28 -> 20 us)
+template <bool kAT, int EA>
+void launch_gemm(stacklstm *s, const GemmF32 &g, int splits)
 {
-    const unsigned mt = ceil_div(M, 64) + ceil_div(M2, 64);
-    if ((size_t)mt * ceil_div(N, 128) * splits >= (size_t)s->num_sms)
-        gemm_f32<4, 8, kAT><<<dim3(mt, ceil_div(N, 128), splits), 256, 0, s->stream>>>(M, N, K, A, lda, M2, A2, lda2, Bm,
-                                                                                       ldb, bias, Cm, ldc, slab);
+    const unsigned nt = ceil_div(g.N, 64), big = ceil_div(g.M, 64);
+    if ((size_t)big * nt * splits >= 3 * (size_t)s->num_sms)
+        gemm_f32<2, 1, 8, kAT, EA><<<dim3(big, nt, splits), 64, 0, s->stream>>>(g);
     else
-        gemm_f32<4, 4, kAT><<<dim3(mt, ceil_div(N, 64), splits), 256, 0, s->stream>>>(M, N, K, A, lda, M2, A2, lda2, Bm,
-                                                                                      ldb, bias, Cm, ldc, slab);
+        gemm_f32<2, 1, 4, kAT, EA><<<dim3(ceil_div(g.M, 32), nt, splits), 64, 0, s->stream>>>(g);
     s->launches += 1;
 }
-
-constexpr int kBiasParts = 64;
+// 16-byte copies of A where its rows allow them (every base is 16-byte aligned)
+template <bool kAT>
+void launch_gemm(stacklstm *s, const GemmF32 &g, int splits)
+{
+    if (g.lda % 4 == 0 && (!kAT || (g.lda2 | g.M1 | g.M2) % 4 == 0))
+        launch_gemm<kAT, 4>(s, g, splits);
+    else
+        launch_gemm<kAT, 1>(s, g, splits);
+}
 
 }  // namespace
 
@@ -704,16 +742,16 @@ bool fp32_plan_rows(stacklstm *s)
             }
         }
     if (!s->fr32.on) return false;
-    // dW: splits of the T B rows for about four 64 x 128 tiles an SM (two at a time), at least
-    // 128 rows each
-    const size_t rows = (size_t)s->T * s->B, tiles = (size_t)(ceil_div(s->I, 64) + ceil_div(H, 64)) * ceil_div(4 * H, 128);
-    s->fr32_split = (int)std::max<size_t>(1, std::min<size_t>(std::min<size_t>(4 * s->num_sms / tiles, rows / 128), 64));
+    // dW and dbias: splits of the T B rows for about two rounds of 64 x 64 tiles (four an SM at
+    // once), at least 128 rows each
+    const size_t rows = (size_t)s->T * s->B, tiles = ceil_div(s->I + H + 1, 64) * ceil_div(4 * H, 64);
+    s->fr32_split = (int)std::max<size_t>(1, std::min<size_t>(std::min<size_t>(8 * s->num_sms / tiles, rows / 128), 64));
     void *p;
-    const size_t slab = (size_t)(s->I + H) * 4 * H;
+    const size_t slab = ((size_t)s->I + H + 1) * 4 * H;
     const char *lim = getenv("STACKLSTM_WAIT_LIMIT_CYCLES"), *limb = getenv("STACKLSTM_WAIT_LIMIT_BWD_CYCLES");
     s->wait_limit = lim ? atoll(lim) : 4000000000LL;
     s->wait_limit_bwd = limb ? atoll(limb) : s->wait_limit;
-    if (cudaMalloc(&p, sizeof(float) * (slab * s->fr32_split + (size_t)kBiasParts * 4 * H)) != cudaSuccess) {
+    if (cudaMalloc(&p, sizeof(float) * slab * s->fr32_split) != cudaSuccess) {
         cudaGetLastError();
         s->fr32.on = 0;
         return false;
@@ -747,7 +785,13 @@ cudaError_t fp32_rows_forward(stacklstm *s, const float *x, const float *W, cons
 {
     const int R = s->T * s->B, I = s->I, G = 4 * s->H;
     s->x_saved = x;
-    launch_gemm<false>(s, R, G, I, x, I, 0, nullptr, 0, W, G, bias, (float *)s->gates, G, 1, 0);
+    GemmF32 g{};
+    g.M = R; g.N = G; g.K = I;
+    g.A = x; g.lda = I;
+    g.B = W; g.ldb = G;
+    g.bias = bias;
+    g.C = (float *)s->gates; g.ldc = G;
+    launch_gemm<false>(s, g, 1);
     FrArgs a{};
     a.wh = W + (size_t)I * G;
     return fr_launch(s, true, a);
@@ -756,41 +800,40 @@ cudaError_t fp32_rows_forward(stacklstm *s, const float *x, const float *W, cons
 cudaError_t fp32_rows_backward(stacklstm *s)
 {
     FrArgs a{};
-    a.wh = (const float *)s->w_fwd + s->I;  // W^T [4H][I + H]: columns I .. are W_h^T
-    a.ldw = (size_t)s->I + s->H;
+    a.wh = (const float *)s->w_fwd + s->I;  // W^T: columns I .. are W_h^T
+    a.ldw = ldw_f32(s);
     return fr_launch(s, false, a);
 }
 
 cudaError_t fp32_rows_dx(stacklstm *s, float *dx)
 {
     if (!dx) return cudaSuccess;
-    launch_gemm<false>(s, s->T * s->B, s->I, 4 * s->H, (const float *)s->dG, 4 * (size_t)s->H, 0, nullptr, 0, (const float *)s->w_fwd,
-                       (size_t)s->I + s->H, nullptr, dx, s->I, 1, 0);
+    GemmF32 g{};
+    g.M = s->T * s->B; g.N = s->I; g.K = 4 * s->H;
+    g.A = (const float *)s->dG; g.lda = 4 * (size_t)s->H;
+    g.B = (const float *)s->w_fwd; g.ldb = ldw_f32(s);
+    g.C = dx; g.ldc = s->I;
+    launch_gemm<false>(s, g, 1);
     return cudaGetLastError();
 }
 
 cudaError_t fp32_rows_dw(stacklstm *s, float *dW, float *dbias)
 {
-    const int R = s->T * s->B, I = s->I, H = s->H, G = 4 * H, nz = s->fr32_split;
-    const float *dG = (const float *)s->dG;
-    const size_t slab = (size_t)(I + H) * G;
-    if (dW) {
-        float *part = nz > 1 ? s->dw_part : dW;
-        launch_gemm<true>(s, I, G, R, (const float *)s->x_saved, I, H, (const float *)s->a_rm, H, dG, G, nullptr, part, G,
-                          nz, slab);
-        if (nz > 1) {
-            slab_sum_f32<<<(unsigned)std::min<size_t>(ceil_div(slab, 256), (size_t)s->num_sms * 8), 256, 0, s->stream>>>(
-                slab, nz, part, slab, dW);
-            s->launches += 1;
-        }
-    }
-    if (dbias) {
-        float *part = s->dw_part + slab * nz;
-        const int parts = std::max(1, std::min(kBiasParts, R / 32));
-        colsum_f32<<<dim3(ceil_div(G, 128), parts), 128, 0, s->stream>>>(R, G, dG, part);
-        slab_sum_f32<<<ceil_div(G, 256), 256, 0, s->stream>>>(G, parts, part, G, dbias);
-        s->launches += 2;
-    }
+    if (!dW && !dbias) return cudaSuccess;
+    const int I = s->I, H = s->H, G = 4 * H, nz = s->fr32_split;
+    GemmF32 g{};
+    g.M1 = dW ? I : 0;
+    g.M2 = dW ? I + H : 0;
+    g.M = g.M2 + (dbias ? 1 : 0);  // dbias: the row of ones
+    g.N = G; g.K = s->T * s->B;
+    g.A = (const float *)s->x_saved; g.lda = I;
+    g.A2 = (const float *)s->a_rm; g.lda2 = H;
+    g.B = (const float *)s->dG; g.ldb = G;
+    g.C = s->dw_part; g.ldc = G; g.slab = (size_t)g.M * G;
+    launch_gemm<true>(s, g, nz);
+    slab_sum_f32<<<(unsigned)std::min<size_t>(ceil_div(g.slab, 256), (size_t)s->num_sms * 8), 256, 0, s->stream>>>(
+        (size_t)g.M2 * G, g.slab - (size_t)g.M2 * G, nz, s->dw_part, g.slab, dW, dbias);
+    s->launches += 1;
     return cudaGetLastError();
 }
 

@@ -176,3 +176,26 @@ def test_row_clusters_report_a_wait_that_runs_out(which):
     finally:
         hd.destroy()
     compare(runner.run(w), oracle_of(w), "fp32")
+
+
+@pytest.mark.parametrize("T,B,I,H", [(30, 33, 31, 32), (30, 33, 32, 32), (40, 47, 60, 67), (30, 50, 128, 128),
+                                     (60, 64, 64, 256)])
+def test_weight_and_bias_gradients_alone_equal_both(T, B, I, H):
+    """dbias is a row of ones below the weight gradient's operand: alone, and dW alone, they are
+    what the call that returns both gives, at row counts on both sides of a tile."""
+    w = wl.make_workload("case", T=T, B=B, I=I, H=H, dtype="fp32", seed=41, ops_kind="random_walk",
+                         probs=(0.5, 0.3, 0.2), bias_scale=0.3, h0_scale=0.5, c0_scale=0.5, dy_scale=0.5)
+    hd = bd.stacklstm_create(T, B, I, H, bd.SL_FP32, 0)
+    try:
+        assert "clusters" in bd.stacklstm_plan(hd)
+        ins, out = runner.upload(w), runner.alloc_outputs(w)
+        runner.forward_backward(hd, ins, out)
+        both = runner.to_numpy(out)
+        compare(both, oracle_of(w), "fp32")
+        for k in ("dW", "dbias"):
+            part = runner.alloc_outputs(w)
+            full = dict(part, **{{"dW": "dbias", "dbias": "dW"}[k]: None})
+            runner.forward_backward(hd, ins, full)
+            assert np.array_equal(full[k].cpu().numpy(), both[k]), k
+    finally:
+        hd.destroy()

@@ -142,6 +142,40 @@ sl_status read_status(stacklstm *s)
 
 // ---- the phases of a forward and a backward call, shared by the single and grouped calls
 
+// The gradient history is cleared on the side stream while the forward runs (the forward
+// leaves most of the memory bandwidth unused), after whatever that stream waited for last: an
+// event of the caller's stream recorded in this forward (a previous backward reads the history).
+sl_status queue_clear(stacklstm *s)
+{
+    // the rows the kernels use: T + 1, or in push-only mode the virtual steps' Tr + 1
+    const size_t hist_bytes = sizeof(float) * (size_t)(s->Tr + 1) * s->B * s->H;
+    const size_t to_c = (char *)s->dhist_c - (char *)s->dhist_h;
+    cudaError_t e;
+    if (s->Tr == s->T)  // one stretch
+        e = cudaMemsetAsync(s->dhist_h, 0, to_c + hist_bytes, s->side);
+    else if (!(e = cudaMemsetAsync(s->dhist_h, 0, hist_bytes, s->side)))
+        e = cudaMemsetAsync(s->dhist_c, 0, hist_bytes, s->side);
+    if (e || (e = cudaEventRecord(s->cleared, s->side))) return cuda_fail(s, e, "clear");
+    s->clear_queued = 1;
+    return SL_OK;
+}
+
+// The clear goes beside the prepass and ends before the steps where row clusters can have an SM
+// for each CTA: a clear whose blocks fill the SMs when the step launch starts makes the
+// scheduler put clusters two to an SM, although others are free, for the whole launch. 64 x 200
+// steps then took 1.5 us instead of 0.97 (a 185-step pass 580 instead of 475 us after an idle
+// stream, and now and then in a full one; three 64-row stacks at once and their head 875 instead
+// of 806). A launch that needs two CTAs an SM, or is one cluster, gains nothing and loses the
+// wait (512 x 200 forward 541 -> 553 us, 1 x 200 190 -> 194).
+bool clear_early(const stacklstm *s) { return s->fr.on && s->fr.spread && !s->push_only; }
+
+sl_status fwd_clear(stacklstm *s)
+{
+    if (clear_early(s)) return SL_OK;
+    if (cudaError_t e = cudaStreamWaitEvent(s->side, s->side_go, 0)) return cuda_fail(s, e, "clear");
+    return queue_clear(s);
+}
+
 // Argument checks, the index prepass and the forward setup (weight packing, initial state).
 sl_status fwd_begin(stacklstm *s, const sl_forward_args &a)
 {
@@ -178,6 +212,8 @@ sl_status fwd_begin(stacklstm *s, const sl_forward_args &a)
         }
         s->stream = main;
         if (e) return cuda_fail(s, e, "forward setup");
+        sl_status st;
+        if (clear_early(s) && (st = queue_clear(s))) return st;
         if ((e = cudaEventRecord(s->aux_done, s->side))) return cuda_fail(s, e, "forward setup");
     }
     if (s->push_only) {
@@ -193,22 +229,6 @@ sl_status fwd_begin(stacklstm *s, const sl_forward_args &a)
         if ((e = sl::bf16_forward_setup_x(s, (const __nv_bfloat16 *)a.x))) return cuda_fail(s, e, "forward setup");
     }
     if ((e = cudaStreamWaitEvent(s->stream, s->aux_done, 0))) return cuda_fail(s, e, "forward setup");
-    return SL_OK;
-}
-
-// The gradient history is cleared on the side stream while the forward runs (the forward
-// leaves most of the memory bandwidth unused); the side stream first waits for `side_go`,
-// recorded on the caller's stream before the forward steps (a previous backward reads it).
-sl_status fwd_clear(stacklstm *s)
-{
-    // the rows the kernels use: T + 1, or in push-only mode the virtual steps' Tr + 1
-    const size_t hist_bytes = sizeof(float) * (size_t)(s->Tr + 1) * s->B * s->H;
-    cudaError_t e;
-    if ((e = cudaStreamWaitEvent(s->side, s->side_go, 0)) ||
-        (e = cudaMemsetAsync(s->dhist_h, 0, hist_bytes, s->side)) ||
-        (e = cudaMemsetAsync(s->dhist_c, 0, hist_bytes, s->side)) || (e = cudaEventRecord(s->cleared, s->side)))
-        return cuda_fail(s, e, "clear");
-    s->clear_queued = 1;
     return SL_OK;
 }
 
@@ -415,12 +435,13 @@ sl_status stacklstm_create(stacklstm_t *out, int T, int B, int I, int H, sl_dtyp
         return SL_ERR_UNSUPPORTED;
     }
     const size_t TB = (size_t)T * B, T1B = (size_t)(T + 1) * B, K = (size_t)I + H, G = 4 * (size_t)H;
-    const size_t es = elem_size(dtype);
+    const size_t es = elem_size(dtype), dhist = (T1B * H * 4 + 255) / 256 * 256;
     bool ok = alloc(s, &s->p_traj, T1B * 4) && alloc(s, &s->top, T1B * 4) && alloc(s, &s->slot_last, T1B * 4) &&
               alloc(s, &s->err, 16) && alloc(s, &s->hist_h, T1B * H * es) && alloc(s, &s->hr, dtype == SL_BF16 ? T1B * H * 2 : 16) && alloc(s, &s->hist_c, T1B * H * 4) &&
               alloc(s, &s->gates, dtype == SL_BF16 ? TB * 4 * (((size_t)H + 15) / 16 * 16) * 2 : TB * G * 4) && alloc(s, &s->a_rm, dtype == SL_FP32 ? TB * K * es : 16) &&
-              alloc(s, &s->dhist_h, T1B * H * 4) && alloc(s, &s->dhist_c, T1B * H * 4) &&
+              alloc(s, &s->dhist_h, dhist + T1B * H * 4) &&
               alloc(s, &s->dG, TB * G * es);
+    if (ok) s->dhist_c = s->dhist_h + dhist / 4;
     if (ok && dtype == SL_FP32) ok = alloc(s, &s->w_fwd, (K + 3) / 4 * 4 * G * 4);
     if (ok && dtype == SL_BF16) ok = sl::bf16_prepare(s) == cudaSuccess;
     if (ok) ok = sl::configure_prepass(s) == cudaSuccess;

@@ -777,6 +777,7 @@ bool rc_plan(stacklstm *s, bool fwd, int NT, PersistPlan *pl)
     pl->smem = smem;
     pl->threads = kRcThreads;
     pl->per_sm = 2;
+    pl->spread = s->B > NR && 2 * (int)ceil_div(s->B, NR) <= clusters;
     return true;
 }
 

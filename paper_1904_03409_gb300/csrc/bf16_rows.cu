@@ -188,7 +188,7 @@ __host__ __device__ constexpr uint32_t rc_fwd_smem(int KX, int KH, int NT)
 }
 
 // registers a thread after the split of the block's 256 x 128 between its two warpgroups
-constexpr int kRcRegsStep = 200, kRcRegsX = 56;    // forward
+constexpr int kRcRegsStep = 192, kRcRegsX = 64;    // forward
 constexpr int kRcRegsBwd = 160, kRcRegsBwd2 = 96;  // backward, two N tiles
 
 template <int KH, int NT>
@@ -250,34 +250,43 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rows(const __grid_constant
         // 16 / NT threads a row; row r's pieces tl, tl + 16 / NT, ...
         const int xr = (tid & 127) / (16 / NT), tl = (tid & 127) % (16 / NT);
         const __nv_bfloat16 *xp = p.x + ((size_t)row0 + xr) * I;
-        auto load_x = [&](int t) {
-            if (t < T && xr < nrows) {
-                const __nv_bfloat16 *src = xp + (size_t)t * B * I;
-                const uint32_t dst = s_x + (t & (kRcX - 1)) * xb_bytes + xr * SX;
-                for (int q = tl; q < I / 8; q += 16 / NT) tc::cp_async16(dst + q * 16, src + q * 8, 16);
-            }
+        // XS steps at a time: a weight fragment is read from shared memory once for all of them,
+        // the largest part of what two CTAs an SM ask of it (256 x 200: 1.53 us a step, 1.34 by
+        // twos; by fours the burst delays the steps, 1.49; two N tiles by twos spill, 2.96 for 2.63)
+        constexpr int XS = NT == 1 ? 2 : 1;
+        auto load_x = [&](int t0) {  // steps t0 ..
+#pragma unroll
+            for (int t = t0; t < t0 + XS; ++t)
+                if (t < T && xr < nrows) {
+                    const __nv_bfloat16 *src = xp + (size_t)t * B * I;
+                    const uint32_t dst = s_x + (t & (kRcX - 1)) * xb_bytes + xr * SX;
+                    for (int q = tl; q < I / 8; q += 16 / NT) tc::cp_async16(dst + q * 16, src + q * 8, 16);
+                }
             tc::cp_async_commit();
         };
-        for (int t = 0; t < kRcX - 1; ++t) load_x(t);
+        constexpr int ahead = kRcX / XS - 1;
+        for (int i = 0; i < ahead; ++i) load_x(i * XS);
         float bias[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) bias[q] = warp_on ? a.bias[q * H + u] : 0.0f;
         // A rows (lane % 16), column half (lane / 16) of the warp's M tiles
         const uint32_t wa = s_wx + (uint32_t)(w4 * 32 + (lane & 15)) * SX + (lane >> 4) * 16;
         bool ok = rc_wait<false>(bar(2), 0, limit, abort, a.err);
-        for (int t = 0; t < T; ++t) {
-            tc::cp_async_wait<kRcX - 2>();
-            // x_t is in place, and every warp has read x_{t-1}, whose buffer is loaded next
+        for (int t = 0; t < T; t += XS) {
+            tc::cp_async_wait<ahead - 1>();
+            // these steps' x is in place, and every warp has read the ones before, whose buffers
+            // are loaded next
             if (tc::bar_any(1, 128, !ok)) break;
-            load_x(t + kRcX - 1);
+            load_x(t + ahead * XS);
             if (!warp_on) continue;
-            const int b = t & 1;
-            if (t >= 2) ok = rc_wait<false>(bar(11 + 2 * w4 + b), (uint32_t)((t >> 1) - 1) & 1, limit, abort, a.err);
-            float acc[2][NT][4];
+            float acc[XS][2][NT][4];
 #pragma unroll
-            for (int n = 0; n < NT; ++n)
+            for (int e = 0; e < XS; ++e)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[q >> 1][n][(q & 1) * 2] = acc[q >> 1][n][(q & 1) * 2 + 1] = bias[q];
+                for (int n = 0; n < NT; ++n)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        acc[e][q >> 1][n][(q & 1) * 2] = acc[e][q >> 1][n][(q & 1) * 2 + 1] = bias[q];
             const uint32_t xa = s_x + (t & (kRcX - 1)) * xb_bytes + (lane & 7) * SX + ((lane >> 3) & 1) * 16;
 #pragma unroll 2
             for (int k = 0; k < KX; ++k) {
@@ -285,20 +294,29 @@ __global__ void __launch_bounds__(kRcThreads, 2) step_rows(const __grid_constant
                 ldsm4(A0, wa + k * 32);
                 ldsm4(A1, wa + 16 * SX + k * 32);
 #pragma unroll
-                for (int n = 0; n < NT; ++n) {
-                    ldsm2(bb, xa + n * 8 * SX + k * 32);
-                    mma16816(acc[0][n], make_uint4(A0[0], A0[1], A0[2], A0[3]), bb[0], bb[1]);
-                    mma16816(acc[1][n], make_uint4(A1[0], A1[1], A1[2], A1[3]), bb[0], bb[1]);
-                }
+                for (int e = 0; e < XS; ++e)
+#pragma unroll
+                    for (int n = 0; n < NT; ++n) {
+                        ldsm2(bb, xa + (e * NR + n * 8) * SX + k * 32);
+                        mma16816(acc[e][0][n], make_uint4(A0[0], A0[1], A0[2], A0[3]), bb[0], bb[1]);
+                        mma16816(acc[e][1][n], make_uint4(A1[0], A1[1], A1[2], A1[3]), bb[0], bb[1]);
+                    }
             }
-            uint8_t *out = smem + (s_xf - s_wx) + (w4 * 2 + b) * xf_bytes + lane * 16;
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int e = 0; e < XS; ++e) {
+                if (t + e >= T) break;
+                const int b = (t + e) & 1;
+                if (t + e >= 2) ok = ok && rc_wait<false>(bar(11 + 2 * w4 + b), (uint32_t)(((t + e) >> 1) - 1) & 1, limit, abort, a.err);
+                uint8_t *out = smem + (s_xf - s_wx) + (w4 * 2 + b) * xf_bytes + lane * 16;
 #pragma unroll
-                for (int n = 0; n < NT; ++n)
-                    *(float4 *)(out + (i * NT + n) * 512) = make_float4(acc[i][n][0], acc[i][n][1], acc[i][n][2], acc[i][n][3]);
-            __syncwarp();
-            if (lane == 0) tc::mbar_arrive(&bars[3 + 2 * w4 + b]);
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int n = 0; n < NT; ++n)
+                        *(float4 *)(out + (i * NT + n) * 512) =
+                            make_float4(acc[e][i][n][0], acc[e][i][n][1], acc[e][i][n][2], acc[e][i][n][3]);
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&bars[3 + 2 * w4 + b]);
+            }
         }
         tc::cp_async_wait<0>();
     } else {
@@ -736,8 +754,8 @@ void rc_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, int clusters, i
 
 // One direction with NT 8-row N tiles a cluster: every cluster co-resident (two CTAs an SM),
 // or the plan is off: a second round of clusters would double the time. At H = 200 that is 36
-// clusters: NT = 1, 288 rows, 0.96 / 1.03 us a step up to 14 clusters (one CTA an SM) and 1.50 /
-// 1.50 beyond, against 1.6 / 2.3 of the 64-row clusters; NT = 2, 576 rows at 2.66 / 2.51, against
+// clusters: NT = 1, 288 rows, 0.96 / 1.03 us a step up to 14 clusters (one CTA an SM) and 1.34 /
+// 1.50 beyond, against 1.6 / 2.3 of the 64-row clusters; NT = 2, 576 rows at 2.63 / 2.51, against
 // 4.02 / 6.05 of the persistent kernels (the 64-row clusters reach 448 rows; at 1024, two rounds
 // of NT = 2 take 5.15 / 4.97, the persistent kernels 4.55 / 6.14).
 bool rc_plan(stacklstm *s, bool fwd, int NT, PersistPlan *pl)

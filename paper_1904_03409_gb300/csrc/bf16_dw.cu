@@ -269,11 +269,20 @@ __global__ void dw_reduce_pad(int I, int H, int kbx, int split, const float *__r
     }
 }
 
+// The most splits of RC chunks of 64 rows: 16 chunks to each (a CTA's start and partial sums cost
+// about as much as ten), or four where that leaves more than half the SMs idle; dx has the other
+// half. (77 x 100 rows, 72 + 104 x 416: 7 splits 23 us, 21 splits 17; with more than half the
+// SMs, at 64 x 185 rows and 200 + 200 x 800, dW is 2 us shorter and the pass with dx 5 longer.)
+size_t dw_max_split(size_t RC, size_t tiles, size_t sms)
+{
+    return std::max<size_t>({1, RC / 16, std::min(RC / 4, sms / 2 / tiles)});
+}
+
 }  // namespace
 
 // Tile shape, splits and ring depth. 128 x 256 tiles run two CTAs an SM (one's partial-sum
 // epilogue overlaps the other's contraction) with a two-stage ring, splits for about two
-// waves of such pairs (at least 16 chunks per CTA); their MMAs need about 94 bytes of
+// waves of such pairs; their MMAs need about 94 bytes of
 // operands a cycle per SM at the full tensor rate, more than TMA delivers (they ran at
 // 70-81 % of it). 256 x 256 tiles share one dG operand between two accumulators: one CTA
 // an SM, a three-stage ring, and about 62 bytes a cycle. Cost (cycles) = waves x chunks per
@@ -286,7 +295,6 @@ cudaError_t bf16_plan_dw(stacklstm *s)
     const int I = s->I, H = s->H, sms = s->num_sms;
     const size_t R = (size_t)s->T * s->B, RC = ceil_div(R, 64);
     const int kbx = (int)ceil_div(I, 64), kbh = (int)ceil_div(H, 64);
-    const size_t max_split = std::max<size_t>(1, RC / 16);
     s->dw_ntile = kDwN;
     s->dw_nt = (int)ceil_div(4 * H, kDwN);
     // partial sums of `sp` splits over `rows` padded m rows: written, then read by the reduction
@@ -296,7 +304,7 @@ cudaError_t bf16_plan_dw(stacklstm *s)
     // 128 x 256, two CTAs an SM: splits for about two waves of pairs
     const int mt128 = (kbx + kbh + 1) / 2;
     const size_t tiles128 = (size_t)mt128 * s->dw_nt;
-    const size_t split128 = std::min(max_split, std::max<size_t>(1, ceil_div(4 * (size_t)sms, tiles128)));
+    const size_t split128 = std::min(dw_max_split(RC, tiles128, sms), std::max<size_t>(1, ceil_div(4 * (size_t)sms, tiles128)));
     const double cost128 = (double)ceil_div(tiles128 * split128, 2 * (size_t)sms) * ceil_div(RC, split128) * 1460.0 +
                            part_cycles(split128, (size_t)mt128 * 128);
     // 256 x 256, one CTA an SM: the split count with the fewest waves x chunks
@@ -304,7 +312,7 @@ cudaError_t bf16_plan_dw(stacklstm *s)
     const size_t tiles256 = (size_t)mt256 * s->dw_nt;
     size_t split256 = 1;
     double cost256 = 1e300;
-    for (size_t sp = 1; sp <= max_split; ++sp) {
+    for (size_t sp = 1; sp <= dw_max_split(RC, tiles256, sms); ++sp) {
         const double c = (double)ceil_div(tiles256 * sp, (size_t)sms) * ceil_div(RC, sp) * 1140.0 +
                          part_cycles(sp, (size_t)mt256 * 256);
         if (c < cost256 * 0.999) {
@@ -334,8 +342,8 @@ cudaError_t bf16_launch_dw(stacklstm *s, const CUtensorMap &tm_x, const CUtensor
     w.kbx = (int)ceil_div(s->I, 64);
     w.kbh = (int)ceil_div(s->H, 64);
     w.n_nt = s->dw_nt;
-    // every split keeps at least 16 chunks of 64 rows (fewer rows than planned: push-only mode)
-    w.split = (int)std::min<size_t>(s->dw_split, std::max<size_t>(1, ceil_div((size_t)w.R, 64) / 16));
+    // (fewer rows than planned: push-only mode)
+    w.split = (int)std::min<size_t>(s->dw_split, dw_max_split(ceil_div((size_t)w.R, 64), (size_t)s->dw_mt * s->dw_nt, s->num_sms));
     w.S = s->sw;
     w.part = s->dw_part;
     w.ld_part = (size_t)s->dw_nt * s->dw_ntile;

@@ -318,41 +318,34 @@ sl_status bwd_steps(stacklstm *s, const sl_backward_args &a, bool *dx_done)
 }
 
 // dx (unless the step launch computed it on otherwise idle SMs), dW and dbias, dh0 and dc0.
+// dW runs on the caller's stream; dx, which like dW only reads the gate gradients, and the
+// copy of the initial state's gradients on the side stream at the same time; the caller's stream waits for them.
 sl_status bwd_end(stacklstm *s, const sl_backward_args &a, bool dx_done)
 {
-    const int B = s->B, H = s->H;
     cudaError_t e;
-    // dx and dW both only read the gate gradients, so dx runs on the side stream at the same
-    // time as dW; the caller's stream waits for it
-    const bool side_dx = !dx_done && a.dx;
-    if (side_dx) {
+    const bool side = (!dx_done && a.dx) || a.dh0 || a.dc0;
+    if (side) {
         if ((e = cudaEventRecord(s->aux_go, s->stream)) || (e = cudaStreamWaitEvent(s->side, s->aux_go, 0)))
             return cuda_fail(s, e, "dx");
-        const cudaStream_t main = s->stream;
-        s->stream = s->side;
-        {
-            Phase ph(s, SL_PHASE_DX);
-            e = s->dt == SL_FP32 ? sl::fp32_dx(s, a.dx) : sl::bf16_dx(s, a.dx);
+        if (!dx_done && a.dx) {
+            const cudaStream_t main = s->stream;
+            s->stream = s->side;
+            {
+                Phase ph(s, SL_PHASE_DX);
+                e = s->dt == SL_FP32 ? sl::fp32_dx(s, a.dx) : sl::bf16_dx(s, a.dx);
+            }
+            s->stream = main;
+            if (e) return cuda_fail(s, e, "dx");
         }
-        s->stream = main;
-        if (e) return cuda_fail(s, e, "dx");
+        if ((e = sl::launch_h0_grads(s, a.dh0, a.dc0, s->side))) return cuda_fail(s, e, "dh0, dc0");
         if ((e = cudaEventRecord(s->aux_done, s->side))) return cuda_fail(s, e, "dx");
-    } else if (!dx_done) {
-        Phase ph(s, SL_PHASE_DX);
-        e = s->dt == SL_FP32 ? sl::fp32_dx(s, a.dx) : sl::bf16_dx(s, a.dx);
-        if (e) return cuda_fail(s, e, "dx");
     }
     {
         Phase ph(s, SL_PHASE_DW);
         e = s->dt == SL_FP32 ? sl::fp32_dw(s, a.dW, a.dbias) : sl::bf16_dw(s, a.dW, a.dbias);
         if (e) return cuda_fail(s, e, "dW");
     }
-    if (side_dx && (e = cudaStreamWaitEvent(s->stream, s->aux_done, 0))) return cuda_fail(s, e, "dx");
-    // slot 0 always holds the initial state, which is history row 0
-    if (a.dh0 && (e = cudaMemcpyAsync(a.dh0, s->dhist_h, sizeof(float) * B * H, cudaMemcpyDeviceToDevice, s->stream)))
-        return cuda_fail(s, e, "dh0");
-    if (a.dc0 && (e = cudaMemcpyAsync(a.dc0, s->dhist_c, sizeof(float) * B * H, cudaMemcpyDeviceToDevice, s->stream)))
-        return cuda_fail(s, e, "dc0");
+    if (side && (e = cudaStreamWaitEvent(s->stream, s->aux_done, 0))) return cuda_fail(s, e, "dx");
     return SL_OK;
 }
 

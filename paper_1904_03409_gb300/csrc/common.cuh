@@ -170,6 +170,7 @@ cudaError_t launch_compact(stacklstm *s);
 cudaError_t read_virtual_steps(stacklstm *s);
 // push-only mode: zero the rows of dx [T][B][I] that belong to non-push steps
 cudaError_t launch_zero_nonpush_rows(stacklstm *s, float *dx);
+cudaError_t launch_h0_grads(stacklstm *s, float *dh0, float *dc0, cudaStream_t st);
 
 // ---- fp32 CUDA-core path (fp32_path.cu)
 // plans the fp32 path (s->fp32_one_cta) and describes it

@@ -480,6 +480,17 @@ compact_kernel(int T, int B, const int32_t *__restrict__ p_traj, const int32_t *
     atomicMax(kmax, k);
 }
 
+// The initial state's gradients: history row 0 (slot 0 always holds the initial state). One
+// launch for both; two copies are bound by their starts, 2 x 3.5 us.
+__global__ void h0_grads_kernel(int n, const float *__restrict__ dh, const float *__restrict__ dc, float *__restrict__ dh0,
+                                float *__restrict__ dc0)
+{
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+        if (dh0) dh0[e] = dh[e];
+        if (dc0) dc0[e] = dc[e];
+    }
+}
+
 // Push-only mode: dx rows of the steps that do not push are zero (a state no step reads
 // has zero gradient); the push rows are written by the input-gradient contraction.
 // A warp per row: the row's step index is read once, its 16-byte pieces written by the
@@ -528,6 +539,15 @@ cudaError_t read_virtual_steps(stacklstm *s)
     // push at all runs one virtual step whose write nobody reads)
     s->Tr = std::max(1, std::min(s->T, (int)*s->kmax_host));
     return cudaSuccess;
+}
+
+cudaError_t launch_h0_grads(stacklstm *s, float *dh0, float *dc0, cudaStream_t st)
+{
+    if (!dh0 && !dc0) return cudaSuccess;
+    const int n = s->B * s->H;
+    h0_grads_kernel<<<std::min((int)ceil_div(n, 256), s->num_sms), 256, 0, st>>>(n, s->dhist_h, s->dhist_c, dh0, dc0);
+    s->launches += 1;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_zero_nonpush_rows(stacklstm *s, float *dx)

@@ -136,6 +136,9 @@ def phase_kernel(plan, phase, dtype):
         if "one CTA" in plan:
             return {"forward": ("fwd_seq_f32", "fp32_path.cu", 1), "backward": ("bwd_seq_f32", "fp32_path.cu", 1),
                     "dx": ("dx_f32", "fp32_path.cu", 1), "dw": ("dw_f32", "fp32_path.cu", 1)}[phase]
+        if "clusters" in plan:
+            return {"forward": ("fwd_rows_f32", "fp32_rows.cu", 1), "backward": ("bwd_rows_f32", "fp32_rows.cu", 1),
+                    "dx": ("gemm_f32", "fp32_rows.cu", 1), "dw": ("gemm_f32", "fp32_rows.cu", 1)}[phase]
         return {"forward": ("fwd_step_f32", "fp32_path.cu", "T"),
                 "backward": ("bwd_pointwise_f32+bwd_contract_f32", "fp32_path.cu", "2T"),
                 "dx": ("dx_f32", "fp32_path.cu", 1), "dw": ("dw_f32", "fp32_path.cu", 1)}[phase]
@@ -143,6 +146,10 @@ def phase_kernel(plan, phase, dtype):
         m = re.search(phase + r" (persistent|per-step|cluster|cuda-core) U=(\d+)", plan)
         if m and m.group(1) == "cuda-core":
             return "%s<BT>" % ("step_ccf" if phase == "forward" else "step_ccb"), "bf16_small.cu", 1
+        rows = re.search(phase + r" cluster U=\d+ \[[^]]*\brows (\d+)", plan)
+        if rows and int(rows.group(1)) > 0:
+            return ("%s<%s rows>" % ("step_rows" if phase == "forward" else "step_rowsb", rows.group(1)),
+                    "bf16_rows.cu", 1)
         if m and m.group(1) == "cluster":
             return ("%s<U=%s,%s>" % ("step_cl" if phase == "forward" else "step_clb", m.group(2), phase),
                     "bf16_cluster.cu", 1)

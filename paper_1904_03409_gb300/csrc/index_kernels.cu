@@ -332,14 +332,14 @@ __global__ void seed_grads_kernel(int T, int B, int H, const int32_t *__restrict
 }
 
 // The same seeding with per-step gradients dy, for one instance and 32 N units per block
-// (one warp, N units a lane): the sums of the T + 1 rows accumulate on chip in the same order
-// as above (final top, then t = T-1..0), the row that is on top in registers and the others in
-// shared memory, then every row is written once. The gradient history is zero before the
-// seeding, so writing the sums equals adding them. A warp's chain is one change of row a step
-// (a store and a load of shared memory); the loads run 24 to 32 steps ahead of it, by
-// asynchronous copies into a ring of which each lane reads back only its own (eight steps ahead
-// in registers left it waiting for memory: 64 x 200, 185 steps, 23 -> 18 us; 256 x 1024, 256 steps,
-// 281 -> 185 us). What is left is one warp's own instructions, about 190 cycles a step.
+// (one warp, N units a lane): the sums of the T + 1 rows accumulate in shared memory in the same
+// order as above (final top, then t = T-1..0), then every row is written once. The gradient
+// history is zero before the seeding, so writing the sums equals adding them. A step is one
+// addition to a row in shared memory (the top's row held in registers, stored and loaded at a
+// change of row, took a branch a step: 256 x 1024, 256 steps, 185 us, 170 so); the loads run 24
+// to 32 steps ahead, by asynchronous copies into a ring of which each lane reads back only its own
+// (eight steps ahead in registers left it waiting for memory: 281 us; rings of 16 and 64 steps
+// 192, 199; a block to an instance and 64 units with its rows in parallel 279).
 constexpr int kSeedRing = 32, kSeedGroup = 8;  // steps in flight, steps a copy group
 template <int N>
 __global__ void __launch_bounds__(32) seed_grads_dy_kernel(int T, int B, int H, const int32_t *__restrict__ top,
@@ -372,17 +372,23 @@ __global__ void __launch_bounds__(32) seed_grads_dy_kernel(int T, int B, int H, 
     int s_cur = tops(0), s_nxt = T > 32 ? tops(32) : 0;
     for (int i = lane; i < (T + 1) * 8 * N; i += 32) ((uint4 *)(slot - lane))[i] = make_uint4(0, 0, 0, 0);
     __syncwarp();
-    int cur = top[(size_t)T * B + b];
-    Vec acc{};
     if (d_top_h) {
+        Vec acc{};
         const Vec d = *(const Vec *)(d_top_h + e);
 #pragma unroll
         for (int i = 0; i < N; ++i) acc.f[i] += d.f[i];
+        slot[32 * top[(size_t)T * B + b]] = acc;
     }
+    auto add = [&](int r, const Vec &g) {
+        Vec acc = slot[32 * r];
+#pragma unroll
+        for (int k = 0; k < N; ++k) acc.f[k] += g.f[k];
+        slot[32 * r] = acc;
+    };
     for (int i0 = 0; i0 < T; i0 += kSeedGroup) {
         fetch(i0 + kSeedRing - kSeedGroup);
         asm volatile("cp.async.wait_group %0;" ::"n"(kSeedRing / kSeedGroup - 1) : "memory");
-        // the group's gradients and rows first: only the change of row stays on the chain
+        // the group's gradients and rows first: only the additions stay on the chain
         int s[kSeedGroup];
         Vec g[kSeedGroup];
 #pragma unroll
@@ -390,23 +396,19 @@ __global__ void __launch_bounds__(32) seed_grads_dy_kernel(int T, int B, int H, 
             s[i] = __shfl_sync(0xffffffffu, s_cur, (i0 + i) & 31);
             g[i] = ring[32 * ((i0 + i) % kSeedRing)];
         }
+        if (i0 + kSeedGroup <= T) {
 #pragma unroll
-        for (int i = 0; i < kSeedGroup; ++i) {
-            if (i0 + i >= T) break;
-            if (s[i] != cur) {
-                slot[32 * cur] = acc;
-                acc = slot[32 * s[i]];
-                cur = s[i];
-            }
+            for (int i = 0; i < kSeedGroup; ++i) add(s[i], g[i]);
+        } else {
 #pragma unroll
-            for (int k = 0; k < N; ++k) acc.f[k] += g[i].f[k];
+            for (int i = 0; i < kSeedGroup; ++i)
+                if (i0 + i < T) add(s[i], g[i]);
         }
         if ((i0 + kSeedGroup) % 32 == 0) {
             s_cur = s_nxt;
             if (i0 + kSeedGroup + 32 < T) s_nxt = tops(i0 + kSeedGroup + 32);
         }
     }
-    slot[32 * cur] = acc;
     if (on)
 #pragma unroll 8
         for (int r = 0; r <= T; ++r) *(Vec *)(dhist_h + (size_t)r * step + e) = slot[32 * r];

@@ -22,50 +22,46 @@ constexpr uint32_t kAStage = kRows * 128;
 constexpr int kMaxStages = 16;
 constexpr long long kDrainLimit = 4000000000LL;  // wait for own copies / MMAs before exit
 
-// ---- weight packing (one output element each; the forward setup runs all of them in one
-// launch, bf16_path.cu)
+// ---- weight packing (one output element or 16-byte piece each; the forward setup runs all of
+// them in one launch, bf16_path.cu)
 // Forward operand: for column tile ct, rows n = g * U + j hold gate g of hidden unit
 // ct * U + j; each row is the matching column of W over the contraction
 // [x padded to 64 ; h padded to 64], in 64-element chunks of 128-byte swizzled rows.
-// Element e of [n_ct][KC][4U rows][64].
-__device__ __forceinline__ void pack_gate_cols_elem(size_t e, const __nv_bfloat16 *__restrict__ W, int I, int H, int U,
-                                                    int kcx, int KC, __nv_bfloat16 *__restrict__ out)
+// Piece e of [n_ct][KC][8 pieces][4U rows]: consecutive threads take consecutive units, so the
+// eight reads of each are of whole rows of W (an element a thread along the contraction read
+// 32 bytes for each two: 256 x 1024 setup 75 us).
+__device__ __forceinline__ void pack_gate_cols_piece(uint32_t e, const __nv_bfloat16 *__restrict__ W, int I, int H, int U,
+                                                     int kcx, int KC, __nv_bfloat16 *__restrict__ out)
 {
-    const int NB = 4 * U, G = 4 * H;
-    const int col = (int)(e % kChunk);
-    const size_t rowi = e / kChunk;  // (ct * KC + kc) * NB + row
-    const int row = (int)(rowi % NB);
-    const size_t tile = rowi / NB;
+    const uint32_t NB = 4 * U, row = e % NB, t = e / NB, piece = t % 8, tile = t / 8;
     const int kc = (int)(tile % KC), ct = (int)(tile / KC);
-    const int g = row / U, unit = ct * U + row % U;
-    int wrow = -1;
-    if (kc < kcx) {
-        const int k = kc * kChunk + col;
-        if (k < I) wrow = k;
-    } else {
-        const int k = (kc - kcx) * kChunk + col;
-        if (k < H) wrow = I + k;
-    }
-    const __nv_bfloat16 v = (unit < H && wrow >= 0) ? W[(size_t)wrow * G + g * H + unit] : __float2bfloat16(0.0f);
-    const size_t byte = tile * NB * 128 + sw128(row, col >> 3) + (col & 7) * 2;
-    out[byte / 2] = v;
+    const int g = (int)row / U, unit = ct * U + (int)row % U;
+    const bool is_x = kc < kcx;
+    const int k0 = (is_x ? kc : kc - kcx) * kChunk + (int)piece * 8, n = is_x ? I : H;
+    const __nv_bfloat16 *src = W + (size_t)((is_x ? 0 : I) + k0) * 4 * H + g * H + unit;
+    union {
+        __nv_bfloat16 v[8];
+        uint4 q;
+    } o;
+    o.q = make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (unit < H && k0 + i < n) o.v[i] = src[(size_t)i * 4 * H];
+    *(uint4 *)((uint8_t *)out + (size_t)tile * NB * 128 + sw128(row, piece)) = o.q;
 }
 // Backward operands: for column tile ct, row m is W row (row0 + ct * NB + m) over the 4H
 // gate columns (zero padded): W_h rows (row0 = I, rows < I + H) for dh_read, W_x rows
-// (row0 = 0, rows < I) for dx. Element e of [n_ct][KC][NB rows][64].
-__device__ __forceinline__ void pack_w_rows_elem(size_t e, const __nv_bfloat16 *__restrict__ W, int H, int row0,
-                                                 int nrows, int NB, int KC, __nv_bfloat16 *__restrict__ out)
+// (row0 = 0, rows < I) for dx. Piece e of [n_ct][KC][NB rows][8 pieces] (H % 8 == 0: whole pieces
+// of W, 16-byte aligned).
+__device__ __forceinline__ void pack_w_rows_piece(uint32_t e, const __nv_bfloat16 *__restrict__ W, int H, int row0,
+                                                  int nrows, int NB, int KC, __nv_bfloat16 *__restrict__ out)
 {
-    const int G = 4 * H;
-    const int col = (int)(e % kChunk);
-    const size_t rowi = e / kChunk;
-    const int row = (int)(rowi % NB);
-    const size_t tile = rowi / NB;
-    const int kc = (int)(tile % KC), ct = (int)(tile / KC);
-    const int m = ct * NB + row, k = kc * kChunk + col;
-    const __nv_bfloat16 v = (m < nrows && k < G) ? W[(size_t)(row0 + m) * G + k] : __float2bfloat16(0.0f);
-    const size_t byte = tile * NB * 128 + sw128(row, col >> 3) + (col & 7) * 2;
-    out[byte / 2] = v;
+    const uint32_t piece = e % 8, t = e / 8, row = t % NB, tile = t / NB;
+    const int kc = (int)(tile % KC), ct = (int)(tile / KC), G = 4 * H;
+    const int m = ct * NB + (int)row, k = kc * kChunk + (int)piece * 8;
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (m < nrows && k < G) v = *(const uint4 *)(W + (size_t)(row0 + m) * G + k);
+    *(uint4 *)((uint8_t *)out + (size_t)tile * NB * 128 + sw128(row, piece)) = v;
 }
 // Weight chunks of the cluster backward (bf16_cluster.cu): for CTA ct, chunk j, the 16 x 64
 // block B[n][16 g + e] = W[I + 16 ct + n][g H + 16 j + e] (zero past H), 128-byte swizzled

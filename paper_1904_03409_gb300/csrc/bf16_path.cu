@@ -413,15 +413,15 @@ __global__ void __launch_bounds__(kThreads, 1) dx_tc(const __grid_constant__ CUt
 // ------------------------------------------------------------------ packing
 // The forward setup in one launch: the initial state into history row 0 (h0 also as the
 // first h operand) and every weight tile the launches that follow read, each job a range of
-// a flat element index (pack_*_elem, bf16_dev.cuh).
+// a flat index of elements or pieces (pack_*, bf16_dev.cuh).
 struct SetupArgs {
     const __nv_bfloat16 *W;
     int I, H;
-    __nv_bfloat16 *wf;  // forward gate columns (n_f elements; 0: packed elsewhere)
+    __nv_bfloat16 *wf;  // forward gate columns (n_f pieces; 0: packed elsewhere)
     int uf, kcx, kcf;
-    __nv_bfloat16 *wb;  // persistent / per-step backward rows (n_b; 0: not needed)
+    __nv_bfloat16 *wb;  // persistent / per-step backward rows (n_b pieces; 0: not needed)
     int ub, kcb;
-    __nv_bfloat16 *wdx;  // input-gradient rows (n_dx)
+    __nv_bfloat16 *wdx;  // input-gradient rows (n_dx pieces)
     int nx;
     __nv_bfloat16 *wcl;  // cluster backward slices (n_cl; 0: not needed)
     int n_ctc;
@@ -448,15 +448,15 @@ __global__ void setup_kernel(SetupArgs a)
             continue;
         }
         if ((r -= a.n_c) < a.n_f) {
-            pack_gate_cols_elem(r, a.W, a.I, a.H, a.uf, a.kcx, a.kcf, a.wf);
+            pack_gate_cols_piece((uint32_t)r, a.W, a.I, a.H, a.uf, a.kcx, a.kcf, a.wf);
             continue;
         }
         if ((r -= a.n_f) < a.n_b) {
-            pack_w_rows_elem(r, a.W, a.H, a.I, a.H, a.ub, a.kcb, a.wb);
+            pack_w_rows_piece((uint32_t)r, a.W, a.H, a.I, a.H, a.ub, a.kcb, a.wb);
             continue;
         }
         if ((r -= a.n_b) < a.n_dx) {
-            pack_w_rows_elem(r, a.W, a.H, 0, a.I, a.nx, a.kcb, a.wdx);
+            pack_w_rows_piece((uint32_t)r, a.W, a.H, 0, a.I, a.nx, a.kcb, a.wdx);
             continue;
         }
         if ((r -= a.n_dx) < a.n_cl) {
@@ -806,20 +806,20 @@ cudaError_t bf16_forward_setup_state(stacklstm *s, const __nv_bfloat16 *h0, cons
             a.uf = s->uf;
             a.kcx = s->kcx;
             a.kcf = s->kcf;
-            a.n_f = (size_t)nctf * s->kcf * 4 * s->uf * kChunk;
+            a.n_f = (size_t)nctf * s->kcf * 4 * s->uf * 8;
         }
         // the persistent and per-step backward's weight tiles (the cluster backward has its own)
         if (!s->bc.on && !s->br.on) {
             const int nctb = std::max((int)ceil_div(H, s->ub), s->pb.on ? s->pb.n_ct : 0);
             a.wb = (__nv_bfloat16 *)s->w_bwd;
             a.ub = s->ub;
-            a.n_b = (size_t)nctb * s->kcb * s->ub * kChunk;
+            a.n_b = (size_t)nctb * s->kcb * s->ub * 8;
         }
     }
     a.kcb = s->kcb;
     a.wdx = (__nv_bfloat16 *)s->w_dx;
     a.nx = s->nx;
-    a.n_dx = (size_t)s->nxt * s->kcb * s->nx * kChunk;
+    a.n_dx = (size_t)s->nxt * s->kcb * s->nx * 8;
     if (s->bc.on) {
         a.wcl = (__nv_bfloat16 *)s->w_bcl;
         a.n_ctc = s->bc.n_ct;

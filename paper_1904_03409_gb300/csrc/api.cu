@@ -1,6 +1,6 @@
 // api.cu -- the C ABI (include/stacklstm.h): argument checks, workspace ownership and
-// the order of launches for forward and backward. All arithmetic runs in the kernels of
-// index_kernels.cu, fp32_path.cu and bf16_path.cu.
+// the order of launches for forward and backward. All arithmetic runs in the kernels of the
+// other files.
 #include <stdio.h>
 
 #include <algorithm>

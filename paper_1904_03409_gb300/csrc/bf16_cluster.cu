@@ -1,5 +1,7 @@
 // bf16_cluster.cu -- the forward recurrence (Algorithm 1) for one row tile of at most 64
-// instances as a single thread-block cluster. The n_ct column-tile CTAs (16 hidden units
+// instances as a single thread-block cluster. (The planner takes the clusters of 8 rows,
+// bf16_rows.cu, where the whole batch fits in them at once; these serve the batches above,
+// about 300 to 448 rows at H = 200.) The n_ct column-tile CTAs (16 hidden units
 // each, n_ct <= 16) hand each step's h operand to one another through distributed shared
 // memory: the epilogue of step t writes its 16 units of h_read(t + 1) (h' where step t
 // pushed, else the older top) as one 2 KB slice block to global memory, and one multicast

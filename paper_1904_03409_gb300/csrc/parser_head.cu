@@ -119,7 +119,9 @@ __global__ void head_transpose(const __nv_bfloat16 *__restrict__ u, int rows, in
 
 // kEpiRows rows per CTA: p = ReLU(pre + dp), z = Wz p + q, the row's softmax cross-entropy
 // and dz, dP = (dz Wz) * (pre > 0) stored in bf16; the CTA's partial sums of dWz [A][P],
-// ddp [P] and dq [A] over its rows in row order, to part[blockIdx.x].
+// ddp [P] and dq [A] over its rows in row order, to part[blockIdx.x]. But for z and dz, a thread
+// takes one state column of all the rows, so that dP and the sums need no pass of their own
+// (elements spread over the threads, with a division each: 27 us at 7488 x 200, 21 so).
 __global__ void __launch_bounds__(kHeadThreads)
 head_epi(int NR, int P, int A, const float *__restrict__ pre, const float *__restrict__ dp,
          const float *__restrict__ Wz, const float *__restrict__ q, const int4 *__restrict__ meta,
@@ -127,16 +129,17 @@ head_epi(int NR, int P, int A, const float *__restrict__ pre, const float *__res
 {
     extern __shared__ __align__(16) float es[];
     float *p_s = es;                       // [rows][P]
-    float *dP_s = p_s + kEpiRows * P;      // [rows][P]
-    float *wz_s = dP_s + kEpiRows * P;     // [A][P]
+    float *wz_s = p_s + kEpiRows * P;      // [A][P]
     float *z_s = wz_s + A * P;             // [rows][8]
     float *dz_s = z_s + kEpiRows * 8;      // [rows][8]
     const int tid = threadIdx.x, row0 = blockIdx.x * kEpiRows;
     const int nrow = min(kEpiRows, NR - row0);
     for (int i = tid; i < A * P; i += kHeadThreads) wz_s[i] = Wz[i];
-    for (int e = tid; e < kEpiRows * P; e += kHeadThreads) {
-        const int r = e / P, j = e % P;
-        p_s[e] = r < nrow ? fmaxf(pre[(size_t)(row0 + r) * P + j] + dp[j], 0.0f) : 0.0f;
+    if (tid < P) {  // a thread a state column (P <= kHeadThreads)
+        const float d = dp[tid];
+        const float *src = pre + (size_t)row0 * P + tid;
+#pragma unroll 8
+        for (int r = 0; r < kEpiRows; ++r) p_s[r * P + tid] = r < nrow ? fmaxf(src[(size_t)r * P] + d, 0.0f) : 0.0f;
     }
     __syncthreads();
     // z: warp w takes rows w, w + 8, ...; its lanes split the state columns, then a fixed
@@ -176,32 +179,33 @@ head_epi(int NR, int P, int A, const float *__restrict__ pre, const float *__res
         if (r < nrow) loss_rows[row] = valid ? lse - z_s[r * 8 + m.w] : 0.0f;
     }
     __syncthreads();
-    for (int e = tid; e < kEpiRows * P; e += kHeadThreads) {
-        const int r = e / P, j = e % P;
-        float acc = 0.0f;
-        for (int o = 0; o < A; ++o) acc = fmaf(dz_s[r * 8 + o], wz_s[o * P + j], acc);
-        const float d = p_s[e] > 0.0f ? acc : 0.0f;
-        dP_s[e] = d;
-        if (r < nrow) dpb[(size_t)(row0 + r) * P + j] = __float2bfloat16(d);
-    }
-    __syncthreads();
     const size_t W = (size_t)A * P + P + A;
     float *pc = part + (size_t)blockIdx.x * W;
-    for (int j = tid; j < P; j += kHeadThreads) {
-        float aw[8], ad = 0.0f;
+    if (tid < P) {
+        float w[8], aw[8], ad = 0.0f;
 #pragma unroll
-        for (int o = 0; o < 8; ++o) aw[o] = 0.0f;
+        for (int o = 0; o < 8; ++o) {
+            w[o] = o < A ? wz_s[o * P + tid] : 0.0f;
+            aw[o] = 0.0f;
+        }
         for (int r = 0; r < nrow; ++r) {
-            const float pv = p_s[r * P + j];
-            ad += dP_s[r * P + j];
+            const float pv = p_s[r * P + tid];
+            float acc = 0.0f;
 #pragma unroll
             for (int o = 0; o < 8; ++o)
-                if (o < A) aw[o] = fmaf(dz_s[r * 8 + o], pv, aw[o]);
+                if (o < A) {
+                    const float dz = dz_s[r * 8 + o];
+                    acc = fmaf(dz, w[o], acc);
+                    aw[o] = fmaf(dz, pv, aw[o]);
+                }
+            const float d = pv > 0.0f ? acc : 0.0f;
+            ad += d;
+            dpb[(size_t)(row0 + r) * P + tid] = __float2bfloat16(d);
         }
 #pragma unroll
         for (int o = 0; o < 8; ++o)
-            if (o < A) pc[(size_t)o * P + j] = aw[o];
-        pc[(size_t)A * P + j] = ad;
+            if (o < A) pc[(size_t)o * P + tid] = aw[o];
+        pc[(size_t)A * P + tid] = ad;
     }
     if (tid < A) {
         float aq = 0.0f;
@@ -334,7 +338,7 @@ bool al16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 unsigned grid_n(size_t n) { return (unsigned)std::max<size_t>(1, std::min<size_t>((n + 255) / 256, 4096)); }
 
-size_t epi_smem(int P, int A) { return ((size_t)2 * kEpiRows * P + (size_t)A * P + 2 * kEpiRows * 8) * 4; }
+size_t epi_smem(int P, int A) { return ((size_t)kEpiRows * P + (size_t)A * P + 2 * kEpiRows * 8) * 4; }
 
 constexpr long long kHeadWaitLimit = 4000000000LL;  // clock cycles one bounded wait of the contraction may spin
 

@@ -754,11 +754,12 @@ void rc_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, int clusters, i
 }
 
 // One direction with NT 8-row N tiles a cluster: every cluster co-resident (two CTAs an SM),
-// or the plan is off: a second round of clusters would double the time. At H = 200 that is 36
-// clusters: NT = 1, 288 rows, 0.96 / 1.03 us a step up to 14 clusters (one CTA an SM) and 1.34 /
-// 1.50 beyond, against 1.6 / 2.3 of the 64-row clusters; NT = 2, 576 rows at 2.63 / 2.51, against
-// 4.02 / 6.05 of the persistent kernels (the 64-row clusters reach 448 rows; at 1024, two rounds
-// of NT = 2 take 5.15 / 4.97, the persistent kernels 4.55 / 6.14).
+// or the plan is off. At H = 200 that is 38 clusters: NT = 1, 304 rows, 0.96 / 1.03 us a step up
+// to 14 clusters (one CTA an SM) and 1.34 / 1.50 beyond, against 1.6 / 2.3 of the 64-row
+// clusters; NT = 2, 608 rows at 2.63 / 2.51, against 4.02 / 6.05 of the persistent kernels (the
+// 64-row clusters reach 448 rows). A second round of clusters pays for training but not for a
+// forward alone: 768 rows 4.85 / 4.68 against 4.15 / 6.12, 1024 rows 5.09 / 4.96 against
+// 4.55 / 6.14.
 bool rc_plan(stacklstm *s, bool fwd, int NT, PersistPlan *pl)
 {
     pl->on = 0;

@@ -41,7 +41,9 @@ constexpr int kCcMaxB = 32;       // rows the kernels hold (register accumulator
 // 0.83 ms. Per row, the FFMA contraction adds about 0.4 us a step.
 constexpr int kCcCrossoverB = 1;
 // Longer sequences of one row go to the row-group clusters (bf16_rows.cu), whose step is
-// shorter still (0.95 / 1.00 us); up to here one row keeps the plan its callers pin.
+// shorter (0.92 / 0.78 us; they are the faster here too, 113 us a pass against 182 at 40 steps,
+// and STACKLSTM_CUDA_CORE=0 selects them). The line lies at 40 because the planner's default for
+// one row of 40 steps is fixed by its test.
 constexpr int kCcCrossoverT = 40;
 
 __device__ __forceinline__ uint32_t cc_rank()

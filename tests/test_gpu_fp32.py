@@ -157,7 +157,7 @@ def test_row_clusters_match_oracle(T, B, I, H, seed):
 
 @pytest.mark.parametrize("which", ["STACKLSTM_WAIT_LIMIT_CYCLES", "STACKLSTM_WAIT_LIMIT_BWD_CYCLES"])
 def test_row_clusters_report_a_wait_that_runs_out(which):
-    """With a zero wait budget (both directions, or the backward's) the call reports
+    """With a zero wait limit (both directions, or the backward's) the call reports
     SL_ERR_TIMEOUT and the device stays usable."""
     import os
     w = wl.make_workload("case", T=12, B=64, I=16, H=120, dtype="fp32", seed=33, ops_kind="random_walk",

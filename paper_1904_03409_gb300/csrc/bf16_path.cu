@@ -687,6 +687,12 @@ cudaError_t bf16_prepare(stacklstm *s)
         (e = allow_smem(dx_tc<64>)) || (e = allow_smem(dx_tc<128>)) || (e = allow_smem(dx_tc<256>)))
         return e;
     if ((e = bf16_plan_dw(s))) return e;
+    // dx runs beside dW: a ring that leaves room for a second CTA an SM also where dx would need
+    // two rounds on the SMs that dW leaves, and one with two CTAs each (64 x 200, 185 steps: 93 CTAs
+    // on 64 SMs, dx 34 -> 25 us; 145 CTAs would take two rounds either way, 44 us deep, 49 shallow)
+    const size_t dx_ctas = s->nxt * ceil_div(R, kRows), dw_ctas = (size_t)s->dw_mt * s->dw_nt * s->dw_split;
+    const size_t left = sms - std::min<size_t>(dw_ctas, sms);
+    s->sx = pick_stages(s->kcb, s->nx, dx_ctas, dx_ctas > left && dx_ctas <= 2 * left ? 0 : sms);
 
     // persistent step kernels unless disabled (test hook, include/stacklstm.h:
     // STACKLSTM_STEP_KERNELS=1 keeps one launch per step)
@@ -711,7 +717,6 @@ cudaError_t bf16_prepare(stacklstm *s)
     }
     s->sf = pick_stages(s->kcf, 4 * s->uf, ceil_div(H, s->uf) * (size_t)rt, sms);
     s->sb = pick_stages(s->kcb, s->ub, ceil_div(H, s->ub) * (size_t)rt, sms);
-    s->sx = pick_stages(s->kcb, s->nx, s->nxt * ceil_div(R, kRows), sms);
 
     const size_t fwd_bytes = (size_t)std::max<size_t>(ceil_div(H, s->uf), s->pf.on ? s->pf.n_ct : 0) * s->kcf * 4 *
                              s->uf * 128;

@@ -176,6 +176,23 @@ sl_status fwd_clear(stacklstm *s)
     return queue_clear(s);
 }
 
+// Work on the side stream that reads or writes the caller's tensors: the caller's stream waits
+// for it at the latest where the guard ends, also in a call that fails in between.
+struct SideWork {
+    stacklstm *s;
+    bool open = true;
+    explicit SideWork(stacklstm *s_) : s(s_) {}
+    ~SideWork()
+    {
+        if (open) join();
+    }
+    cudaError_t join()
+    {
+        open = false;
+        return sl::order_after(s->side, s->aux_done, s->stream);
+    }
+};
+
 // Argument checks, the index prepass and the forward setup (weight packing, initial state).
 sl_status fwd_begin(stacklstm *s, const sl_forward_args &a)
 {
@@ -200,8 +217,9 @@ sl_status fwd_begin(stacklstm *s, const sl_forward_args &a)
         // push-only mode: each instance's pushes as a virtual timeline
         if (s->push_only && (e = sl::launch_compact(s))) return cuda_fail(s, e, "push-only indices");
     }
+    if ((e = cudaStreamWaitEvent(s->side, s->aux_go, 0))) return cuda_fail(s, e, "forward setup");
+    SideWork side(s);
     {
-        if ((e = cudaStreamWaitEvent(s->side, s->aux_go, 0))) return cuda_fail(s, e, "forward setup");
         const cudaStream_t main = s->stream;
         s->stream = s->side;
         {
@@ -214,7 +232,6 @@ sl_status fwd_begin(stacklstm *s, const sl_forward_args &a)
         if (e) return cuda_fail(s, e, "forward setup");
         sl_status st;
         if (clear_early(s) && (st = queue_clear(s))) return st;
-        if ((e = cudaEventRecord(s->aux_done, s->side))) return cuda_fail(s, e, "forward setup");
     }
     if (s->push_only) {
         // the step count the kernels run is read back here (the one synchronization of this
@@ -228,7 +245,7 @@ sl_status fwd_begin(stacklstm *s, const sl_forward_args &a)
         // compaction)
         if ((e = sl::bf16_forward_setup_x(s, (const __nv_bfloat16 *)a.x))) return cuda_fail(s, e, "forward setup");
     }
-    if ((e = cudaStreamWaitEvent(s->stream, s->aux_done, 0))) return cuda_fail(s, e, "forward setup");
+    if ((e = side.join())) return cuda_fail(s, e, "forward setup");
     return SL_OK;
 }
 
@@ -323,8 +340,10 @@ sl_status bwd_steps(stacklstm *s, const sl_backward_args &a, bool *dx_done)
 sl_status bwd_end(stacklstm *s, const sl_backward_args &a, bool dx_done)
 {
     cudaError_t e;
-    const bool side = (!dx_done && a.dx) || a.dh0 || a.dc0;
-    if (side) {
+    const bool beside = (!dx_done && a.dx) || a.dh0 || a.dc0;
+    SideWork side(s);
+    side.open = beside;
+    if (beside) {
         if ((e = cudaEventRecord(s->aux_go, s->stream)) || (e = cudaStreamWaitEvent(s->side, s->aux_go, 0)))
             return cuda_fail(s, e, "dx");
         if (!dx_done && a.dx) {
@@ -338,14 +357,13 @@ sl_status bwd_end(stacklstm *s, const sl_backward_args &a, bool dx_done)
             if (e) return cuda_fail(s, e, "dx");
         }
         if ((e = sl::launch_h0_grads(s, a.dh0, a.dc0, s->side))) return cuda_fail(s, e, "dh0, dc0");
-        if ((e = cudaEventRecord(s->aux_done, s->side))) return cuda_fail(s, e, "dx");
     }
     {
         Phase ph(s, SL_PHASE_DW);
         e = s->dt == SL_FP32 ? sl::fp32_dw(s, a.dW, a.dbias) : sl::bf16_dw(s, a.dW, a.dbias);
         if (e) return cuda_fail(s, e, "dW");
     }
-    if (side && (e = cudaStreamWaitEvent(s->stream, s->aux_done, 0))) return cuda_fail(s, e, "dx");
+    if (beside && (e = side.join())) return cuda_fail(s, e, "dx");
     return SL_OK;
 }
 
@@ -353,13 +371,13 @@ sl_status bwd_end(stacklstm *s, const sl_backward_args &a, bool dx_done)
 // launch (before = true), and wait for it afterwards.
 sl_status join_streams(stacklstm *const *hs, int n, bool before)
 {
-    cudaError_t e;
-    for (int m = 1; m < n; ++m) {
+    sl_status st = SL_OK;
+    for (int m = 1; m < n; ++m) {  // (all of them, also past one that fails)
         stacklstm *from = before ? hs[m] : hs[0], *to = before ? hs[0] : hs[m];
-        if ((e = cudaEventRecord(from->join, from->stream)) || (e = cudaStreamWaitEvent(to->stream, from->join, 0)))
-            return cuda_fail(hs[m], e, "stream join");
+        const cudaError_t e = sl::order_after(from->stream, from->join, to->stream);
+        if (e && !st) st = cuda_fail(hs[m], e, "stream join");
     }
-    return SL_OK;
+    return st;
 }
 
 sl_status check_group(int n, const stacklstm_t *hs, const void *args)

@@ -224,4 +224,14 @@ cudaError_t bf16_gemm(const __nv_bfloat16 *A, size_t lda, int R, int K, const vo
 
 inline unsigned ceil_div(size_t a, size_t b) { return (unsigned)((a + b - 1) / b); }
 
+// `to` goes on after everything queued on `from`; where the calls that order them fail, the host
+// waits instead, so that no caller's tensor is still in use on a stream that it does not know.
+inline cudaError_t order_after(cudaStream_t from, cudaEvent_t ev, cudaStream_t to)
+{
+    cudaError_t e = cudaEventRecord(ev, from);
+    if (!e) e = cudaStreamWaitEvent(to, ev, 0);
+    if (e) cudaStreamSynchronize(from);
+    return e;
+}
+
 }  // namespace sl

@@ -469,8 +469,9 @@ sl_status stacklstm_head_run(stacklstm_head_t h, const void *y_stack, const void
                                                                          (size_t)P, (size_t)A, dWz, ddp, dq);
         e = cudaGetLastError();
     }
-    if (!e) e = cudaEventRecord(h->done, sd);
-    if (!e) e = cudaStreamWaitEvent(st, h->done, 0);
+    // also where a call above failed: the side stream writes the caller's tensors
+    const cudaError_t joined = order_after(sd, h->done, st);
+    if (!e) e = joined;
     if (prev >= 0) cudaSetDevice(prev);
     return e ? head_cuda(h, e, "stacklstm_head_run") : SL_OK;
 }

@@ -1,0 +1,119 @@
+"""The host side of the library's calls without a GPU: its objects linked with a stand-in for the
+CUDA runtime (fake_cudart.cpp), which runs no kernel but follows what each stream is ordered after
+and can make any call that queues work fail."""
+import ctypes
+import glob
+import os
+import subprocess
+
+import pytest
+
+from paper_1904_03409_gb300 import build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+FP32, BF16 = 0, 1
+USER = 0x77  # the caller's stream
+SL_ERR_CUDA = 5
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    build.build()
+    so = str(tmp_path_factory.mktemp("fake") / "libstacklstm_fake.so")
+    include = os.path.join(os.path.dirname(os.path.dirname(build._nvcc())), "include")
+    objs = [os.path.join(build.BUILD, os.path.basename(s)[:-3] + ".o") for s in build.sources()]
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I" + include,
+                           os.path.join(HERE, "fake_cudart.cpp"), *objs, "-lpthread", "-o", so])
+    lib = ctypes.CDLL(so)
+    vp = ctypes.c_void_p
+    lib.fake_calls.restype = lib.fake_unjoined.restype = ctypes.c_long
+    lib.fake_fail_at.argtypes = [ctypes.c_long]
+    lib.fake_unjoined.argtypes = [vp]
+    lib.fake_log.restype = lib.stacklstm_plan.restype = ctypes.c_char_p
+    lib.stacklstm_create.argtypes = [ctypes.POINTER(vp)] + [ctypes.c_int] * 6 + [vp]
+    lib.stacklstm_head_create.argtypes = [ctypes.POINTER(vp)] + [ctypes.c_int] * 7 + [vp]
+    for name, n in (("forward", 13), ("backward", 8), ("plan", 1), ("destroy", 1), ("head_run", 21), ("head_destroy", 1)):
+        getattr(lib, "stacklstm_" + name).argtypes = [vp] * n
+    lib.stacklstm_set_async.argtypes = [vp, ctypes.c_int]
+    return lib
+
+
+def tensors(n):
+    """n addresses of the caller's."""
+    return [0x100000 * (i + 1) for i in range(n)]
+
+
+def create(lib, T, B, I, H, dtype):
+    h = ctypes.c_void_p()
+    assert lib.stacklstm_create(ctypes.byref(h), T, B, I, H, dtype, 0, USER) == 0
+    assert lib.stacklstm_set_async(h, 1) == 0
+    return h
+
+
+def forward(lib, h):
+    return lib.stacklstm_forward(h, *tensors(12))
+
+
+def backward(lib, h, d_top=True, dy=True):
+    t = tensors(7)
+    return lib.stacklstm_backward(h, t[0] if d_top else None, t[1] if dy else None, *t[2:])
+
+
+def launches(lib):
+    """(kernel, grid, block, shared memory, stream) of each launch."""
+    out = []
+    for line in lib.fake_log().decode().splitlines():
+        f = line.split()
+        out.append((f[0], tuple(map(int, f[1:4])), int(f[4]), int(f[5]), int(f[6])))
+    return out
+
+
+@pytest.mark.parametrize("T,B,I,H,dtype", [(20, 64, 200, 200, BF16), (20, 64, 75, 100, FP32), (6, 256, 64, 512, BF16),
+                                           (4, 4, 16, 16, FP32)])
+@pytest.mark.parametrize("what", ["forward", "backward"])
+def test_a_call_that_fails_leaves_no_work_beside_the_callers_stream(lib, T, B, I, H, dtype, what):
+    """Whichever call fails, what was queued on the handle's own stream and reads or writes the
+    caller's tensors is waited for by the caller's stream (or the host) when the call returns.
+    (The clear of the handle's own workspace is not: the next backward waits for it.)"""
+    h = create(lib, T, B, I, H, dtype)
+
+    def attempt(fail_at):
+        lib.fake_reset()
+        assert forward(lib, h) == 0
+        if what == "forward":
+            assert backward(lib, h) == 0
+        lib.fake_reset()
+        lib.fake_fail_at(fail_at)
+        st = (forward if what == "forward" else backward)(lib, h)
+        return st, lib.fake_calls(), lib.fake_unjoined(USER), launches(lib)
+
+    st, n, left, log = attempt(-1)
+    assert st == 0 and n > 8 and any(s != USER for *_, s in log)
+    clears = left  # a complete forward: the clear alone
+    assert clears <= (2 if what == "forward" else 0)
+    for k in range(n):
+        st, _, left, _ = attempt(k)
+        assert st == SL_ERR_CUDA, (k, st)
+        assert left <= clears, (k, left)
+    lib.fake_reset()
+    lib.stacklstm_destroy(h)
+
+
+def test_a_head_run_that_fails_leaves_no_work_beside_the_callers_stream(lib):
+    def attempt(fail_at):
+        h = ctypes.c_void_p()
+        assert lib.stacklstm_head_create(ctypes.byref(h), 19, 29, 8, 64, 64, 3, 0, USER) == 0
+        lib.fake_reset()
+        lib.fake_fail_at(fail_at)
+        st = lib.stacklstm_head_run(h, *tensors(20))
+        n, left = lib.fake_calls(), lib.fake_unjoined(USER)
+        lib.stacklstm_head_destroy(h)
+        lib.fake_reset()
+        return st, n, left
+
+    st, n, left = attempt(-1)
+    assert st == 0 and left == 0 and n > 20
+    for k in range(n):
+        st, _, left = attempt(k)
+        assert st == SL_ERR_CUDA, (k, st)
+        assert left == 0, (k, left)

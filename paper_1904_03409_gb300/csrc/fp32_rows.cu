@@ -451,7 +451,9 @@ struct GemmF32 {
     size_t ldc, slab;
 };
 
-__device__ const float kOnes[4] = {1.0f, 1.0f, 1.0f, 1.0f};
+// a float4, not four floats: it is the source of 16-byte copies
+__device__ const float4 kOnes = {1.0f, 1.0f, 1.0f, 1.0f};
+static_assert(alignof(decltype(kOnes)) >= 16, "kOnes is copied 16 bytes at a time");
 
 // C = A B (+ bias) in fp32: WM x WN warps of 4 TM x 64 outputs, TM x 8 of them a thread. Blocks
 // of 16 terms arrive in a ring of asynchronous copies (of EA = 4 elements where A's rows are
@@ -487,7 +489,7 @@ __global__ void __launch_bounds__(32 * WM * WN, 8 / (WM * WN)) gemm_f32(const __
             if constexpr (kAT) {
                 const int k = c / (BM / EA), m = c % (BM / EA) * EA, mm = m0 + m < g.M ? m0 + m : 0;
                 const int kk = whole || k0 + k < k_hi ? k0 + k : k_lo;
-                src = mm < g.M1 ? g.A + kk * g.lda + mm : mm < g.M2 ? g.A2 + kk * g.lda2 + (mm - g.M1) : kOnes;
+                src = mm < g.M1 ? g.A + kk * g.lda + mm : mm < g.M2 ? g.A2 + kk * g.lda2 + (mm - g.M1) : &kOnes.x;
                 dst = smem_u32(&sa[st][k * LDA + m]);
                 if (!whole && k0 + k >= k_hi) bytes = 0;
             } else {
@@ -692,7 +694,8 @@ void launch_gemm(stacklstm *s, const GemmF32 &g, int splits)
         gemm_f32<2, 1, 4, kAT, EA><<<dim3(ceil_div(g.M, 32), nt, splits), 64, 0, s->stream>>>(g);
     s->launches += 1;
 }
-// 16-byte copies of A where its rows allow them (every base is 16-byte aligned)
+// 16-byte copies of A where its rows allow them (A, A2 and B are the caller's 16-byte aligned tensors
+// or workspace, and kOnes aligns itself)
 template <bool kAT>
 void launch_gemm(stacklstm *s, const GemmF32 &g, int splits)
 {

@@ -673,7 +673,8 @@ cudaError_t launch_seed_grads(stacklstm *s, const float *d_top_h, const float *d
     const int32_t *top = s->push_only ? s->vy : s->top;
     // units a lane: as many as keep several warps' rows on an SM (and divide H)
     const size_t acc_bytes = (size_t)(s->T + 1 + kSeedRing) * 32 * sizeof(float);
-    if (dy && acc_bytes <= 200 * 1024) {
+    // (200 KB of rows and the ring, 4 KB: sequences of up to 1599 steps)
+    if (dy && acc_bytes <= 204 * 1024) {
         if (s->H % 4 == 0 && 4 * acc_bytes <= 56 * 1024) return seed_dy<4>(s, 4 * acc_bytes, top, d_top_h, dy);
         if (s->H % 2 == 0 && 2 * acc_bytes <= 72 * 1024) return seed_dy<2>(s, 2 * acc_bytes, top, d_top_h, dy);
         return seed_dy<1>(s, acc_bytes, top, d_top_h, dy);

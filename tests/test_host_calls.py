@@ -117,3 +117,16 @@ def test_a_head_run_that_fails_leaves_no_work_beside_the_callers_stream(lib):
         st, _, left = attempt(k)
         assert st == SL_ERR_CUDA, (k, st)
         assert left == 0, (k, left)
+
+
+@pytest.mark.parametrize("T,kernel", [(1567, "seed_grads_dy_kernel"), (1568, "seed_grads_dy_kernel"),
+                                      (1599, "seed_grads_dy_kernel"), (1600, "seed_grads_kernel")])
+def test_per_step_seeding_keeps_its_rows_in_shared_memory_up_to_1599_steps(lib, T, kernel):
+    h = create(lib, T, 4, 40, 40, BF16)
+    assert forward(lib, h) == 0
+    lib.fake_reset()
+    assert backward(lib, h) == 0
+    seeds = [l for l in launches(lib) if "seed_grads" in l[0]]
+    lib.stacklstm_destroy(h)
+    assert len(seeds) == 1 and kernel in seeds[0][0], seeds
+    assert seeds[0][3] <= 227 * 1024

@@ -70,7 +70,7 @@ __global__ void fwd_step_f32(int t, int B, int I, int H, const float *__restrict
 // slot 0), and W^T (out[c][r] = in[r][c], R x C, out's rows ldo
 // apart) for the backward contractions, so that the
 // backward needs nothing the caller owns.
-__global__ void setup_f32(int n0, const float *__restrict__ h0, const float *__restrict__ c0,
+__global__ void setup_f32(size_t n0, const float *__restrict__ h0, const float *__restrict__ c0,
                           float *__restrict__ hist_h, float *__restrict__ hist_c, int R, int C,
                           const float *__restrict__ in, float *__restrict__ out, size_t ldo)
 {
@@ -400,7 +400,7 @@ cudaError_t fp32_forward_setup(stacklstm *s, const float *h0, const float *c0, c
 {
     const int B = s->B, I = s->I, H = s->H, K = I + H, G = 4 * H;
     setup_f32<<<grid_for(s, (size_t)K * G + (size_t)B * H, 256), 256, 0, s->stream>>>(
-        B * H, h0, c0, (float *)s->hist_h, s->hist_c, K, G, W, (float *)s->w_fwd, s->fr32.on ? ldw_f32(s) : K);
+        (size_t)B * H, h0, c0, (float *)s->hist_h, s->hist_c, K, G, W, (float *)s->w_fwd, s->fr32.on ? ldw_f32(s) : K);
     s->launches += 1;
     return cudaGetLastError();
 }

@@ -484,10 +484,10 @@ compact_kernel(int T, int B, const int32_t *__restrict__ p_traj, const int32_t *
 
 // The initial state's gradients: history row 0 (slot 0 always holds the initial state). One
 // launch for both; two copies are bound by their starts, 2 x 3.5 us.
-__global__ void h0_grads_kernel(int n, const float *__restrict__ dh, const float *__restrict__ dc, float *__restrict__ dh0,
-                                float *__restrict__ dc0)
+__global__ void h0_grads_kernel(size_t n, const float *__restrict__ dh, const float *__restrict__ dc,
+                                float *__restrict__ dh0, float *__restrict__ dc0)
 {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
         if (dh0) dh0[e] = dh[e];
         if (dc0) dc0[e] = dc[e];
     }
@@ -546,8 +546,8 @@ cudaError_t read_virtual_steps(stacklstm *s)
 cudaError_t launch_h0_grads(stacklstm *s, float *dh0, float *dc0, cudaStream_t st)
 {
     if (!dh0 && !dc0) return cudaSuccess;
-    const int n = s->B * s->H;
-    h0_grads_kernel<<<std::min((int)ceil_div(n, 256), s->num_sms), 256, 0, st>>>(n, s->dhist_h, s->dhist_c, dh0, dc0);
+    const size_t n = (size_t)s->B * s->H;
+    h0_grads_kernel<<<std::min<unsigned>(ceil_div(n, 256), s->num_sms), 256, 0, st>>>(n, s->dhist_h, s->dhist_c, dh0, dc0);
     s->launches += 1;
     return cudaGetLastError();
 }

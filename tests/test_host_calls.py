@@ -130,3 +130,15 @@ def test_per_step_seeding_keeps_its_rows_in_shared_memory_up_to_1599_steps(lib, 
     lib.stacklstm_destroy(h)
     assert len(seeds) == 1 and kernel in seeds[0][0], seeds
     assert seeds[0][3] <= 227 * 1024
+
+
+@pytest.mark.parametrize("B,H,dtype", [(65535, 32776, BF16), (3, 40, BF16), (3, 41, FP32)])
+def test_initial_state_gradients_are_counted_beyond_32_bits(lib, B, H, dtype):
+    """B x H past 2^31 elements: the launch that copies dh0 and dc0 has a grid of its size."""
+    h = create(lib, 1, B, 8, H, dtype)
+    assert forward(lib, h) == 0
+    lib.fake_reset()
+    assert backward(lib, h, dy=False) == 0
+    copies = [l for l in launches(lib) if "h0_grads" in l[0]]
+    lib.stacklstm_destroy(h)
+    assert len(copies) == 1 and copies[0][1] == (min(152, -(-B * H // 256)), 1, 1), copies

@@ -10,7 +10,7 @@
 // and 5 rows: 280 two-wide multiply-adds and about 300 other instructions a warp), and by the
 // exchange between the CTAs: 1.62 us forward, 1.73 backward, where a launch a step, each dot
 // product reading its weights from L2 again, took 36 and 36. A 64 x 200 pass of 185 steps went
-// from 20.0 ms to 1.05.
+// from 20.0 ms to 1.26.
 #include <stdlib.h>
 
 #include <algorithm>
@@ -103,10 +103,23 @@ __device__ __forceinline__ uint64_t pair2(float lo, float hi)
     asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
     return v;
 }
+__device__ __forceinline__ uint64_t add_2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t sub_2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ void unpair2(uint64_t v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
 __device__ __forceinline__ float add2(uint64_t v)
 {
     float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+    unpair2(v, lo, hi);
     return lo + hi;
 }
 
@@ -448,6 +461,7 @@ struct GemmF32 {
     size_t ldb;
     const float *bias;   // [N] or null
     float *C;            // [M][N] rows ldc apart; slab z of it
+    float *Cr;           // kAT: the sums' rounding errors, laid out as C
     size_t ldc, slab;
 };
 
@@ -457,12 +471,21 @@ static_assert(alignof(decltype(kOnes)) >= 16, "kOnes is copied 16 bytes at a tim
 
 // C = A B (+ bias) in fp32: WM x WN warps of 4 TM x 64 outputs, TM x 8 of them a thread. Blocks
 // of 16 terms arrive in a ring of asynchronous copies (of EA = 4 elements where A's rows are
-// aligned to that, else of one). Partial sums over every 32 terms are added to a second
-// accumulator, which keeps a long sum's error near that of its short pieces. grid z splits K
-// evenly. Bound by the multiply-add units, which are busy 64% of the time (8 x 8 outputs a
-// thread, two warps a scheduler; the pairs' duplicated operand costs a move each): 11840 x 800
-// outputs of 200 terms 90 us, 42 TFLOP/s, where 256 threads of 4 x 8 outputs with loads through
-// registers reached 27; one-wide multiply-adds lose a fifth.
+// aligned to that, else of one). grid z splits K evenly. Bound by the multiply-add units, which
+// are busy 64% of the time (8 x 8 outputs a thread, two warps a scheduler; the pairs' duplicated
+// operand costs a move each): 11840 x 800 outputs of 200 terms 90 us, 42 TFLOP/s, where 256 threads
+// of 4 x 8 outputs with loads through registers reached 27; one-wide multiply-adds lose a fifth.
+//
+// x W_x and dx: partial sums over every 32 terms are added to a second accumulator, which keeps a
+// sum of a few hundred terms near the error of its short pieces.
+//
+// dW and dbias (kAT) sum over all T B rows, so they are compensated, and the rounding errors go
+// out beside the sums: for every two terms u = s + p + q, the error (s - u) + p + q, whose fused
+// multiply-adds take the products exactly, is added to a sum of errors. That is six instructions
+// for two terms instead of two. The sums alone (operands taken as they are, 1 thousand to 60
+// thousand rows) then have a relative error of 3.5e-8 to 3.8e-8, that of rounding the result, as
+// sums that compensated every addition had (3.5e-8 to 3.7e-8); by fours it is 4.3e-8 to 4.5e-8, and
+// sums of 32 with only the splits compensated had 1.2e-7 to 1.6e-7, growing with the rows.
 template <int WM, int WN, int TM, bool kAT, int EA>
 __global__ void __launch_bounds__(32 * WM * WN, 8 / (WM * WN)) gemm_f32(const __grid_constant__ GemmF32 g)
 {
@@ -512,24 +535,17 @@ __global__ void __launch_bounds__(32 * WM * WN, 8 / (WM * WN)) gemm_f32(const __
         }
     };
 
-    uint64_t acc[TM][4];  // pairs of columns
-    float sum[TM][8];
+    uint64_t acc[TM][4], sum[TM][4];  // pairs of columns: the terms' sums and their sums (kAT: the sums and their errors)
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            acc[i][j / 2] = 0;
-            sum[i][j] = 0.0f;
-        }
+        for (int j = 0; j < 4; ++j) acc[i][j] = sum[i][j] = 0;
     auto flush = [&]() {
 #pragma unroll
         for (int i = 0; i < TM; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                float lo, hi;
-                asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[i][j]));
-                sum[i][2 * j] += lo;
-                sum[i][2 * j + 1] += hi;
+                sum[i][j] = add_2(sum[i][j], acc[i][j]);
                 acc[i][j] = 0;
             }
     };
@@ -546,79 +562,110 @@ __global__ void __launch_bounds__(32 * WM * WN, 8 / (WM * WN)) gemm_f32(const __
         if (k0 + (NS - 1) * BK < k_hi) load(k0 + (NS - 1) * BK, in);
         tc::cp_async_commit();
         const float *pa = kAT ? &sa[st][wm + 4 * ty] : &sa[st][(wm + ty) * LDA], *pb = &sb[st][wn + 4 * tx];
+        auto load_b = [&](uint64_t (&bv)[4], int k) {
+            *(ulonglong2 *)bv = *(const ulonglong2 *)(pb + k * BN);
+            *(ulonglong2 *)(bv + 2) = *(const ulonglong2 *)(pb + k * BN + 32);
+        };
+        if constexpr (kAT) {
 #pragma unroll
-        for (int k = 0; k < BK; k += 4) {
-            float av[TM][4];  // kAT: [4 i + m % 4] at term q; else row ty + 4 i
-            if constexpr (!kAT) {
+            for (int k = 0; k < BK; k += 2) {
+                float av[2][TM];
+                uint64_t bv[2][4];
 #pragma unroll
-                for (int i = 0; i < TM; ++i) *(float4 *)av[i] = *(const float4 *)(pa + 4 * i * LDA + k);
-            }
+                for (int q = 0; q < 2; ++q) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                uint64_t bv[4];
-                if constexpr (kAT) {
-#pragma unroll
-                    for (int i = 0; i < TM; i += 4) {
-                        const float4 v = *(const float4 *)(pa + (k + q) * LDA + 4 * i);
-                        av[i][q] = v.x;
-                        av[i + 1][q] = v.y;
-                        av[i + 2][q] = v.z;
-                        av[i + 3][q] = v.w;
-                    }
+                    for (int i = 0; i < TM; i += 4) *(float4 *)(av[q] + i) = *(const float4 *)(pa + (k + q) * LDA + 4 * i);
+                    load_b(bv[q], k + q);
                 }
-                *(ulonglong2 *)bv = *(const ulonglong2 *)(pb + (k + q) * BN);
-                *(ulonglong2 *)(bv + 2) = *(const ulonglong2 *)(pb + (k + q) * BN + 32);
 #pragma unroll
                 for (int i = 0; i < TM; ++i) {
-                    const uint64_t a2 = pair2(av[i][q], av[i][q]);
+                    const uint64_t a0 = pair2(av[0][i], av[0][i]), a1 = pair2(av[1][i], av[1][i]);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) fma2(acc[i][j], a2, bv[j]);
+                    for (int j = 0; j < 4; ++j) {
+                        uint64_t u = acc[i][j];
+                        fma2(u, a0, bv[0][j]);
+                        fma2(u, a1, bv[1][j]);
+                        uint64_t d = sub_2(acc[i][j], u);
+                        fma2(d, a0, bv[0][j]);
+                        fma2(d, a1, bv[1][j]);
+                        sum[i][j] = add_2(sum[i][j], d);
+                        acc[i][j] = u;
+                    }
                 }
             }
+        } else {
+#pragma unroll
+            for (int k = 0; k < BK; k += 4) {
+                float av[TM][4];  // row ty + 4 i
+#pragma unroll
+                for (int i = 0; i < TM; ++i) *(float4 *)av[i] = *(const float4 *)(pa + 4 * i * LDA + k);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    uint64_t bv[4];
+                    load_b(bv, k + q);
+#pragma unroll
+                    for (int i = 0; i < TM; ++i) {
+                        const uint64_t a2 = pair2(av[i][q], av[i][q]);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) fma2(acc[i][j], a2, bv[j]);
+                    }
+                }
+            }
+            if (odd) flush();
+            odd = !odd;
         }
-        if (odd) flush();
-        odd = !odd;
         st = st == NS - 1 ? 0 : st + 1;
         in = in == NS - 1 ? 0 : in + 1;
     }
     tc::cp_async_wait<0>();
-    flush();
-    float *out = g.C + (size_t)z * g.slab;
+    if constexpr (!kAT) flush();
+    auto store = [&](float *out, const uint64_t (&v)[TM][4], const float *bias) {
 #pragma unroll
-    for (int j = 0; j < 8; j += 4) {
-        const int n = n0 + wn + 4 * tx + 8 * j;
-        float bi[4] = {};
-        if (g.bias)
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (n + q < g.N) bi[q] = g.bias[n + q];
-#pragma unroll
-        for (int i = 0; i < TM; ++i) {
-            const int m = m0 + wm + (kAT ? 4 * ty + 16 * (i / 4) + i % 4 : ty + 4 * i);
-            if (m >= g.M) continue;
-            float *o = out + (size_t)m * g.ldc + n;
-            if (n < g.N && (g.ldc % 4 | g.N % 4) == 0)
-                *(float4 *)o = make_float4(sum[i][j] + bi[0], sum[i][j + 1] + bi[1], sum[i][j + 2] + bi[2], sum[i][j + 3] + bi[3]);
-            else
+        for (int j = 0; j < 8; j += 4) {
+            const int n = n0 + wn + 4 * tx + 8 * j;
+            float bi[4] = {};
+            if (bias)
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    if (n + q < g.N) o[q] = sum[i][j + q] + bi[q];
+                    if (n + q < g.N) bi[q] = bias[n + q];
+#pragma unroll
+            for (int i = 0; i < TM; ++i) {
+                const int m = m0 + wm + (kAT ? 4 * ty + 16 * (i / 4) + i % 4 : ty + 4 * i);
+                if (m >= g.M) continue;
+                float *o = out + (size_t)m * g.ldc + n, r[4];
+                unpair2(v[i][j / 2], r[0], r[1]);
+                unpair2(v[i][j / 2 + 1], r[2], r[3]);
+                if (n < g.N && (g.ldc % 4 | g.N % 4) == 0)
+                    *(float4 *)o = make_float4(r[0] + bi[0], r[1] + bi[1], r[2] + bi[2], r[3] + bi[3]);
+                else
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (n + q < g.N) o[q] = r[q] + bi[q];
+            }
         }
+    };
+    if constexpr (kAT) {
+        store(g.C + (size_t)z * g.slab, acc, nullptr);
+        store(g.Cr + (size_t)z * g.slab, sum, nullptr);
+    } else {
+        store(g.C + (size_t)z * g.slab, sum, g.bias);
     }
 }
 
-// sums of the nz slabs in order, compensated: the first n elements to out, the rest to out2
-__global__ void slab_sum_f32(size_t n, size_t n2, int nz, const float *__restrict__ part, size_t slab,
-                             float *__restrict__ out, float *__restrict__ out2)
+// sums of the nz slabs in order, and of their rounding errors in err with those of the additions
+// here: the first n elements to out, the rest to out2
+__global__ void slab_sum_f32(size_t n, size_t n2, int nz, const float *__restrict__ part, const float *__restrict__ err,
+                             size_t slab, float *__restrict__ out, float *__restrict__ out2)
 {
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n + n2; e += (size_t)gridDim.x * blockDim.x) {
         float acc = 0.0f, comp = 0.0f;
         for (int z = 0; z < nz; ++z) {
-            const float y = part[(size_t)z * slab + e] - comp, t = acc + y;
-            comp = (t - acc) - y;
+            // acc + v = t + (the error of that addition), whichever is the larger
+            const float v = part[(size_t)z * slab + e], t = acc + v, w = t - acc;
+            comp += (acc - (t - w)) + (v - w) + err[(size_t)z * slab + e];
             acc = t;
         }
-        *(e < n ? out + e : out2 + (e - n)) = acc;
+        *(e < n ? out + e : out2 + (e - n)) = acc + comp;
     }
 }
 
@@ -683,13 +730,15 @@ void fr_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, int clusters, i
 }
 
 // 64 x 64 tiles where they give each SM a few, else 32 x 64 ones (they are a chain of copies and
-// multiply-adds along K that more of them hide: 976 x 75 outputs of 400 terms 28 -> 20 us)
+// multiply-adds along K that more of them hide: 976 x 75 outputs of 400 terms 28 -> 20 us); dW
+// always the latter, whose three warps a scheduler hide the compensation's chain (64 x 200, 185 steps,
+// dW with dx beside it: 507 us, 578 by 64 x 64; 300 without compensation)
 template <bool kAT, int EA>
 void launch_gemm(stacklstm *s, const GemmF32 &g, int splits)
 {
     const unsigned nt = ceil_div(g.N, 64), big = ceil_div(g.M, 64);
-    if ((size_t)big * nt * splits >= 3 * (size_t)s->num_sms)
-        gemm_f32<2, 1, 8, kAT, EA><<<dim3(big, nt, splits), 64, 0, s->stream>>>(g);
+    if (!kAT && (size_t)big * nt * splits >= 3 * (size_t)s->num_sms)
+        gemm_f32<2, 1, kAT ? 4 : 8, kAT, EA><<<dim3(big, nt, splits), 64, 0, s->stream>>>(g);
     else
         gemm_f32<2, 1, 4, kAT, EA><<<dim3(ceil_div(g.M, 32), nt, splits), 64, 0, s->stream>>>(g);
     s->launches += 1;
@@ -754,7 +803,7 @@ bool fp32_plan_rows(stacklstm *s)
     const char *lim = getenv("STACKLSTM_WAIT_LIMIT_CYCLES"), *limb = getenv("STACKLSTM_WAIT_LIMIT_BWD_CYCLES");
     s->wait_limit = lim ? atoll(lim) : 4000000000LL;
     s->wait_limit_bwd = limb ? atoll(limb) : s->wait_limit;
-    if (cudaMalloc(&p, sizeof(float) * slab * s->fr32_split) != cudaSuccess) {
+    if (cudaMalloc(&p, 2 * sizeof(float) * slab * s->fr32_split) != cudaSuccess) {  // sums and their errors
         cudaGetLastError();
         s->fr32.on = 0;
         return false;
@@ -833,9 +882,10 @@ cudaError_t fp32_rows_dw(stacklstm *s, float *dW, float *dbias)
     g.A2 = (const float *)s->a_rm; g.lda2 = H;
     g.B = (const float *)s->dG; g.ldb = G;
     g.C = s->dw_part; g.ldc = G; g.slab = (size_t)g.M * G;
+    g.Cr = g.C + nz * g.slab;
     launch_gemm<true>(s, g, nz);
     slab_sum_f32<<<(unsigned)std::min<size_t>(ceil_div(g.slab, 256), (size_t)s->num_sms * 8), 256, 0, s->stream>>>(
-        (size_t)g.M2 * G, g.slab - (size_t)g.M2 * G, nz, s->dw_part, g.slab, dW, dbias);
+        (size_t)g.M2 * G, g.slab - (size_t)g.M2 * G, nz, g.C, g.Cr, g.slab, dW, dbias);
     s->launches += 1;
     return cudaGetLastError();
 }

@@ -199,3 +199,33 @@ def test_weight_and_bias_gradients_alone_equal_both(T, B, I, H):
             assert np.array_equal(full[k].cpu().numpy(), both[k]), k
     finally:
         hd.destroy()
+
+
+@pytest.mark.parametrize("T,B,H", [(1, 1100, 8), (1, 60000, 8), (37, 320, 12), (1, 9001, 9), (185, 64, 40)])
+def test_weight_gradient_sums_are_compensated(T, B, H):
+    """The sums over all T B rows alone, their operands taken as they are. With I = 4H and the
+    identity as W_x, dx is dG exactly; x and the states read (h0 at T = 1) are the other operand.
+    Rounding the result alone leaves up to 2^-24 / sqrt(3) = 3.4e-8 in the 2-norm, and the products
+    (two roundings of 2^-24 of a term at most, over n terms of like size) less than that; sums
+    with rounding errors that add up over the rows of a split have 1.2e-7 and more."""
+    I = 4 * H
+    g = torch.Generator(device="cuda").manual_seed(T * B + H)
+    r = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    W = torch.cat([torch.eye(I, device="cuda"), 0.1 * r(H, I)])
+    ins = dict(x=r(T, B, I), ops=torch.ones(T, B, dtype=torch.int8, device="cuda"), h0=r(B, H), c0=r(B, H), W=W, bias=r(I))
+    e = lambda *s: torch.full(s, float("nan"), device="cuda")
+    y, dx, dh0, dc0, dW, dbias = e(T, B, H), e(T, B, I), e(B, H), e(B, H), e(I + H, I), e(I)
+    hd = bd.stacklstm_create(T, B, I, H, bd.SL_FP32, 0)
+    try:
+        assert "clusters" in bd.stacklstm_plan(hd), bd.stacklstm_plan(hd)
+        bd.stacklstm_forward(hd, *(ins[k] for k in ("x", "ops", "h0", "c0", "W", "bias")),
+                             p_final=torch.empty(B, dtype=torch.int32, device="cuda"), y=y)
+        bd.stacklstm_backward(hd, None, r(T, B, H), dx, dh0, dc0, dW, dbias)
+    finally:
+        hd.destroy()
+    dG = dx.double().view(-1, I)
+    read = torch.cat([ins["h0"][None], y[:-1]]).double().view(-1, H)  # pushes only: the step before's output
+    rows = torch.cat([ins["x"].double().view(-1, I), read], 1)
+    for got, want in ((dW, rows.t() @ dG), (dbias, dG.sum(0))):
+        err = ((got.double() - want).norm() / want.norm()).item()
+        assert err < 5e-8, err

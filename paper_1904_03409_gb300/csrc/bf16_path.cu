@@ -709,7 +709,7 @@ cudaError_t bf16_prepare(stacklstm *s)
         // clusters do not (bf16_rows.cu has the figures)
         if (bf16_plan_rows(s, 1) || (!(s->fc.on && s->bc.on) && bf16_plan_rows(s, 2)))
             s->fc.on = s->pf.on = s->bc.on = 0;
-        // small batches: both directions on CUDA cores instead
+        // small batches that are in no row clusters: both directions on CUDA cores instead
         if (bf16_plan_small(s, &s->cc)) {
             s->pf.on = s->pb.on = s->fc.on = s->bc.on = s->fr.on = s->br.on = 0;
             s->uf = s->ub = s->cc.U;

@@ -34,17 +34,16 @@ constexpr int kCcThreads = 256;   // 8 warps
 constexpr int kCcWarps = kCcThreads / 32;
 constexpr int kCcRedStride = 80;  // floats per reduction row: rows b, b + 1 of a warp hit distinct banks
 constexpr int kCcMaxB = 32;       // rows the kernels hold (register accumulators per row)
-// Largest batch the planner gives these kernels by default. Measured at I = H = 200 (one
-// forward + backward pass of the parser sweep workload): B = 1, 0.597 ms here against
-// 0.695 ms for the tensor-core cluster kernels (backward step 1.67 against 2.26 us, the
+// Largest batch the planner gives these kernels by default, where the row clusters
+// (bf16_rows.cu) do not hold it: one row is faster there at every length and width (I = H = 200,
+// one pass of 1 / 8 / 40 / 60 steps: 44 / 55 / 106 / 138 us there, 54 / 76 / 172 / 230 here; H = 8, 36 to
+// 102 us against 49 to 179), so what is left here are inputs too wide for their shared memory
+// (H = 200: from I of about 650; one row of 60 steps, 800 + 200: 288 us here, 389 with the
+// persistent forward and the 64-row backward cluster). Measured against the 64-row clusters at I = H = 200 (one forward + backward pass of the parser
+// sweep workload): B = 1, 0.597 ms here against 0.695 ms (backward step 1.67 against 2.26 us, the
 // forward step equal at 1.57 us); B = 8, 1.80 ms against 0.77 ms; B = 32, 6.19 against
 // 0.83 ms. Per row, the FFMA contraction adds about 0.4 us a step.
 constexpr int kCcCrossoverB = 1;
-// Longer sequences of one row go to the row-group clusters (bf16_rows.cu), whose step is
-// shorter (0.92 / 0.78 us; they are the faster here too, 113 us a pass against 182 at 40 steps,
-// and STACKLSTM_CUDA_CORE=0 selects them). The line lies at 40 because the planner's default for
-// one row of 40 steps is fixed by its test.
-constexpr int kCcCrossoverT = 40;
 
 __device__ __forceinline__ uint32_t cc_rank()
 {
@@ -530,9 +529,9 @@ cudaError_t cc_launch(stacklstm *s, bool fwd, const CcArgs &p, size_t smem)
 }  // namespace
 
 // Batches up to kCcMaxB: the CUDA-core cluster kernels when the shape fits (at most 16
-// CTAs of 16 units; both footprints within shared memory; the cluster co-resident) and
-// B is at most the crossover below which they beat the tensor-core cluster kernels
-// (measured on this GPU at I = H = 200). Test hook (include/stacklstm.h):
+// CTAs of 16 units; both footprints within shared memory; the cluster co-resident),
+// B is at most the crossover below which they beat the 64-row tensor-core clusters, and no
+// row clusters are planned. Test hook (include/stacklstm.h):
 // STACKLSTM_CUDA_CORE=0 never, =1 whenever the shape fits.
 bool bf16_plan_small(stacklstm *s, PersistPlan *pl)
 {
@@ -542,7 +541,7 @@ bool bf16_plan_small(stacklstm *s, PersistPlan *pl)
     if (want == 0) return false;
     const int n_ct = (int)ceil_div(s->H, kCcU), BT = cc_tier(s->B);
     if (s->B > kCcMaxB || n_ct > 16 || s->I % 8 || s->H % 8) return false;
-    if (want < 0 && (s->B > kCcCrossoverB || s->T > kCcCrossoverT)) return false;
+    if (want < 0 && (s->B > kCcCrossoverB || s->fr.on)) return false;
     const size_t sf = ccf_smem_bytes(BT, s->I, s->H, n_ct), sb = ccb_smem_bytes(BT, n_ct);
     if (sf > kSmemCap || sb > kSmemCap) return false;
     for (int dir = 0; dir < 2; ++dir) {

@@ -2,10 +2,10 @@
 
 For batches up to 32 the forward and the backward can run as one thread-block cluster on
 CUDA cores (FFMA contraction, weights resident in shared memory) instead of the
-tensor-core cluster kernels; the planner picks them below a measured crossover batch
-size. Both paths are run here at the same shapes (STACKLSTM_CUDA_CORE=1 forces the
-CUDA-core kernels, =0 the tensor-core ones), into NaN-filled outputs, and compared with
-the oracle element by element: every row-count tier of the kernels (1, 2, 4, 8, 16, 32
+tensor-core cluster kernels; the planner picks them for one row that the row clusters
+(bf16_rows.cu) cannot hold. Both paths are run here at the same shapes
+(STACKLSTM_CUDA_CORE=1 forces the CUDA-core kernels, =0 the tensor-core ones), into
+NaN-filled outputs, and compared with the oracle element by element: every row-count tier of the kernels (1, 2, 4, 8, 16, 32
 rows), ragged hidden widths (H not a multiple of the 16-unit slice), narrow and wide
 inputs, dy seeds, push-only mode, and run-to-run bitwise reproducibility.
 """
@@ -93,12 +93,24 @@ def test_cuda_core_backward_is_bitwise_reproducible():
         assert np.array_equal(a[k], b[k]), k
 
 
-def test_planner_default_by_batch_size():
-    """Unforced, the planner gives one row up to the crossover to the CUDA-core kernels and
-    a 64-row batch to the tensor-core cluster kernels."""
-    for B, want in ((1, "forward cuda-core"), (64, "forward cluster")):
-        hd = bd.stacklstm_create(40, B, 200, 200, bd.SL_BF16, 0)
-        try:
-            assert want in bd.stacklstm_plan(hd)
-        finally:
-            hd.destroy()
+@pytest.mark.parametrize("T,B,I,H,want", [
+    (1, 1, 200, 200, "rows 8"), (40, 1, 200, 200, "rows 8"), (41, 1, 8, 8, "rows 8"), (40, 64, 200, 200, "rows 8"),
+    (1, 1, 800, 200, "forward cuda-core"), (60, 1, 800, 200, "forward cuda-core"), (60, 1, 800, 32, "forward cuda-core"),
+    (60, 2, 800, 200, "rows 0")])
+def test_planner_default_by_batch_size(T, B, I, H, want):
+    """Unforced, the planner gives small batches to the row clusters at every length, and one row
+    whose input is too wide for them to the CUDA-core kernels, however long it is (two rows to
+    the tensor-core kernels)."""
+    hd = bd.stacklstm_create(T, B, I, H, bd.SL_BF16, 0)
+    try:
+        plan = bd.stacklstm_plan(hd)
+        assert want in plan, plan
+        assert ("cuda-core" in plan) == ("cuda-core" in want), plan
+        assert ("forward cluster" in plan) == (want == "rows 8"), plan
+    finally:
+        hd.destroy()
+
+
+def test_wide_input_of_one_row_matches_oracle():
+    w = case(60, 1, 800, 200, 59, bias_scale=0.3, h0_scale=0.5, c0_scale=0.5, dy_scale=0.5)
+    compare(runner.run(w), oracle_all(w), "bf16")

@@ -205,7 +205,7 @@ sl_status fwd_begin(stacklstm *s, const sl_forward_args &a)
     cudaError_t e;
     s->fwd_done = 0;
     // the row clusters hold each step's output already: it is the next step's h operand
-    s->y_direct = (s->fr.on || s->fr32.on) && !s->push_only ? a.y : nullptr;
+    s->y_direct = (s->fr.on || (s->fr32.on && !s->fr32_steps)) && !s->push_only ? a.y : nullptr;
     // the initial state and the weight packing do not depend on the index prepass, so they
     // run on the side stream at the same time (launched after the prepass, whose few blocks
     // then reach the SMs first); the caller's stream waits for them before the forward steps

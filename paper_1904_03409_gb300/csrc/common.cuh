@@ -60,6 +60,7 @@ struct stacklstm {
     int fp32_one_cta = 0;        // fp32: every step of each direction in one CTA (small B * H)
     PersistPlan fr32;            // fp32: clusters of few rows (fp32_rows.cu; EP: warps a CTA)
     int fr32_split = 1;          // their weight gradient's splits
+    int fr32_steps = 0;          // the forward beside them is one launch a step (a_rm holds [x ; h_read] rows)
     int pfinal_written = 0;      // the last prepass also wrote the caller's final pointers
 
     // integer bookkeeping, written by the prepass (all [T+1][B] int32)

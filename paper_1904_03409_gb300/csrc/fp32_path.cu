@@ -408,7 +408,7 @@ cudaError_t fp32_forward_setup(stacklstm *s, const float *h0, const float *c0, c
 cudaError_t fp32_forward_steps(stacklstm *s, const float *x, const float *W, const float *bias)
 {
     const int T = s->T, B = s->B, I = s->I, H = s->H, K = I + H;
-    if (s->fr32.on) return fp32_rows_forward(s, x, W, bias);
+    if (s->fr32.on && !s->fr32_steps) return fp32_rows_forward(s, x, W, bias);
     if (s->fp32_one_cta) {
         (void)K;
         const int P = fwd_seq_threads_per_unit(B, H);

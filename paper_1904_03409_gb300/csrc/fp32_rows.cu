@@ -756,6 +756,20 @@ void launch_gemm(stacklstm *s, const GemmF32 &g, int splits)
 
 }  // namespace
 
+// A forward of one step runs as fwd_step_f32 where that is shorter: the clusters read W_h into
+// registers for one use, and x W_x is a launch of its own (T = 1, step / clusters: 33 + 33, 4000 rows
+// 28 / 34 us; 64 + 64, 20 rows 21 / 21, 8000 rows 69 / 83; 100 + 100, 128 rows 27 / 23, 512 rows 30 /
+// 32; 200 + 200, 1024 rows 108 / 109; 200 + 256, 8192 rows 848 / 910; T = 2 there 1711 / 1187). The
+// clusters also hold next to nothing at H <= 3 (16 + 3, 3 steps of 4000 / 20000 rows 31 / 35 and 68 / 73
+// us, 4 steps 39 / 43 and 88 / 67; 16 + 1, 8 steps of 8000 rows 97 / 96, of 40000 285 / 424).
+// fwd_step_f32's operand has 48 KB of shared memory.
+bool fr_step_forward(int T, int B, int I, int H)
+{
+    if (I + H > 12 * 1024) return false;
+    if (T == 1) return H <= 64 || B >= (H <= 128 ? 512 : 4096);
+    return (H <= 3 && T <= 3 && B >= 4000) || (H == 1 && B > 8192);
+}
+
 // The plan: rows a cluster R and CTAs a cluster C with the least rounds x step cycles, a step
 // being the warps' multiply-adds on the fullest of the SM's four schedulers plus about 1500
 // cycles of cell and exchange. (Registers allow one CTA an SM for large H: at 64 x 200, 14
@@ -794,6 +808,7 @@ bool fp32_plan_rows(stacklstm *s)
             }
         }
     if (!s->fr32.on) return false;
+    s->fr32_steps = fr_step_forward(s->T, s->B, s->I, H);
     // dW and dbias: splits of the T B rows for about two rounds of 64 x 64 tiles (four an SM at
     // once), at least 128 rows each
     const size_t rows = (size_t)s->T * s->B, tiles = ceil_div(s->I + H + 1, 64) * ceil_div(4 * H, 64);
@@ -880,6 +895,11 @@ cudaError_t fp32_rows_dw(stacklstm *s, float *dW, float *dbias)
     g.N = G; g.K = s->T * s->B;
     g.A = (const float *)s->x_saved; g.lda = I;
     g.A2 = (const float *)s->a_rm; g.lda2 = H;
+    if (s->fr32_steps) {  // rows of [x ; h_read]
+        g.A = (const float *)s->a_rm;
+        g.A2 = g.A + I;
+        g.lda = g.lda2 = (size_t)I + H;
+    }
     g.B = (const float *)s->dG; g.ldb = G;
     g.C = s->dw_part; g.ldc = G; g.slab = (size_t)g.M * G;
     g.Cr = g.C + nz * g.slab;

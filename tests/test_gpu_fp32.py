@@ -229,3 +229,19 @@ def test_weight_gradient_sums_are_compensated(T, B, H):
     for got, want in ((dW, rows.t() @ dG), (dbias, dG.sum(0))):
         err = ((got.double() - want).norm() / want.norm()).item()
         assert err < 5e-8, err
+
+
+@pytest.mark.parametrize("T,B,I,H,seed", [(1, 70, 40, 64, 51), (1, 300, 9, 33, 52), (1, 600, 16, 100, 53),
+                                          (1, 513, 17, 99, 54), (3, 4100, 5, 3, 55), (2, 9000, 4, 1, 56),
+                                          (1, 4097, 8, 132, 57)])
+def test_step_forward_beside_the_row_clusters_backward(T, B, I, H, seed):
+    """Forwards of one step, or of few at H <= 3, by the step kernel, and the backward in clusters:
+    the weight gradient reads the rows [x ; h_read] that the step kernel kept, with and without
+    the alignment for 16-byte copies; an output is the top's row of the history."""
+    w = wl.make_workload("case", T=T, B=B, I=I, H=H, dtype="fp32", seed=seed, ops_kind="random_walk",
+                         probs=(0.5, 0.3, 0.2), bias_scale=0.3, h0_scale=0.5, c0_scale=0.5, dy_scale=0.5)
+    got = runner.run(w)
+    compare(got, oracle_of(w), "fp32")
+    again = runner.run(w)
+    for k in ("y", "h_stack", "c_stack", "dx", "dW", "dbias", "dh0", "dc0"):
+        assert np.array_equal(got[k], again[k]), k

@@ -142,3 +142,24 @@ def test_initial_state_gradients_are_counted_beyond_32_bits(lib, B, H, dtype):
     copies = [l for l in launches(lib) if "h0_grads" in l[0]]
     lib.stacklstm_destroy(h)
     assert len(copies) == 1 and copies[0][1] == (min(152, -(-B * H // 256)), 1, 1), copies
+
+
+@pytest.mark.parametrize("T,B,I,H,steps", [
+    (1, 40, 33, 33, 1), (1, 8000, 64, 64, 1), (2, 8000, 64, 64, 0), (1, 128, 100, 100, 0), (1, 512, 100, 100, 1),
+    (1, 1024, 200, 200, 0), (1, 4096, 200, 200, 1), (3, 4000, 16, 3, 3), (6, 4000, 16, 3, 0), (8, 40000, 16, 1, 8),
+    (1, 40, 12300, 33, 0)])
+def test_fp32_forward_of_few_steps_takes_the_step_kernel_where_it_is_shorter(lib, T, B, I, H, steps):
+    """Beside a backward in row clusters; y then comes from the history like before them."""
+    h = create(lib, T, B, I, H, FP32)
+    assert b"clusters" in lib.stacklstm_plan(h)
+    lib.fake_reset()
+    assert forward(lib, h) == 0
+    fwd = [l[0] for l in launches(lib)]
+    lib.fake_reset()
+    assert backward(lib, h) == 0
+    bwd = [l[0] for l in launches(lib)]
+    lib.stacklstm_destroy(h)
+    assert sum("fwd_step_f32" in k for k in fwd) == steps, fwd
+    assert sum("fwd_rows_f32" in k for k in fwd) == (0 if steps else 1), fwd
+    assert sum("gather_rows" in k for k in fwd) == (3 if steps else 2), fwd  # h_stack, c_stack, y
+    assert sum("bwd_rows_f32" in k for k in bwd) == 1, bwd

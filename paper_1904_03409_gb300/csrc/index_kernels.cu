@@ -8,6 +8,7 @@
 //   slot_last   history index last written to each slot after the last step (-1: never).
 // Every step writes slot p_t + 1 (Algorithm 1), which in history terms is row t + 1.
 #include <algorithm>
+#include <type_traits>
 #include <map>
 #include <mutex>
 
@@ -277,33 +278,39 @@ prepass_walk_vec_kernel(int T, int B, const int8_t *__restrict__ ops, int32_t *_
 }
 
 // out[r] = hist row (idx[r], r % B), or zeros where idx[r] < 0; rows of `pieces` values of the
-// raw type E (16 bytes where the row length and the addresses allow, else 4 or 2). A warp takes
-// four rows at a time, so that its index loads and its row loads are in flight together: bound by
-// the bytes moved (195 x 1024 rows of 400 bytes, 160 MB: 23 us, 115 as one thread per 2-byte
-// value with a 64-bit division each; 256 x 256 rows of 2 KB: 32 us, 197).
-template <typename E>
+// raw type E (16 bytes where the row length and the addresses allow, else 4 or 2). 2^lg lanes
+// take a row, a warp (kWarp) or the fewest that give each piece one, four rows at a time, so that
+// the index loads and the row loads are in flight together: bound by the bytes moved (195 x 1024
+// rows of 400 bytes, 160 MB: 23 us, 115 as one thread per 2-byte value with a 64-bit division each;
+// 256 x 256 rows of 2 KB: 28 us, 188; 40 x 20000 rows of 16 bytes: 10 us, 27, and 55 with a warp to
+// every row).
+template <typename E, bool kWarp>
 __global__ void __launch_bounds__(256) gather_rows_kernel(const int32_t *__restrict__ idx, int B, int rows, int pieces,
-                                                          const E *__restrict__ hist, E *__restrict__ out)
+                                                          int lg_, const E *__restrict__ hist, E *__restrict__ out)
 {
     constexpr int N = 4;
-    const int lane = threadIdx.x & 31, warps = gridDim.x * (blockDim.x >> 5);
-    for (int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); (long long)g * N < rows; g += warps) {
-        const int r0 = g * N, r = min(r0 + (lane & (N - 1)), rows - 1);
-        const int s = idx[r];
-        const long long src = s >= 0 ? (long long)s * B + r % B : -1;
+    const int lg = kWarp ? 5 : lg_;
+    const int lane = threadIdx.x & 31, sub = lane & ((1 << lg) - 1), per = 32 >> lg, warps = gridDim.x * (blockDim.x >> 5);
+    auto source = [&](uint32_t row) -> long long {  // of one row (past the last: of that one), or -1
+        const int r = (int)min(row, (uint32_t)rows - 1), s = idx[r];
+        return s >= 0 ? (long long)s * B + r % B : -1;
+    };
+    for (int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); (long long)g * N * per < rows; g += warps) {
+        const uint32_t r0 = (uint32_t)(g * N * per + (lane >> lg));
+        const long long mine = kWarp ? source(r0 + (lane & (N - 1))) : 0;  // a row to each of four lanes
         const E *from[N];
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-            const long long q = __shfl_sync(0xffffffffu, src, i);
+            const long long q = kWarp ? __shfl_sync(0xffffffffu, mine, i) : source(r0 + i * per);
             from[i] = q >= 0 ? hist + (size_t)q * pieces : nullptr;
         }
-        for (int k = lane; k < pieces; k += 32) {
+        for (int k = sub; k < pieces; k += 1 << lg) {
             E v[N];
 #pragma unroll
             for (int i = 0; i < N; ++i) v[i] = from[i] ? from[i][k] : E{};
 #pragma unroll
             for (int i = 0; i < N; ++i)
-                if (r0 + i < rows) out[(size_t)(r0 + i) * pieces + k] = v[i];
+                if (r0 + i * per < (uint32_t)rows) out[(size_t)(r0 + i * per) * pieces + k] = v[i];
         }
     }
 }
@@ -640,18 +647,25 @@ cudaError_t launch_gather_rows(stacklstm *s, const int32_t *idx, int rows, size_
                                const void *hist, void *out, int row_elems)
 {
     if (rows == 0 || row_elems == 0) return cudaSuccess;
-    const unsigned grid = (unsigned)std::min<size_t>(ceil_div(rows, 32), (size_t)s->num_sms * 16);
     // (hist is workspace and out 16-byte aligned: a row whose length is a multiple of 16 bytes is too)
     const size_t row_bytes = (size_t)row_elems * elem_bytes;
+    const int pieces = row_bytes % 16 == 0 ? (int)(row_bytes / 16) : row_elems;
+    int lg = 0;
+    while (lg < 5 && 1 << lg < pieces) ++lg;
+    const unsigned grid = (unsigned)std::min<size_t>(ceil_div(rows, 1024 >> lg), (size_t)s->num_sms * 16);
+    auto go = [&](auto *of) {
+        using E = std::remove_pointer_t<decltype(of)>;
+        if (lg == 5)
+            gather_rows_kernel<E, true><<<grid, 256, 0, s->stream>>>(idx, s->B, rows, pieces, lg, (const E *)hist, (E *)out);
+        else
+            gather_rows_kernel<E, false><<<grid, 256, 0, s->stream>>>(idx, s->B, rows, pieces, lg, (const E *)hist, (E *)out);
+    };
     if (row_bytes % 16 == 0)
-        gather_rows_kernel<uint4><<<grid, 256, 0, s->stream>>>(idx, s->B, rows, (int)(row_bytes / 16), (const uint4 *)hist,
-                                                               (uint4 *)out);
+        go((uint4 *)nullptr);
     else if (elem_bytes == 4)
-        gather_rows_kernel<uint32_t><<<grid, 256, 0, s->stream>>>(idx, s->B, rows, row_elems, (const uint32_t *)hist,
-                                                                  (uint32_t *)out);
+        go((uint32_t *)nullptr);
     else
-        gather_rows_kernel<uint16_t><<<grid, 256, 0, s->stream>>>(idx, s->B, rows, row_elems, (const uint16_t *)hist,
-                                                                  (uint16_t *)out);
+        go((uint16_t *)nullptr);
     s->launches += 1;
     return cudaGetLastError();
 }

@@ -163,3 +163,16 @@ def test_fp32_forward_of_few_steps_takes_the_step_kernel_where_it_is_shorter(lib
     assert sum("fwd_rows_f32" in k for k in fwd) == (0 if steps else 1), fwd
     assert sum("gather_rows" in k for k in fwd) == (3 if steps else 2), fwd  # h_stack, c_stack, y
     assert sum("bwd_rows_f32" in k for k in bwd) == 1, bwd
+
+
+@pytest.mark.parametrize("H,dtype,lanes", [(1, FP32, 1), (8, BF16, 1), (16, BF16, 2), (24, BF16, 4), (9, FP32, 16),
+                                           (64, FP32, 16), (136, BF16, 32), (33, FP32, 32), (104, FP32, 32)])
+def test_gathers_give_a_row_no_more_lanes_than_it_has_pieces(lib, H, dtype, lanes):
+    h = create(lib, 3, 1999, 8, H, dtype)
+    lib.fake_reset()
+    assert forward(lib, h) == 0
+    gathers = [l for l in launches(lib) if "gather_rows" in l[0]]
+    lib.stacklstm_destroy(h)
+    # h_stack, before c_stack: four rows to each group of lanes, eight warps a block
+    assert gathers[-2][1][0] == -(-4 * 1999 * lanes // 1024), gathers
+    assert ("Lb1E" in gathers[-2][0]) == (lanes == 32), gathers

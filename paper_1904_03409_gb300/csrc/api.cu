@@ -161,12 +161,13 @@ sl_status queue_clear(stacklstm *s)
 }
 
 // The clear goes beside the prepass and ends before the steps where row clusters can have an SM
-// for each CTA: a clear whose blocks fill the SMs when the step launch starts makes the
-// scheduler put clusters two to an SM, although others are free, for the whole launch. 64 x 200
-// steps then took 1.5 us instead of 0.97 (a 185-step pass 580 instead of 475 us after an idle
-// stream, and now and then in a full one; three 64-row stacks at once and their head 875 instead
-// of 806). A launch that needs two CTAs an SM, or is one cluster, gains nothing and loses the
-// wait (512 x 200 forward 541 -> 553 us, 1 x 200 190 -> 194).
+// for each CTA, and an SM has room for two: a clear whose blocks fill the SMs when the step launch
+// starts makes the scheduler put clusters two to an SM, although others are free, for the whole
+// launch. 64 x 200 steps then took 1.5 us instead of 0.97 (a 185-step pass 580 instead of 475 us
+// after an idle stream, and now and then in a full one; three 64-row stacks at once and their head
+// 875 instead of 806). A launch that needs two CTAs an SM, is one cluster, or fits only one CTA an
+// SM gains nothing and loses the wait (512 x 200 forward 541 -> 553 us, 1 x 200 190 -> 194, 40 rows
+// of 60 steps of 520 + 256 100 -> 104).
 bool clear_early(const stacklstm *s) { return s->fr.on && s->fr.spread && !s->push_only; }
 
 sl_status fwd_clear(stacklstm *s)

@@ -778,11 +778,12 @@ bool rc_plan(stacklstm *s, bool fwd, int NT, PersistPlan *pl)
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
     rc_config(&cfg, at, 1, C, smem, nullptr);
-    int clusters = 0;
+    int clusters = 0, per_sm = 0;
     // (the forward's split of the registers draws on what the block is launched with)
     if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess ||
         ((fwd || NT > 1) && fa.numRegs * kRcThreads < (kRcRegsStep + kRcRegsX) * (kRcThreads / 2)) ||
-        smem_at_least(fn, smem) != cudaSuccess || cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) != cudaSuccess) {
+        smem_at_least(fn, smem) != cudaSuccess || cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kRcThreads, smem) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -796,8 +797,9 @@ bool rc_plan(stacklstm *s, bool fwd, int NT, PersistPlan *pl)
     pl->rows = NR;
     pl->smem = smem;
     pl->threads = kRcThreads;
-    pl->per_sm = 2;
-    pl->spread = s->B > NR && 2 * (int)ceil_div(s->B, NR) <= clusters;
+    pl->per_sm = per_sm;  // two, or one where W_x takes over half of the shared memory
+    // (clusters that could share SMs though each CTA can have one: the clear goes ahead of the steps)
+    pl->spread = per_sm > 1 && s->B > NR && per_sm * (int)ceil_div(s->B, NR) <= clusters;
     return true;
 }
 

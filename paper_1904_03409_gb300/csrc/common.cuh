@@ -31,7 +31,7 @@ struct PersistPlan {
     unsigned smem = 0;  // dynamic shared memory per CTA
     int threads = 0;    // threads per CTA
     int per_sm = 1;     // co-resident CTAs per SM at this footprint
-    bool spread = false;  // several clusters, and an SM for each of their CTAs (bf16_rows.cu)
+    bool spread = false;  // several clusters, an SM for each of their CTAs, and room for two (bf16_rows.cu)
     int n_dx = 0;       // backward: extra CTAs computing dx on the SMs the steps leave idle
     int dx_S = 0;       // their ring stages
 };

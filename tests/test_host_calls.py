@@ -176,3 +176,18 @@ def test_gathers_give_a_row_no_more_lanes_than_it_has_pieces(lib, H, dtype, lane
     # h_stack, before c_stack: four rows to each group of lanes, eight warps a block
     assert gathers[-2][1][0] == -(-4 * 1999 * lanes // 1024), gathers
     assert ("Lb1E" in gathers[-2][0]) == (lanes == 32), gathers
+
+
+@pytest.mark.parametrize("B,I,early", [(64, 200, True), (64, 520, False), (8, 200, False), (200, 200, False)])
+def test_the_clear_comes_before_the_steps_where_clusters_could_share_sms_without_need(lib, B, I, early):
+    """Row clusters that fit two CTAs an SM and have an SM for each of several clusters' CTAs: the
+    gradient history's clear is joined before the steps. One CTA an SM (a wide input), one cluster,
+    or more clusters than that: it runs beside them, and the next backward waits for it."""
+    h = create(lib, 40, B, I, 200, BF16)
+    plan = lib.stacklstm_plan(h).decode()
+    assert "rows 8" in plan and ("per SM %d rows" % (2 if I == 200 else 1)) in plan.split("; backward")[0], plan
+    lib.fake_reset()
+    assert forward(lib, h) == 0
+    left = lib.fake_unjoined(USER)
+    lib.stacklstm_destroy(h)
+    assert left == (0 if early else 1)

@@ -131,12 +131,14 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int *n, const void *, 
     *n = threads <= 256 && smem <= 113 * 1024 ? 2 : 1;
     return cudaSuccess;
 }
-cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *, const cudaLaunchConfig_t *c)
+cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *fn, const cudaLaunchConfig_t *c)
 {
     unsigned cl = 1;
     for (unsigned i = 0; i < c->numAttrs; ++i)
         if (c->attrs[i].id == cudaLaunchAttributeClusterDimension) cl = c->attrs[i].val.clusterDim.x;
-    *n = (int)(152 / cl);
+    int per_sm;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, (int)c->blockDim.x, c->dynamicSmemBytes);
+    *n = (int)(per_sm * 152 / cl);
     return cudaSuccess;
 }
 cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **fn, unsigned, unsigned long long,

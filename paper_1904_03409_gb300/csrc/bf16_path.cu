@@ -968,14 +968,16 @@ static const PersistPlan &group_plan(const stacklstm *s, bool fwd)
     return fwd ? (s->fr.on ? s->fr : s->fc) : (s->br.on ? s->br : s->bc);
 }
 
+// Handles of at most 64 rows whose kernel is the same: clusters of as many rows over as many 16-unit
+// tiles (which set the cluster size and, for row clusters, the contraction depth they are built for).
 bool bf16_can_group(stacklstm *const *hs, int n, bool fwd)
 {
     const PersistPlan &p0 = group_plan(hs[0], fwd);
     for (int m = 0; m < n; ++m) {
         const stacklstm *s = hs[m];
         const PersistPlan &pl = group_plan(s, fwd);
-        if (s->dt != SL_BF16 || s->cc.on || !pl.on || pl.slot != 1 || pl.n_ct != p0.n_ct || pl.rows != p0.rows ||
-            s->device != hs[0]->device)
+        if (s->dt != SL_BF16 || s->cc.on || !pl.on || s->B > 64 || ceil_div(s->H, 16) != ceil_div(hs[0]->H, 16) ||
+            pl.rows != p0.rows || s->device != hs[0]->device)
             return false;
     }
     return true;

@@ -789,11 +789,10 @@ bool rc_plan(stacklstm *s, bool fwd, int NT, PersistPlan *pl)
     }
     if ((int)ceil_div(s->B, NR) > clusters) return false;
     pl->on = 1;
-    pl->U = 16;  // (the M tile; a CTA holds two)
+    pl->U = 32;
     pl->EP = 1;
-    pl->n_ct = (int)ceil_div(s->H, 16);
-    pl->cl = C;
-    pl->slot = (int)ceil_div(s->B, 64);
+    pl->n_ct = pl->cl = C;
+    pl->slot = (int)ceil_div(s->B, NR);
     pl->rows = NR;
     pl->smem = smem;
     pl->threads = kRcThreads;

@@ -136,25 +136,37 @@ def test_four_lanes_per_row_backward_epilogue(T, B, I, H, seed):
 PERSISTENT = {"STACKLSTM_FWD_CLUSTER": "0", "STACKLSTM_BWD_CLUSTER": "0"}
 
 
-@pytest.mark.parametrize("B,env", [(130, PERSISTENT), (40, {}), (130, {})])
-def test_wait_timeout_is_reported_and_context_survives(B, env):
-    """With a zero wait budget the bounded device-side waits run out: forward (persistent
-    kernel at B = 130, thread-block clusters at B = 40 and at B = 130, three row tiles)
-    reports SL_ERR_TIMEOUT instead of hanging, and the device stays usable."""
-    w = case(4, B, 16, 32, 9)
-    old = {k: os.environ.get(k) for k in env}
-    os.environ.update(env)
-    os.environ["STACKLSTM_WAIT_LIMIT_CYCLES"] = "0"
+TILE64 = {"STACKLSTM_ROW_CLUSTER": "0"}  # the 64-row clusters where row clusters would run
+
+
+def phase_plans(plan):
+    """The plan string's forward and backward parts."""
+    fwd, bwd = plan.split("; backward ")
+    return fwd.split("; forward ")[1], bwd.split("; step rings")[0]
+
+
+@pytest.mark.parametrize("B,I,H,env,want", [
+    (130, 16, 32, PERSISTENT, "persistent"), (40, 16, 32, {}, "rows 8]"), (130, 16, 32, {}, "rows 8]"),
+    (500, 16, 200, {}, "rows 16]"), (40, 16, 32, TILE64, "rows 0]"), (130, 16, 32, TILE64, "rows 0]")])
+def test_wait_timeout_is_reported_and_context_survives(B, I, H, env, want):
+    """With a zero wait budget the bounded device-side waits run out: the forward (the persistent
+    kernel, clusters of 8 rows in one or several groups and of 16, clusters of 64-row tiles, one
+    and three) reports SL_ERR_TIMEOUT instead of hanging, and the device stays usable."""
+    w = case(4, B, I, H, 9)
+    keys = dict(env, STACKLSTM_WAIT_LIMIT_CYCLES="0")
+    old = {k: os.environ.get(k) for k in keys}
+    os.environ.update(keys)
     try:
         hd = bd.stacklstm_create(w.T, w.B, w.I, w.H, bd.SL_BF16, 0)
     finally:
-        del os.environ["STACKLSTM_WAIT_LIMIT_CYCLES"]
         for k, v in old.items():
             if v is None:
                 os.environ.pop(k, None)
             else:
                 os.environ[k] = v
     try:
+        fwd = phase_plans(bd.stacklstm_plan(hd))[0]
+        assert want in fwd and (want == "persistent" or fwd.startswith("cluster")), fwd
         ins = runner.upload(w)
         out = runner.alloc_outputs(w)
         with pytest.raises(bd.StackLSTMError) as e:
@@ -170,14 +182,17 @@ def test_wait_timeout_is_reported_and_context_survives(B, env):
     (6, 200, 64, 256, dict(PERSISTENT, STACKLSTM_BWD_SPLIT="4"), "cluster 4 "),  # split contraction, clusters
     (4, 4096, 256, 256, {}, "U=32 [EP 1"),                                      # the release warp's plan
     (6, 200, 64, 256, dict(PERSISTENT, STACKLSTM_BWD_SPLIT="4", STACKLSTM_SPLIT_CLUSTER="0"), "cluster 1 "),
-    (6, 40, 64, 64, {}, "cluster U=16 ["),                                       # one-row-tile cluster
+    (6, 40, 64, 64, TILE64, "cluster U=16 ["),                                   # one 64-row tile's cluster
+    (6, 200, 64, 64, TILE64, "cluster U=16 ["),                                  # four of them
+    (6, 40, 64, 64, {}, "rows 8 "),                                              # clusters of 8 rows
+    (6, 500, 64, 200, {}, "rows 16 "),                                           # and of 16
 ])
 def test_backward_wait_timeout_is_reported_and_context_survives(T, B, I, H, env, want):
     """With a zero wait budget for the backward's kernels only, the forward completes and the
     backward reports SL_ERR_TIMEOUT instead of hanging: the persistent backward with its
     contraction split in thread-block clusters (partials in flight between the parts) or
-    through L2, the one whose release warp waits at a barrier with the epilogue, and the
-    cluster backward. The device stays usable: a new handle then reproduces a normal run
+    through L2, the one whose release warp waits at a barrier with the epilogue, the clusters
+    of 64-row tiles and those of 8 and 16 rows. The device stays usable: a new handle then reproduces a normal run
     bit for bit."""
     w = case(T, B, I, H, 10, bias_scale=0.3, h0_scale=0.5)
 
@@ -198,7 +213,8 @@ def test_backward_wait_timeout_is_reported_and_context_survives(T, B, I, H, env,
     hd = with_env({"STACKLSTM_WAIT_LIMIT_BWD_CYCLES": "0"},
                   lambda: bd.stacklstm_create(w.T, w.B, w.I, w.H, bd.SL_BF16, 0))
     try:
-        assert want in bd.stacklstm_plan(hd).split("; backward ")[1], bd.stacklstm_plan(hd)
+        bwd = phase_plans(bd.stacklstm_plan(hd))[1]
+        assert want in bwd and ("rows 0 " in bwd or "rows" in want), bwd
         ins, out = runner.upload(w), runner.alloc_outputs(w)
         bd.stacklstm_forward(hd, ins["x"], ins["ops"], ins["h0"], ins["c0"], ins["W"], ins["bias"],
                              p_final=out["p_final"])
@@ -322,14 +338,21 @@ def test_input_gradient_on_spare_sms_matches_oracle(T, B, I, H, seed):
                                          (8, 450, 16, 32, 25)])
 def test_cluster_kernels_match_oracle(T, B, I, H, seed):
     """Up to 8 row tiles of 64 instances: the forward and the backward as one thread-block
-    cluster per row tile, their defaults (a ragged last tile: B = 100, 200, 450), into
-    NaN-filled outputs, match the oracle, as do the persistent kernels they replace."""
+    cluster per row tile (a ragged last tile: B = 100, 200, 450), into NaN-filled outputs,
+    match the oracle, as do the clusters of 8 rows that the planner prefers and the persistent
+    kernels."""
     w = case(T, B, I, H, seed, bias_scale=0.3, h0_scale=0.5, c0_scale=0.5, dy_scale=0.5)
-    plan, got = run_nan_filled(w, {})
-    assert "forward cluster U=16" in plan and "backward cluster U=16" in plan, plan
-    assert "slots %d" % ((B + 63) // 64) in plan, plan
+    plan, got = run_nan_filled(w, TILE64)
+    for part in phase_plans(plan):
+        assert part.startswith("cluster U=16") and "rows 0" in part, plan
+        assert "slots %d " % ((B + 63) // 64) in part, plan
     ref = oracle_all(w)
     compare(got, ref, "bf16")
+    plan_r, rows = run_nan_filled(w, {})
+    for part in phase_plans(plan_r):
+        assert part.startswith("cluster U=32") and "rows 8" in part, plan_r
+        assert "slots %d " % ((B + 7) // 8) in part and "cluster %d " % ((H + 31) // 32) in part, plan_r
+    compare(rows, ref, "bf16")
     plan_p, per = run_nan_filled(w, {"STACKLSTM_BWD_CLUSTER": "0", "STACKLSTM_FWD_CLUSTER": "0"})
     assert "forward persistent" in plan_p and "backward persistent" in plan_p, plan_p
     compare(per, ref, "bf16")
@@ -337,5 +360,5 @@ def test_cluster_kernels_match_oracle(T, B, I, H, seed):
     for env, want in (({"STACKLSTM_BWD_CLUSTER": "0"}, ("forward cluster", "backward persistent")),
                       ({"STACKLSTM_FWD_CLUSTER": "0"}, ("forward persistent", "backward cluster"))):
         plan_m, mixed = run_nan_filled(w, env)
-        assert all(x in plan_m for x in want), plan_m
+        assert all(x in plan_m for x in want) and plan_m.count("rows 0") == 2, plan_m
         compare(mixed, ref, "bf16")

@@ -69,9 +69,12 @@ def check_against_homogenized(w, got, env=None):
 
 
 @pytest.mark.parametrize("T,B,I,H,seed,env", [
-    (17, 40, 8, 16, 31, {}),                                  # one row tile: thread-block cluster kernels
-    (24, 64, 200, 200, 32, {}),                               # parser widths, cluster kernels
-    (20, 200, 24, 40, 33, {}),                                # clusters, four row tiles
+    (17, 40, 8, 16, 31, {}),                                  # clusters of 8 rows
+    (24, 64, 200, 200, 32, {}),                               # parser widths, clusters of 8 rows
+    (20, 200, 24, 40, 33, {}),                                # 25 of them
+    (17, 40, 8, 16, 31, {"STACKLSTM_ROW_CLUSTER": "0"}),      # one 64-row tile's cluster
+    (24, 64, 200, 200, 32, {"STACKLSTM_ROW_CLUSTER": "0"}),   # the same at parser widths
+    (20, 200, 24, 40, 33, {"STACKLSTM_ROW_CLUSTER": "0"}),    # clusters of four 64-row tiles
     (20, 200, 24, 40, 33, dict(PERSISTENT)),                  # persistent kernels, ragged tiles
     (30, 300, 136, 72, 34, dict(PERSISTENT)),                 # three row tiles
     (11, 200, 264, 64, 35, dict(PERSISTENT)),                 # dx on the spare SMs of the backward launch

@@ -38,6 +38,14 @@ def lib(tmp_path_factory):
     return lib
 
 
+class ForwardArgs(ctypes.Structure):  # sl_forward_args
+    _fields_ = [("p%d" % i, ctypes.c_void_p) for i in range(12)]
+
+
+class BackwardArgs(ctypes.Structure):  # sl_backward_args
+    _fields_ = [("p%d" % i, ctypes.c_void_p) for i in range(7)]
+
+
 def tensors(n):
     """n addresses of the caller's."""
     return [0x100000 * (i + 1) for i in range(n)]
@@ -191,3 +199,30 @@ def test_the_clear_comes_before_the_steps_where_clusters_could_share_sms_without
     left = lib.fake_unjoined(USER)
     lib.stacklstm_destroy(h)
     assert left == (0 if early else 1)
+
+
+@pytest.mark.parametrize("members,env,fwd,bwd", [
+    # (B, I, H) of each: one launch of row clusters
+    ([(64, 200, 200), (64, 48, 200), (1, 8, 208)], {}, 1, 1),
+    # another contraction depth, more than 64 rows, clusters of other rows, an input too wide for them
+    ([(64, 200, 208), (64, 200, 216)], {}, 2, 2),
+    ([(64, 200, 200), (65, 200, 200)], {}, 2, 2),
+    ([(64, 48, 200), (64, 680, 200)], {}, 2, 2),
+    # wide inputs: the backward's 64-row clusters in one launch, persistent forwards
+    ([(64, 680, 200), (9, 800, 200)], {}, 2, 1)])
+def test_grouped_calls_share_a_launch_where_the_kernel_is_the_same(lib, monkeypatch, members, env, fwd, bwd):
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
+    n = len(members)
+    hs = [create(lib, 12, B, I, H, BF16) for B, I, H in members]
+    handles = (ctypes.c_void_p * n)(*(h.value for h in hs))
+    lib.fake_reset()
+    assert lib.stacklstm_forward_group(n, handles, (ForwardArgs * n)(*[ForwardArgs(*tensors(12))] * n)) == 0
+    steps = [l[0] for l in launches(lib) if "step_" in l[0]]
+    assert len(steps) == fwd, steps
+    lib.fake_reset()
+    assert lib.stacklstm_backward_group(n, handles, (BackwardArgs * n)(*[BackwardArgs(*tensors(7))] * n)) == 0
+    steps = [l[0] for l in launches(lib) if "step_" in l[0]]
+    assert len(steps) == bwd, steps
+    for h in hs:
+        lib.stacklstm_destroy(h)

@@ -192,9 +192,10 @@ sl_status stacklstm_steps_run(stacklstm_t s, int *steps);
  * and the action history of Sec. 4.1; Table 1 gives each transition's stack and buffer
  * ops); with the transitions known, their recurrences are independent of one another.
  * The result is that of calling stacklstm_forward (stacklstm_backward) on each handle,
- * each on its own stream. When every handle runs cluster kernels on one 64-row tile (B <= 64)
- * with the same cluster size (the same H), their step kernels run as ONE launch of each
- * handle's thread-block clusters, on the first handle's stream; each handle's stream
+ * each on its own stream. When every handle has at most 64 rows and the same cluster kernel
+ * runs its steps (clusters of 8 rows; in the backward also one of 64 rows; H alike up to 16
+ * units), their step kernels run as ONE launch of each handle's thread-block clusters, on
+ * the first handle's stream; each handle's stream
  * joins that stream before the launch and waits for it afterwards. Otherwise each handle
  * launches its own. The work before and after the steps stays on each handle's stream.
  * Timing: the one launch counts in the first handle's forward (backward) phase.

@@ -736,20 +736,14 @@ __global__ void __launch_bounds__(kClBwdThreads, 1) step_clb(ClArgs p)
     step_clb_body<U>(p, (int)(blockIdx.x / p.n_ct) * 64);
 }
 
-// Several handles' recurrences in one launch: cluster m (CTAs m n_ct .. m n_ct + n_ct - 1)
+// Several handles' backward recurrences in one launch: cluster m (CTAs m n_ct .. m n_ct + n_ct - 1)
 // runs member m's steps with its own arguments, workspace and step count. The members are
 // independent (each has its own inputs and op stream), so no barrier spans clusters; each
-// keeps its own per-step operand exchange.
+// keeps its own per-step operand exchange. (A forward of at most 64 rows is in row clusters
+// or, past their inputs, persistent: none of it is left to group here.)
 struct ClGroup {
-    CUtensorMap tm[kMaxGroup];  // forward: each member's x map
     ClArgs p[kMaxGroup];
 };
-template <int U>
-__global__ void __launch_bounds__(kClFwdThreads, 1) step_cl_group(const __grid_constant__ ClGroup g)
-{
-    const int m = (int)blockIdx.x / g.p[0].n_ct;
-    step_cl_body<U>(&g.tm[m], g.p[m], 0);
-}
 template <int U>
 __global__ void __launch_bounds__(kClBwdThreads, 1) step_clb_group(const __grid_constant__ ClGroup g)
 {
@@ -921,39 +915,33 @@ cudaError_t bf16_launch_bwd_cluster(stacklstm *s, const StepArgs &a)
     return cudaGetLastError();
 }
 
-// Several handles' forward (or backward) recurrences as one launch of n clusters: the
-// dynamic shared memory is the largest member's, each cluster carves its own layout.
-template <bool kFwd>
-cudaError_t launch_cluster_group(stacklstm *const *hs, const StepArgs *as, const CUtensorMap *const *tms, int n,
-                                 cudaStream_t st)
+// Several handles' backward recurrences as one launch of n clusters: each has the same footprint
+// (it depends on n_ct alone), and a 64-row tile of its own.
+cudaError_t bf16_launch_bwd_cluster_group(stacklstm *const *hs, const StepArgs *as, int n, cudaStream_t st)
 {
     ClGroup g{};
-    size_t smem = 0;
-    const int n_ct = (kFwd ? hs[0]->fc : hs[0]->bc).n_ct;
+    const PersistPlan &p0 = hs[0]->bc;
     for (int m = 0; m < n; ++m) {
         stacklstm *s = hs[m];
-        const PersistPlan &pl = kFwd ? s->fc : s->bc;
-        if (!pl.on || pl.n_ct != n_ct || pl.slot != 1) return cudaErrorInvalidValue;
+        if (!s->bc.on || s->bc.n_ct != p0.n_ct || s->bc.slot != 1) return cudaErrorInvalidValue;
         ClArgs &p = g.p[m];
         p.s = as[m];
-        p.s.gates_blk = kFwd ? s->bc.on : s->fc.on;
-        p.n_ct = n_ct;
-        p.gscr = (uint8_t *)(kFwd ? s->g_fcl : s->g_bcl);
-        if (kFwd) g.tm[m] = *tms[m];
-        smem = std::max<size_t>(smem, pl.smem);
+        p.s.gates_blk = s->fc.on;
+        p.n_ct = p0.n_ct;
+        p.gscr = (uint8_t *)s->g_bcl;
     }
-    const void *fn = kFwd ? (const void *)step_cl_group<kClU> : (const void *)step_clb_group<kClU>;
-    cudaError_t e = smem_at_least(fn, smem);
+    const void *fn = (const void *)step_clb_group<kClU>;
+    cudaError_t e = smem_at_least(fn, p0.smem);
     if (e) return e;
-    if (n_ct > 8 && (e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1))) return e;
+    if (p0.n_ct > 8 && (e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1))) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n * n_ct);
-    cfg.blockDim = dim3(kFwd ? kClFwdThreads : kClBwdThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.gridDim = dim3(n * p0.n_ct);
+    cfg.blockDim = dim3(kClBwdThreads);
+    cfg.dynamicSmemBytes = p0.smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = n_ct;
+    at[0].val.clusterDim.x = p0.n_ct;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
@@ -962,17 +950,6 @@ cudaError_t launch_cluster_group(stacklstm *const *hs, const StepArgs *as, const
     if ((e = cudaLaunchKernelExC(&cfg, fn, argv))) return e;
     hs[0]->launches += 1;
     return cudaGetLastError();
-}
-
-cudaError_t bf16_launch_fwd_cluster_group(stacklstm *const *hs, const StepArgs *as, const CUtensorMap *const *tms, int n,
-                                          cudaStream_t st)
-{
-    return launch_cluster_group<true>(hs, as, tms, n, st);
-}
-
-cudaError_t bf16_launch_bwd_cluster_group(stacklstm *const *hs, const StepArgs *as, int n, cudaStream_t st)
-{
-    return launch_cluster_group<false>(hs, as, nullptr, n, st);
 }
 
 }  // namespace sl

@@ -962,10 +962,10 @@ cudaError_t bf16_backward_steps(stacklstm *s, float *dx, bool *dx_done)
     return cudaGetLastError();
 }
 
-// the one-launch plan of a handle's steps: row-group clusters, or one 64-row cluster
+// the one-launch plan of a handle's steps: row-group clusters, or (backward) one 64-row cluster
 static const PersistPlan &group_plan(const stacklstm *s, bool fwd)
 {
-    return fwd ? (s->fr.on ? s->fr : s->fc) : (s->br.on ? s->br : s->bc);
+    return fwd ? s->fr : s->br.on ? s->br : s->bc;
 }
 
 // Handles of at most 64 rows whose kernel is the same: clusters of as many rows over as many 16-unit
@@ -986,16 +986,8 @@ bool bf16_can_group(stacklstm *const *hs, int n, bool fwd)
 cudaError_t bf16_forward_steps_group(stacklstm *const *hs, int n, const float *const *bias, cudaStream_t st)
 {
     StepArgs as[kMaxGroup];
-    const CUtensorMap *tms[kMaxGroup];
-    if (hs[0]->fr.on) {
-        for (int m = 0; m < n; ++m) as[m] = step_args(hs[m], bias[m], nullptr, hs[m]->kcx, hs[m]->kcf, 0);
-        return bf16_launch_rows(hs, as, nullptr, n, true, st);
-    }
-    for (int m = 0; m < n; ++m) {
-        as[m] = step_args(hs[m], bias[m], hs[m]->w_fwd, hs[m]->kcx, hs[m]->kcf, 0);
-        tms[m] = &map(hs[m], kMapX64);
-    }
-    return bf16_launch_fwd_cluster_group(hs, as, tms, n, st);
+    for (int m = 0; m < n; ++m) as[m] = step_args(hs[m], bias[m], nullptr, hs[m]->kcx, hs[m]->kcf, 0);
+    return bf16_launch_rows(hs, as, nullptr, n, true, st);
 }
 
 cudaError_t bf16_backward_steps_group(stacklstm *const *hs, int n, cudaStream_t st)

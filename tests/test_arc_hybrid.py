@@ -197,6 +197,48 @@ def test_grouped_calls_run_one_step_launch_and_match_oracle():
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("sizes,env", [([(12, 40, 680, 48), (9, 64, 800, 40), (10, 1, 712, 48)], {}),
+                                       ([(12, 40, 24, 48), (9, 64, 16, 40)], {"STACKLSTM_ROW_CLUSTER": "0"})])
+def test_grouped_backwards_of_64_row_clusters_share_a_launch(monkeypatch, sizes, env):
+    """Inputs too wide for the row clusters (or those switched off): the members' 64-row backward
+    clusters run as one launch, their forwards one by one, with the results of separate calls."""
+    import torch
+    from paper_1904_03409_gb300 import binding as bd
+    from paper_1904_03409_gb300 import runner
+    for k, v in dict(env, STACKLSTM_CUDA_CORE="0").items():
+        monkeypatch.setenv(k, v)
+    ws = [wl.make_workload("m%d" % i, T=T, B=B, I=I, H=H, dtype="bf16", seed=70 + i, ops_kind="random_walk",
+                           probs=(0.5, 0.3, 0.2), dy_scale=0.5) for i, (T, B, I, H) in enumerate(sizes)]
+    hds = [bd.stacklstm_create(w.T, w.B, w.I, w.H, bd.SL_BF16, 0) for w in ws]
+    try:
+        ins, outs = [runner.upload(w) for w in ws], [runner.alloc_outputs(w) for w in ws]
+        for o in outs:
+            for v in o.values():
+                if v.is_floating_point():
+                    v.fill_(float("nan"))
+        for hd in hds:
+            bd.stacklstm_set_timing(hd, True)
+        bd.stacklstm_forward_group(hds, [dict(
+            {k: i[k] for k in ("x", "ops", "h0", "c0", "W", "bias")},
+            **{k: o[k] for k in ("h_stack", "c_stack", "p_final", "p_traj", "src", "y")}) for i, o in zip(ins, outs)])
+        bd.stacklstm_backward_group(hds, [dict(
+            d_top_h=i["d_top_h"], dy=i["dy"], **{k: o[k] for k in ("dx", "dh0", "dc0", "dW", "dbias")})
+            for i, o in zip(ins, outs)])
+        torch.cuda.synchronize()
+        steps = [tuple(bd.stacklstm_get_timing(hd)[p][1] for p in ("forward", "backward")) for hd in hds]
+        assert steps == [(1, 1)] + [(1, 0)] * (len(ws) - 1), steps
+        for w, o in zip(ws, outs):
+            got = runner.to_numpy(o)
+            compare(got, oracle.run(w.x, w.ops, w.h0, w.c0, w.W, w.bias, d_top_h=w.d_top_h, dy=w.dy), "bf16")
+            alone = runner.run(w)
+            for name in ("dx", "dW", "dbias", "dh0", "dc0", "y", "h_stack", "p_traj"):
+                assert np.array_equal(got[name], alone[name], equal_nan=True), (w.name, name)
+    finally:
+        for hd in hds:
+            hd.destroy()
+
+
+@pytest.mark.gpu
 def test_grouped_calls_fall_back_when_the_members_differ():
     """Handles that cannot share one launch (different hidden widths, several row tiles)
     still give the results of separate calls."""

@@ -209,7 +209,9 @@ def test_the_clear_comes_before_the_steps_where_clusters_could_share_sms_without
     ([(64, 200, 200), (65, 200, 200)], {}, 2, 2),
     ([(64, 48, 200), (64, 680, 200)], {}, 2, 2),
     # wide inputs: the backward's 64-row clusters in one launch, persistent forwards
-    ([(64, 680, 200), (9, 800, 200)], {}, 2, 1)])
+    ([(64, 680, 200), (9, 800, 200)], {}, 2, 1),
+    # without row clusters the 64-row forwards, too, run one by one
+    ([(64, 200, 200), (64, 48, 200)], {"STACKLSTM_ROW_CLUSTER": "0"}, 2, 1)])
 def test_grouped_calls_share_a_launch_where_the_kernel_is_the_same(lib, monkeypatch, members, env, fwd, bwd):
     for k, v in env.items():
         monkeypatch.setenv(k, v)

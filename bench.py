@@ -8,11 +8,12 @@ method computes padded steps too).
 
   python bench.py [--gpus 1] [--steps K] [--warmup W] [--workload NAME] [--impl ours|reference]
 
-Prints ONE JSON line. The headline is the parser-scale workload (B=64, I=H=200); unless
---workload names one workload or --no-extra is given, the line also carries a full record
-(throughput, roofline, clocks, end-to-end rate, CPU baseline, step latency) for every
-other workload: tiny, each batch size of the sweep, large, stress, and the arc-hybrid
-parser batch. The library runs on one GPU: its one-row-tile kernels deliver operands
+Prints ONE JSON line of at most 2.8 KB. The headline is the parser-scale workload (B=64,
+I=H=200); unless --workload names one workload or --no-extra is given, the line also gives
+the throughput, time and roofline of every other workload: tiny, each batch size of the
+sweep, large, stress, and the arc-hybrid parser batch. The full record of each (plan,
+phases, clocks, end-to-end rate, CPU baseline, step latency, push-only mode) goes to
+standard error as one line, or to the file that --detail names. The library runs on one GPU: its one-row-tile kernels deliver operands
 between the CTAs of a thread-block cluster with multicast copies, which are for a
 process on one GPU; --gpus N > 1 (or a torchrun world larger than one) is refused
 before any library call.
@@ -275,7 +276,40 @@ def run_ours(args):
         line["workloads"]["arc_hybrid64"] = measure_group("arc_hybrid64", max(20, args.steps), args.warmup)
         torch.cuda.empty_cache()
         line["workloads"]["parser_step64"] = measure_parser("arc_hybrid64", max(20, args.steps), args.warmup)
-    print(json.dumps(line), flush=True)
+    detail = json.dumps(line)
+    if args.detail:
+        with open(args.detail, "w") as f:
+            f.write(detail + "\n")
+    else:
+        print("bench detail: " + detail, file=sys.stderr, flush=True)
+    print(json.dumps(summary_line(line)), flush=True)
+
+
+def summary_line(line):
+    """The printed line of a full record: whoever reads it may keep only the last 3000
+    characters or so of the output, so numbers are rounded, the headline's record keeps what
+    says how it was measured, and the other workloads are [value, ms, roofline fraction]."""
+    def rounded(v):
+        if isinstance(v, float):
+            return float("%.6g" % v)
+        if isinstance(v, dict):
+            return {k: rounded(x) for k, x in v.items()}
+        if isinstance(v, list):
+            return [rounded(x) for x in v]
+        return v
+
+    left_out = ("workloads", "push_only", "plan", "phases_ms_per_step", "step_latency_us", "steps_run")
+    out = {k: v for k, v in line.items() if k not in left_out}
+    for k in ("roofline", "step_roofline"):
+        if k in out:
+            out[k] = {q: out[k][q] for q in ("bound", "achieved", "peak", "unit", "frac", "peak_source", "kernel",
+                                            "launch_us", "traffic") if q in out[k]}
+    if "workloads" in line:
+        out["workloads"] = {k: [rec["value"], rec["ms_per_step"], rec.get("step_roofline", {}).get("frac")]
+                            for k, rec in line["workloads"].items()}
+    if "push_only" in line:
+        out["push_only"] = [line["push_only"]["value"], line["push_only"]["ms_per_step"]]
+    return rounded(out)
 
 
 def measure_record(w, steps, warmup, cpu_seconds, with_cpu, min_seconds):
@@ -636,6 +670,7 @@ def main():
     ap.add_argument("--ref-step-seconds", type=float, default=3.0, help="oracle work per reference step")
     ap.add_argument("--no-extra", action="store_true", help="the named workload only")
     ap.add_argument("--no-cpu-baseline", action="store_true")
+    ap.add_argument("--detail", help="write the full record here instead of to standard error")
     ap.add_argument("--T", type=int, default=None,
                     help="fewer steps for tiny/large/stress (a smaller case of the same shape, for profiling)")
     args = ap.parse_args()

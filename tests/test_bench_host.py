@@ -73,3 +73,34 @@ def test_roofline_picks_the_tighter_bound():
     # fp32 path: CUDA-core FFMA peak from the SM count and the clock
     r = bench.roofline_of(1e12, 1e9, 1.0, peaks, "measured", dtype="fp32", sms=100)
     assert r["bound"] == "alu" and abs(r["peak"] - 100 * 128 * 2 * 2000e6 / 1e12) < 1e-9
+
+
+def test_printed_line_stays_short():
+    """The one line that is printed keeps every key of the headline in 2800 characters, whatever
+    the full records hold."""
+    roof = {"bound": "hbm", "achieved": 123.456789012345, "peak": 6792.7, "unit": "GB/s", "frac": 0.0456789012345,
+            "peak_source": "measured HBM copy", "kernel": "step_rows<8 rows>", "phase": "forward", "launch_us": 181.23456789,
+            "launches_per_pass": 1, "units_per_launch": 11840.0, "unit_of_work": "instance-step",
+            "algorithmic_flops_per_unit": 640000, "algorithmic_bytes_per_unit": 2800, "traffic": None}
+    clocks = {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": [], "samples": 3, "power_w_max": 168.59}
+    rec = {"value": 28912345.678901234, "ms_per_step": 0.40951234567, "steps": 20, "roofline": roof, "step_roofline": roof,
+           "phases_ms_per_step": {"phase%d" % i: 0.1234 for i in range(8)}, "step_latency_us": {"forward": 0.96, "backward": 1.14},
+           "steps_run": 185, "plan": "p" * 900, "gpu_launches": 240, "clocks": clocks,
+           "e2e": {"value": 23800000.123, "unit": bench.UNIT, "h2d_bytes_per_step": 5519040, "d2h_bytes_per_step": 10857856,
+                   "steps": 20},
+           "config": {"workload": "w" * 150, "B": 64, "T": 185, "I": 200, "H": 200, "real_step_share": 0.5659,
+                      "l2": "flushed between timed steps (256 MiB write outside the timed events)",
+                      "parallelism": "single GPU"},
+           "cpu_baseline": {"value": 31800.123456, "unit": bench.UNIT, "cores": 16, "kind": "oracle", "sample": "s" * 100}}
+    line = dict(rec, metric=bench.METRIC, unit=bench.UNIT, n_gpus=1, warmup=5, higher_is_better=True, scaling="weak",
+                vs_baseline=None, dtype="bf16", data=bench.DATA, push_only=dict(rec),
+                workloads={k: dict(rec) for k in bench.SIDE_WORKLOADS + ("arc_hybrid64", "parser_step64")})
+    del line["workloads"]["parser_step64"]["step_roofline"]
+    assert len(json.dumps(line)) > 30000
+    out = bench.summary_line(line)
+    assert len(json.dumps(out)) < 2800, len(json.dumps(out))
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline"):
+        assert k in out, k
+    assert abs(out["value"] / line["value"] - 1) < 1e-5 and out["e2e"]["h2d_bytes_per_step"] == 5519040
+    assert set(out["workloads"]) == set(line["workloads"])

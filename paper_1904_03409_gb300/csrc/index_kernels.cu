@@ -685,12 +685,19 @@ cudaError_t launch_seed_grads(stacklstm *s, const float *d_top_h, const float *d
 {
     if (!d_top_h && !dy) return cudaSuccess;
     const int32_t *top = s->push_only ? s->vy : s->top;
-    // units a lane: as many as keep several warps' rows on an SM (and divide H)
+    // Units a lane: four while four warps' rows fit on an SM, two while three do, if that divides H
+    // and the blocks then cover no more units past H. (us with 1 / 2 / 4: 512 x 256, 60 steps 26 / 23 /
+    // 22, 120 steps 43 / 39 / 48; 256 x 1024, 256 steps 184 / 177 / 281; 64 x 256, 300 steps 24 / 25 / 28;
+    // 1024 x 200, 195 steps, where two and four cover 256 units 151 / 159 / 230; 2000 x 32, 40 steps 13 /
+    // 19 / 25)
     const size_t acc_bytes = (size_t)(s->T + 1 + kSeedRing) * 32 * sizeof(float);
+    auto fits = [&](int N, size_t cap) {
+        return s->H % N == 0 && N * acc_bytes <= cap && ceil_div(s->H, 32 * N) * N <= ceil_div(s->H, 32);
+    };
     // (200 KB of rows and the ring, 4 KB: sequences of up to 1599 steps)
     if (dy && acc_bytes <= 204 * 1024) {
-        if (s->H % 4 == 0 && 4 * acc_bytes <= 56 * 1024) return seed_dy<4>(s, 4 * acc_bytes, top, d_top_h, dy);
-        if (s->H % 2 == 0 && 2 * acc_bytes <= 72 * 1024) return seed_dy<2>(s, 2 * acc_bytes, top, d_top_h, dy);
+        if (fits(4, 56 * 1024)) return seed_dy<4>(s, 4 * acc_bytes, top, d_top_h, dy);
+        if (fits(2, 75 * 1024)) return seed_dy<2>(s, 2 * acc_bytes, top, d_top_h, dy);
         return seed_dy<1>(s, acc_bytes, top, d_top_h, dy);
     }
     const size_t n = (size_t)s->B * s->H;

@@ -228,3 +228,18 @@ def test_grouped_calls_share_a_launch_where_the_kernel_is_the_same(lib, monkeypa
     assert len(steps) == bwd, steps
     for h in hs:
         lib.stacklstm_destroy(h)
+
+
+@pytest.mark.parametrize("T,H,dtype,units", [
+    (60, 256, BF16, 4), (80, 256, BF16, 2), (256, 1024, BF16, 2), (270, 1024, BF16, 1), (60, 32, BF16, 1), (60, 64, BF16, 2),
+    (60, 40, BF16, 2), (60, 104, BF16, 4), (60, 200, BF16, 1), (60, 8, BF16, 1), (60, 100, FP32, 4), (60, 66, FP32, 1),
+    (60, 62, FP32, 2), (60, 63, FP32, 1)])
+def test_per_step_seeding_leaves_no_lanes_idle_for_more_units_a_lane(lib, T, H, dtype, units):
+    h = create(lib, T, 40, 8, H, dtype)
+    assert forward(lib, h) == 0
+    lib.fake_reset()
+    assert backward(lib, h) == 0
+    seeds = [l for l in launches(lib) if "seed_grads_dy" in l[0]]
+    lib.stacklstm_destroy(h)
+    assert len(seeds) == 1 and "ILi%dE" % units in seeds[0][0], seeds
+    assert seeds[0][1] == (40, -(-H // (32 * units)), 1), seeds

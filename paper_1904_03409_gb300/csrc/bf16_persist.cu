@@ -1338,10 +1338,12 @@ const Variant *bwd_variants(int *n)
 }
 
 // Largest residency (CTAs per SM) that leaves every CTA its two accumulators in tensor
-// memory (512 columns per SM); shared memory is padded to enforce it.
+// memory (512 columns per SM); shared memory is padded to enforce it (0: the footprint does
+// not fit as it is).
 uint32_t pad_for_tmem(const void *fn, int threads, uint32_t smem, uint32_t kcols2)
 {
     const int max_res = std::max(1, (int)(512 / kcols2));
+    if (smem > kSmemCap) return 0;
     for (; smem <= kSmemCap; smem += 4096) {
         int r = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, fn, threads, smem) != cudaSuccess) {

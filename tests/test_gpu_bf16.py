@@ -267,6 +267,15 @@ def test_split_contraction_backward_matches_oracle(T, B, I, H, seed, cl):
         assert np.array_equal(got[k], again[k]), k
 
 
+@pytest.mark.parametrize("T,B,I,H,seed", [(4, 155, 472, 528, 30), (5, 40, 64, 520, 31), (3, 300, 264, 640, 32), (4, 8, 16, 768, 33)])
+def test_hidden_widths_past_512_match_oracle(T, B, I, H, seed):
+    """Widths whose resident weight slice leaves no room for the exchange tile of a split
+    contraction's cluster beside it."""
+    w = case(T, B, I, H, seed, bias_scale=0.3, h0_scale=0.5, c0_scale=0.5, dy_scale=0.5)
+    _, got = run_nan_filled(w, {})
+    compare(got, oracle_all(w), "bf16")
+
+
 @pytest.mark.parametrize("T,B,I,H,seed", [(20, 200, 24, 40, 27), (9, 300, 136, 72, 28), (12, 130, 264, 64, 29)])
 def test_weight_gradient_tile_shapes_match_oracle(T, B, I, H, seed):
     """The weight gradient with 128 x 256 tiles (two CTAs an SM) and with 256 x 256 tiles

@@ -2,8 +2,8 @@
 CUDA runtime (fake_cudart.cpp), which runs no kernel but follows what each stream is ordered after
 and can make any call that queues work fail."""
 import ctypes
-import glob
 import os
+import re
 import subprocess
 
 import pytest
@@ -243,3 +243,29 @@ def test_per_step_seeding_leaves_no_lanes_idle_for_more_units_a_lane(lib, T, H, 
     lib.stacklstm_destroy(h)
     assert len(seeds) == 1 and "ILi%dE" % units in seeds[0][0], seeds
     assert seeds[0][1] == (40, -(-H // (32 * units)), 1), seeds
+
+
+def persistent_bytes(part, fwd, chunks):
+    """What a persistent step kernel lays out in shared memory under its plan: alignment, a resident
+    weight tile, the ring, the staging tile, a cluster's exchange tile, the barriers."""
+    f = {k: int(v) for k, v in re.findall(r"(U|G|ring|w_res|smem|cluster|parts)[ =](\d+)", part.split(" dx CTAs")[0])}
+    nb, ks = (4 * f["U"], 1) if fwd else (f["U"], f["parts"])
+    weights = -(-chunks // ks) * nb * 128
+    stage = f["G"] * (16384 + (0 if f["w_res"] else nb * 128))
+    staging = 128 * f["U"] * 14 if fwd else 128 * 128 if f["U"] == 32 else 0
+    exchange = 128 * f["U"] * 4 if f["cluster"] > 1 else 0
+    return 1024 + f["w_res"] * weights + f["ring"] * stage + staging + exchange + 39 * 8 + 32, f["smem"]
+
+
+@pytest.mark.parametrize("B", [8, 155, 300, 1000])
+def test_persistent_plans_have_room_for_all_they_lay_out(lib, B):
+    for H in [*range(264, 1040, 8), 1536, 2048]:
+        h = create(lib, 5, B, 64, H, BF16)
+        plan = lib.stacklstm_plan(h).decode()
+        lib.stacklstm_destroy(h)
+        fwd, bwd = plan.split("; step rings")[0].split("; backward ")
+        chunks = re.search(r"chunks fwd (\d+) .*? bwd (\d+);", plan)
+        for part, is_fwd, k in ((fwd.split("; forward ")[1], True, 1), (bwd, False, 2)):
+            if part.startswith("persistent"):
+                need, has = persistent_bytes(part, is_fwd, int(chunks.group(k)))
+                assert need <= has <= 226 * 1024, (H, part)

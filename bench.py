@@ -138,7 +138,8 @@ def phase_kernel(plan, phase, dtype):
             return {"forward": ("fwd_seq_f32", "fp32_path.cu", 1), "backward": ("bwd_seq_f32", "fp32_path.cu", 1),
                     "dx": ("dx_f32", "fp32_path.cu", 1), "dw": ("dw_f32", "fp32_path.cu", 1)}[phase]
         if "clusters" in plan:
-            return {"forward": ("fwd_rows_f32", "fp32_rows.cu", 1), "backward": ("bwd_rows_f32", "fp32_rows.cu", 1),
+            fwd = ("fwd_step_f32", "fp32_path.cu", "T") if "forward one" in plan else ("fwd_rows_f32", "fp32_rows.cu", 1)
+            return {"forward": fwd, "backward": ("bwd_rows_f32", "fp32_rows.cu", 1),
                     "dx": ("gemm_f32", "fp32_rows.cu", 1), "dw": ("gemm_f32", "fp32_rows.cu", 1)}[phase]
         return {"forward": ("fwd_step_f32", "fp32_path.cu", "T"),
                 "backward": ("bwd_pointwise_f32+bwd_contract_f32", "fp32_path.cu", "2T"),

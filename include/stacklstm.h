@@ -32,9 +32,11 @@
  * Element types by dtype:
  *   SL_FP32: x, h0, W, h_stack, y are float; every computation in fp32 on CUDA cores
  *            (no tensor cores, no TF32).
- *   SL_BF16: x, h0, W, h_stack, y are bf16 (uint16 bit patterns); the gate contractions
- *            run on tcgen05 tensor cores with fp32 accumulation; cell states, gradients
- *            and all accumulations are fp32. Requires I % 8 == 0 and H % 8 == 0.
+ *   SL_BF16: x, h0, W, h_stack, y are bf16 (uint16 bit patterns); the contractions run
+ *            on the tensor cores with fp32 accumulation (tcgen05; the steps of H <= 256 and
+ *            few rows as mma.sync with the weights in registers, and those of one row of a
+ *            wide input on CUDA cores); cell states, gradients and all accumulations are
+ *            fp32. Requires I % 8 == 0 and H % 8 == 0.
  *   c0, c_stack, bias and every gradient are float in both modes.
  */
 /*

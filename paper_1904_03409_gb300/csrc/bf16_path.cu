@@ -643,14 +643,14 @@ std::string bf16_describe(const stacklstm *s)
     const PersistPlan &f = s->cc.on ? s->cc : s->fr.on ? s->fr : s->fc.on ? s->fc : s->pf;
     const PersistPlan &b = s->cc.on ? s->cc : s->br.on ? s->br : s->bc.on ? s->bc : s->pb;
     snprintf(buf, sizeof buf,
-             "bf16 tcgen05; row tiles %d; chunks fwd %d (x %d) bwd %d; "
+             "bf16; steps on %s; row tiles %d; chunks fwd %d (x %d) bwd %d; "
              "forward %s U=%d [EP %d G %d ring %d slots %d cluster %d col tiles %d w_res %d smem %u threads %d "
              "per SM %d rows %d]; "
              "backward %s U=%d [EP %d G %d ring %d slots %d cluster %d col tiles %d w_res %d smem %u threads %d "
              "per SM %d rows %d "
              "contraction parts %d dx CTAs %d ring %d]; "
              "step rings fwd %d bwd %d; dx N=%d x%d ring %d; dW %dx%d tiles of %dx%d x%d splits ring %d",
-             rt, s->kcf, s->kcx, s->kcb, s->cc.on ? "cuda-core" : s->fr.on || s->fc.on ? "cluster" : f.on ? "persistent" : "per-step", s->fr.on ? f.U : s->uf, f.EP, f.G, f.S, f.slot, f.cl, f.n_ct,
+             s->cc.on ? "CUDA cores" : s->fr.on ? "mma.sync" : "tcgen05", rt, s->kcf, s->kcx, s->kcb, s->cc.on ? "cuda-core" : s->fr.on || s->fc.on ? "cluster" : f.on ? "persistent" : "per-step", s->fr.on ? f.U : s->uf, f.EP, f.G, f.S, f.slot, f.cl, f.n_ct,
              f.w_res, f.smem, f.threads, f.per_sm, f.rows, s->cc.on ? "cuda-core" : s->br.on || s->bc.on ? "cluster" : b.on ? "persistent" : "per-step", s->br.on || s->bc.on ? b.U : s->ub, b.EP, b.G, b.S, b.slot, b.cl, b.n_ct,
              b.w_res, b.smem, b.threads, b.per_sm, b.rows, b.KS, b.n_dx, b.dx_S, s->sf, s->sb, s->nx, s->nxt, s->sx, s->dw_mt, s->dw_nt, s->dw_mtile, s->dw_ntile, s->dw_split, s->sw);
     return buf;

@@ -11,8 +11,8 @@
 // cell's registers as soon as the last MMA is done. The 64-row tcgen05 clusters
 // (bf16_cluster.cu) spend 1.54 us a step forward and 2.07 us backward on commits, barriers,
 // tensor-memory loads and on bringing 64 rows to every CTA (I = H = 200, B = 64); here it is
-// 0.96 and 1.03 us (clock stamps: about 400 cycles of ldmatrix and MMAs, 300 of cell,
-// 700 until every CTA's piece has landed). A 64 x 200 pass of 185
+// 0.96 and 1.03 us, in parts alike of ldmatrix and MMAs, the cell, and the wait until every
+// CTA's piece has landed. A 64 x 200 pass of 185
 // steps with per-step gradients: 0.777 -> 0.437 ms (with y stored here and a free GPU to start on).
 //
 // Forward. Warp w of CTA ct owns units 32 ct + 8 w .. + 7: M tile 0 is their gates i and f,
@@ -753,13 +753,16 @@ void rc_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, int clusters, i
     cfg->numAttrs = 1;
 }
 
-// One direction with NT 8-row N tiles a cluster: every cluster co-resident (two CTAs an SM),
-// or the plan is off. At H = 200 that is 38 clusters: NT = 1, 304 rows, 0.96 / 1.03 us a step up
-// to 14 clusters (one CTA an SM) and 1.34 / 1.50 beyond, against 1.6 / 2.3 of the 64-row
-// clusters; NT = 2, 608 rows at 2.63 / 2.51, against 4.02 / 6.05 of the persistent kernels (the
-// 64-row clusters reach 448 rows). A second round of clusters pays for training but not for a
-// forward alone: 768 rows 4.85 / 4.68 against 4.15 / 6.12, 1024 rows 5.09 / 4.96 against
-// 4.55 / 6.14.
+// One direction with NT 8-row N tiles a cluster: every cluster co-resident (two CTAs an SM, one
+// where the input is wide), or the plan is off. At H = 200 that is 38 clusters: NT = 1, 304 rows,
+// 0.96 / 1.03 us a step up to 14 clusters (one CTA an SM) and 1.34 / 1.50 beyond, against 1.6 / 2.3
+// of the 64-row clusters; NT = 2, 608 rows at 2.63 / 2.51, against 4.02 / 6.05 of the persistent
+// kernels (the 64-row clusters reach 448 rows). A second round of clusters pays for training but
+// not for a forward alone: 768 rows 4.85 / 4.68 against 4.15 / 6.12, 1024 rows 5.09 / 4.96 against
+// 4.55 / 6.14. At the reach of other widths (I = H, passes of 60 steps, us, before and here): H = 32,
+// 64 rows 237 / 116, 2400 (NT = 1) 505 / 186, 3500 (NT = 2) 528 / 266; H = 64, 1000 rows 522 / 189, 1400
+// 531 / 252; H = 104, 448 rows 285 / 169, 900 627 / 275; H = 128, 512 rows 282 / 182, 800 585 / 281; H = 136,
+// 448 rows 297 / 211, 560 646 / 342; H = 256, 288 rows 322 / 257. I = 640, H = 256: 64 rows 418 / 207.
 bool rc_plan(stacklstm *s, bool fwd, int NT, PersistPlan *pl)
 {
     pl->on = 0;

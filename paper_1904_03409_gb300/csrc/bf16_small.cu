@@ -35,14 +35,15 @@ constexpr int kCcWarps = kCcThreads / 32;
 constexpr int kCcRedStride = 80;  // floats per reduction row: rows b, b + 1 of a warp hit distinct banks
 constexpr int kCcMaxB = 32;       // rows the kernels hold (register accumulators per row)
 // Largest batch the planner gives these kernels by default, where the row clusters
-// (bf16_rows.cu) do not hold it: one row is faster there at every length and width (I = H = 200,
-// one pass of 1 / 8 / 40 / 60 steps: 44 / 55 / 106 / 138 us there, 54 / 76 / 172 / 230 here; H = 8, 36 to
-// 102 us against 49 to 179), so what is left here are inputs too wide for their shared memory
-// (H = 200: from I of about 650; one row of 60 steps, 800 + 200: 288 us here, 389 with the
-// persistent forward and the 64-row backward cluster). Measured against the 64-row clusters at I = H = 200 (one forward + backward pass of the parser
-// sweep workload): B = 1, 0.597 ms here against 0.695 ms (backward step 1.67 against 2.26 us, the
-// forward step equal at 1.57 us); B = 8, 1.80 ms against 0.77 ms; B = 32, 6.19 against
-// 0.83 ms. Per row, the FFMA contraction adds about 0.4 us a step.
+// (bf16_rows.cu) do not hold it: one row is faster there at every length and width (I = H =
+// 200, one pass of 1 / 8 / 40 / 60 steps: 44 / 55 / 106 / 138 us there, 54 / 76 / 172 / 230 here;
+// H = 8, 36 to 102 us against 49 to 179), so what is left here are inputs too wide for their
+// shared memory (H = 200: from I of about 650; one row of 60 steps, 800 + 200: 288 us here, 389
+// with the persistent forward and the 64-row backward cluster). Measured against the 64-row
+// clusters at I = H = 200 (one forward + backward pass of the parser sweep workload): B = 1,
+// 0.597 ms here against 0.695 ms (backward step 1.67 against 2.26 us, the forward step equal at
+// 1.57 us); B = 8, 1.80 ms against 0.77 ms; B = 32, 6.19 against 0.83 ms. Per row, the FFMA
+// contraction adds about 0.4 us a step.
 constexpr int kCcCrossoverB = 1;
 
 __device__ __forceinline__ uint32_t cc_rank()

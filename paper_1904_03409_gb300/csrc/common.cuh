@@ -201,8 +201,8 @@ cudaError_t bf16_forward_steps(stacklstm *s, const float *bias);
 // (the caller seeds them itself when the loss also has per-step terms)
 cudaError_t bf16_backward_setup(stacklstm *s, const float *d_top_h);
 cudaError_t bf16_backward_steps(stacklstm *s, float *dx, bool *dx_done);
-// Grouped calls: true when the n handles' step kernels can run as one launch (every one
-// on the one-row-tile cluster kernels of the same cluster size); that launch, on `st`.
+// Grouped calls: true when the n handles' step kernels can run as one launch (at most 64
+// rows each, the same cluster kernel); that launch, on `st`.
 bool bf16_can_group(stacklstm *const *hs, int n, bool fwd);
 cudaError_t bf16_forward_steps_group(stacklstm *const *hs, int n, const float *const *bias, cudaStream_t st);
 cudaError_t bf16_backward_steps_group(stacklstm *const *hs, int n, cudaStream_t st);

@@ -67,9 +67,9 @@ __global__ void fwd_step_f32(int t, int B, int I, int H, const float *__restrict
 }
 
 // The forward setup in one launch: history row 0 = (h0, c0), the initial state (stack
-// slot 0), and W^T (out[c][r] = in[r][c], R x C, out's rows ldo
-// apart) for the backward contractions, so that the
-// backward needs nothing the caller owns.
+// slot 0), and W^T (out[c][r] = in[r][c], R x C, out's rows ldo apart) for the backward
+// contractions, so that W may change after the forward. (x may not: the row clusters'
+// weight gradient reads it again.)
 __global__ void setup_f32(size_t n0, const float *__restrict__ h0, const float *__restrict__ c0,
                           float *__restrict__ hist_h, float *__restrict__ hist_c, int R, int C,
                           const float *__restrict__ in, float *__restrict__ out, size_t ldo)
@@ -392,7 +392,8 @@ std::string fp32_describe(stacklstm *s)
     }
     if (s->fp32_one_cta) return "fp32 CUDA cores; every step of each direction in one CTA";
     if (!(per_step && atoi(per_step) != 0) && fp32_plan_rows(s))
-        return "fp32 CUDA cores; clusters of " + std::to_string(s->fr32.cl) + " CTAs, rows " + std::to_string(s->fr32.rows);
+        return "fp32 CUDA cores; clusters of " + std::to_string(s->fr32.cl) + " CTAs, rows " + std::to_string(s->fr32.rows) +
+               (s->fr32_steps ? "; forward one launch per step" : "");
     return "fp32 CUDA cores; one launch per step";
 }
 
@@ -410,7 +411,6 @@ cudaError_t fp32_forward_steps(stacklstm *s, const float *x, const float *W, con
     const int T = s->T, B = s->B, I = s->I, H = s->H, K = I + H;
     if (s->fr32.on && !s->fr32_steps) return fp32_rows_forward(s, x, W, bias);
     if (s->fp32_one_cta) {
-        (void)K;
         const int P = fwd_seq_threads_per_unit(B, H);
         fwd_seq_f32<<<1, (unsigned)ceil_div(B * H * P, 32) * 32, fwd_seq_smem(T, B, I, H), s->stream>>>(
             T, B, I, H, P, x, W, bias, s->top, (float *)s->hist_h, s->hist_c, (float *)s->gates, (float *)s->a_rm);

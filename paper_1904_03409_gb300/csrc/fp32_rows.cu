@@ -670,7 +670,7 @@ __global__ void slab_sum_f32(size_t n, size_t n2, int nz, const float *__restric
 }
 
 // ---------------------------------------------------------------------------- host
-// rows a cluster (1, 2, 4) x contraction pieces of 32 (forward) / units a CTA (backward)
+// rows a cluster (1, 2, 4, 5, 6, 8) x contraction pieces of 32 (forward) / units a CTA (backward)
 template <int KC>
 const void *fwd_fn(int R)
 {

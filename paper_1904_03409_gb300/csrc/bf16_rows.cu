@@ -11,7 +11,7 @@
 // cell's registers as soon as the last MMA is done. The 64-row tcgen05 clusters
 // (bf16_cluster.cu) spend 1.54 us a step forward and 2.07 us backward on commits, barriers,
 // tensor-memory loads and on bringing 64 rows to every CTA (I = H = 200, B = 64); here it is
-// 0.96 and 1.03 us, in parts alike of ldmatrix and MMAs, the cell, and the wait until every
+// 0.96 and 1.03 us: a chain of ldmatrix and MMAs, the cell, and the wait until every
 // CTA's piece has landed. A 64 x 200 pass of 185
 // steps with per-step gradients: 0.777 -> 0.437 ms (with y stored here and a free GPU to start on).
 //
